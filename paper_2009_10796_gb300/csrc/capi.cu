@@ -1226,7 +1226,7 @@ ddgi_status cascade_enqueue(ddgi_cascade_s* c, const DevScene& sc, const Lights&
     DDGI_CK(launch_build_list_multi(vs, (int)c->total, 1, c->lists + c->total, c->counts + 1, st));
     DDGI_CK(launch_trace_wavefront_multi(sc, vs, L, c->dirs, c->R, c->perm, c->lists + c->total, c->counts + 1,
                                          c->records, c->shadow_list, c->hit_list, c->shadow_count, sms * c->trace_mult,
-                                         st, query_fast_view(c->h_params[slot]->views[0])));
+                                         st, query_form(c->h_params[slot]->views[0])));
     if (tensor)
         DDGI_CK(launch_blend_tc_set(vs, true, bp, precision, d0.irr_n, d0.dist_n, c->pack_w, c->inv_irr_r,
                                     c->inv_dist_r, c->records, c->lists + c->total, c->counts + 1, c->status, sms, st));
@@ -1427,7 +1427,7 @@ ddgi_status ddgi_cascade_query(ddgi_cascade c, const float* pos_dev, const float
     vs.table = c->d_params->views;
     vs.n = c->n;
     DDGI_CK(launch_query_cascade(vs, pos_dev, nrm_dev, n, make_float3(camera_pos[0], camera_pos[1], camera_pos[2]),
-                                 out_dev, (cudaStream_t)stream));
+                                 out_dev, query_form(cascade_view(c, 0, camera_pos)), (cudaStream_t)stream));
     return DDGI_OK;
 }
 

@@ -6,6 +6,7 @@
 
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "ddgi.h"
@@ -94,12 +95,42 @@ inline void set_view_divisors(VolView& w) {
     w.div_xy = make_fast_div((uint32_t)w.counts.x * (uint32_t)w.counts.y);
 }
 
-// Views the specialised (FAST) probe query serves: FP32 atlases, gamma 5 and
-// no probe offsets; its kernels skip the per-probe format, gamma and offset
-// tests and otherwise compute the same operations in the same order.
-inline bool query_fast_view(const VolView& w) {
-    return w.irr_format == DDGI_IRR_FP32 && w.dist_format == DDGI_DIST_FP32 && w.half_gamma == 2.5f &&
-           w.offsets == nullptr;
+// Forms of the probe query with a specialised device function (the storage
+// format, gamma and offsets fixed at compile time; otherwise the general
+// form's operations in the same order).  The line between them is which
+// combinations are used: FP32 and FP16 atlases and RGB9E5 irradiance with
+// the default gamma, probe offsets (the position optimizer) and gamma 1 (the
+// differentiable path) with FP32 atlases; anything else is general.
+enum QueryFormId {
+    kQueryFp32 = 0,     // FP32 atlases, gamma 5, no offsets
+    kQueryHalf = 1,     // FP16 atlases, gamma 5, no offsets
+    kQueryE5 = 2,       // RGB9E5 irradiance and FP32 distance, gamma 5, no offsets
+    kQueryMoved = 3,    // FP32 atlases, gamma 5, probe offsets
+    kQueryGamma1 = 4,   // FP32 atlases, gamma 1, no offsets
+    kQueryGeneral = 5
+};
+
+inline int query_form(const VolView& w) {
+    const bool f32 = w.irr_format == DDGI_IRR_FP32 && w.dist_format == DDGI_DIST_FP32;
+    const bool g5 = w.half_gamma == 2.5f, fixed = w.offsets == nullptr;
+    if (f32 && g5) return fixed ? kQueryFp32 : kQueryMoved;
+    if (f32 && fixed && w.half_gamma == 0.5f) return kQueryGamma1;
+    if (g5 && fixed && w.irr_format == DDGI_IRR_FP16 && w.dist_format == DDGI_DIST_FP16) return kQueryHalf;
+    if (g5 && fixed && w.irr_format == DDGI_IRR_RGB9E5 && w.dist_format == DDGI_DIST_FP32) return kQueryE5;
+    return kQueryGeneral;
+}
+
+// f(std::integral_constant<int, form>) for a view's form.
+template <typename F>
+inline cudaError_t with_query_form(int form, F&& f) {
+    switch (form) {
+        case kQueryFp32: return f(std::integral_constant<int, kQueryFp32>{});
+        case kQueryHalf: return f(std::integral_constant<int, kQueryHalf>{});
+        case kQueryE5: return f(std::integral_constant<int, kQueryE5>{});
+        case kQueryMoved: return f(std::integral_constant<int, kQueryMoved>{});
+        case kQueryGamma1: return f(std::integral_constant<int, kQueryGamma1>{});
+        default: return f(std::integral_constant<int, kQueryGeneral>{});
+    }
 }
 
 // Largest BVH leaf (triangles); the traversal packs a leaf's first triangle
@@ -282,7 +313,7 @@ cudaError_t launch_trace_wavefront_multi(const DevScene& s, const VolSet& vs, co
                                          const float4* dirs, int R, const int32_t* perm, const int32_t* active,
                                          const int32_t* count, float4* records, int32_t* shadow_list,
                                          int32_t* hit_list, int32_t* shadow_count, int grid, cudaStream_t st,
-                                         bool fast_query);
+                                         int form);
 // Morton order of the octahedral positions of the unrotated spherical-
 // Fibonacci directions (host; a rotation keeps neighbouring directions together)
 std::vector<int32_t> ray_order_morton(int R);
@@ -345,7 +376,7 @@ cudaError_t launch_query(const VolView& v, const float* pos, const float* nrm, i
                          float3 camera, float* out, cudaStream_t st,
                          bool out_host = false);
 cudaError_t launch_query_cascade(const VolSet& vs, const float* pos, const float* nrm, int64_t n, float3 camera,
-                                 float* out, cudaStream_t st);
+                                 float* out, int form, cudaStream_t st);
 // Resets probe planes that a tracking window leapfrogged: planes[i] =
 // (volume, axis, physical plane index); count on the device.
 cudaError_t launch_reset_planes(const VolSet& vs, const int4* planes, const int32_t* count, int max_planes,

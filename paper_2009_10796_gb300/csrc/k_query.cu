@@ -9,12 +9,14 @@ namespace ddgi {
 // (16-byte stores when the run is aligned), so each warp writes whole lines,
 // for page-locked host memory written across the host link; otherwise each
 // thread stores its own three floats (device memory).
-// The specialised form runs five CTAs per SM (48 registers, a short spill),
-// which measured 1 us faster on the 1080p query than four; the general form
-// keeps four.
+// Five CTAs per SM (48 registers, a short spill) measured 1 us faster on the
+// 1080p query than four in the specialised forms; the general form keeps four,
+// and so do the gamma 1 and moved forms, whose points are often in random
+// order (281 and 300 us for 1080p of them, 290 and 312 us at five).
 constexpr int kQueryThreads = 256;
-template <bool STAGE_OUT, bool FAST>
-__global__ void __launch_bounds__(kQueryThreads, FAST ? 5 : 4) k_query(VolView v, const float* __restrict__ pos,
+constexpr int query_ctas(int form) { return form == kQueryGeneral || form == kQueryGamma1 || form == kQueryMoved ? 4 : 5; }
+template <bool STAGE_OUT, int FORM>
+__global__ void __launch_bounds__(kQueryThreads, query_ctas(FORM)) k_query(VolView v, const float* __restrict__ pos,
                                                          const float* __restrict__ nrm, int64_t n, float3 cam,
                                                          float* __restrict__ out) {
     pdl_wait();
@@ -30,7 +32,7 @@ __global__ void __launch_bounds__(kQueryThreads, FAST ? 5 : 4) k_query(VolView v
                 float3 wo = cam - x;
                 float l = length(wo);
                 wo = l < 1e-6f ? nn : (1.0f / l) * wo;
-                float3 M = query_M<FAST>(v, x, nn, wo);
+                float3 M = query_M<FORM>(v, x, nn, wo);
                 const float pi = 3.14159265358979323846f;
                 E = f3(pi * M.x, pi * M.y, pi * M.z);
             }
@@ -63,7 +65,7 @@ __global__ void __launch_bounds__(kQueryThreads, FAST ? 5 : 4) k_query(VolView v
 // Second-order glossy lookup (Sec. 4.4): one thread per reflection-ray hit;
 // dirs are the unit directions the hits were reached along.  Output is the
 // prefiltered radiance M read in the mirror direction (no factor pi).
-template <bool FAST>
+template <int FORM>
 __global__ void __launch_bounds__(256) k_query_glossy(VolView v, const float* __restrict__ pos,
                                                       const float* __restrict__ nrm, const float* __restrict__ dirs,
                                                       int64_t n, float* __restrict__ out) {
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(256) k_query_glossy(VolView v, const float* __
             float3 r = d - (2.0f * dn) * nn;
             float lr = length(r);
             if (lr > 0.0f) r = (1.0f / lr) * r;
-            M = query_M_look<FAST>(v, x, nn, f3(-d.x, -d.y, -d.z), r);
+            M = query_M_look<FORM>(v, x, nn, f3(-d.x, -d.y, -d.z), r);
         }
         out[3 * q] = M.x;
         out[3 * q + 1] = M.y;
@@ -142,6 +144,7 @@ cudaError_t launch_wake(const VolView& v, const float* boxes, int n_boxes, int b
 }
 
 // Cascade query (Sec. 7.3): one thread per point, volumes densest first.
+template <int FORM>
 __global__ void __launch_bounds__(256) k_query_cascade(VolSet vs, const float* __restrict__ pos,
                                                        const float* __restrict__ nrm, int64_t n, float3 cam,
                                                        float* __restrict__ out) {
@@ -154,7 +157,7 @@ __global__ void __launch_bounds__(256) k_query_cascade(VolSet vs, const float* _
             float3 wo = cam - x;
             float l = length(wo);
             wo = l < 1e-6f ? nn : (1.0f / l) * wo;
-            float3 M = cascade_M(vs.table, vs.n, x, nn, wo);
+            float3 M = cascade_M<FORM>(vs.table, vs.n, x, nn, wo);
             const float pi = 3.14159265358979323846f;
             E = f3(pi * M.x, pi * M.y, pi * M.z);
         }
@@ -223,12 +226,14 @@ __global__ void k_reset_planes(VolSet vs, const int4* __restrict__ planes, const
 }
 
 cudaError_t launch_query_cascade(const VolSet& vs, const float* pos, const float* nrm, int64_t n, float3 camera,
-                                 float* out, cudaStream_t st) {
+                                 float* out, int form, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + 255) / 256;
     int grid = (int)(blocks < 1048576 ? blocks : 1048576);
-    k_query_cascade<<<grid, 256, 0, st>>>(vs, pos, nrm, n, camera, out);
-    return cudaGetLastError();
+    return with_query_form(form, [&](auto f) {
+        k_query_cascade<decltype(f)::value><<<grid, 256, 0, st>>>(vs, pos, nrm, n, camera, out);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_build_list_multi(const VolSet& vs, int total, int which, int32_t* list, int32_t* count,
@@ -256,11 +261,11 @@ cudaError_t launch_query(const VolView& v, const float* pos, const float* nrm, i
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + kQueryThreads - 1) / kQueryThreads;
     int grid = (int)(blocks < 1048576 ? blocks : 1048576);
-    const bool fast = query_fast_view(v);
-    if (out_host && fast) return launch_pdl(k_query<true, true>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out);
-    if (out_host) return launch_pdl(k_query<true, false>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out);
-    if (fast) return launch_pdl(k_query<false, true>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out);
-    return launch_pdl(k_query<false, false>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out);
+    return with_query_form(query_form(v), [&](auto f) {
+        constexpr int F = decltype(f)::value;
+        return out_host ? launch_pdl(k_query<true, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out)
+                        : launch_pdl(k_query<false, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out);
+    });
 }
 
 cudaError_t launch_query_glossy(const VolView& v, const float* pos, const float* nrm, const float* dirs, int64_t n,
@@ -268,11 +273,10 @@ cudaError_t launch_query_glossy(const VolView& v, const float* pos, const float*
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + 255) / 256;
     int grid = (int)(blocks < 1048576 ? blocks : 1048576);
-    if (query_fast_view(v))
-        k_query_glossy<true><<<grid, 256, 0, st>>>(v, pos, nrm, dirs, n, out);
-    else
-        k_query_glossy<false><<<grid, 256, 0, st>>>(v, pos, nrm, dirs, n, out);
-    return cudaGetLastError();
+    return with_query_form(query_form(v), [&](auto f) {
+        k_query_glossy<decltype(f)::value><<<grid, 256, 0, st>>>(v, pos, nrm, dirs, n, out);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_build_list(const uint8_t* states, int P, int which, int32_t* list, int32_t* count,

@@ -158,8 +158,7 @@ __device__ __forceinline__ Footprint footprint(float2 u, int n) {
 // (bias 15), as in the OpenGL EXT_texture_shared_exponent specification.
 
 __device__ __forceinline__ float3 rgb9e5_decode(uint32_t w) {
-    int e = (int)(w >> 27) - 15 - 9;
-    float s = ldexpf(1.0f, e);
+    const float s = __int_as_float(((int)(w >> 27) - 15 - 9 + 127) << 23);   // 2^(e - 15 - 9)
     return f3((float)(w & 511u) * s, (float)((w >> 9) & 511u) * s, (float)((w >> 18) & 511u) * s);
 }
 
@@ -400,47 +399,174 @@ __device__ __forceinline__ uint64_t gamma_decode_g5_pair(float er, float eg) {
     return f2_mul(f2_mul(E, E), S);
 }
 
-// The specialised query of query_M_look<true> (FP32 atlases, gamma 5, no
-// probe offsets; query_fast_view): the same operations in the same order,
-// except the decode's zero test (gamma_decode_g5_pair), with the eight cage
-// corners unrolled, so each corner's probe index, grid offset and
-// trilinear factor are registers rather than per-probe selects, and the red
-// and green channels of the irradiance taps and their decode carried as
-// packed FP32 pairs (the blue channel scalar).
-__device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, float3 n, float3 wo, float3 look) {
-    const LocalPoint q = local_point(v, x, n, wo);
+// What a specialised query form fixes at compile time (query_form).
+template <int FORM>
+struct QueryForm {
+    static constexpr bool kHalf = FORM == kQueryHalf;        // FP16 atlases
+    static constexpr bool kE5 = FORM == kQueryE5;            // RGB9E5 irradiance
+    static constexpr bool kGamma1 = FORM == kQueryGamma1;    // gamma 1 (else 5)
+    static constexpr bool kMoved = FORM == kQueryMoved;      // probe offsets
+};
+
+// The four taps of a probe's irradiance tile at a footprint, bilinearly
+// weighted: red and green as a packed pair, blue.
+template <int FORM>
+__device__ __forceinline__ uint64_t irr_taps(const VolView& v, int p, const Footprint& f, const Bilerp& w, float& eb) {
+    const int row = v.irr_n + 2;
+    const int64_t t = (int64_t)p * v.irr_tile + ((int64_t)f.y0 * row + f.x0);
+    float3 q00, q10, q01, q11;
+    if constexpr (FORM == kQueryGeneral) {
+        const float3 e = sample_irr_at(v, p, f, w);
+        eb = e.z;
+        return f2_pack(e.x, e.y);
+    } else if constexpr (QueryForm<FORM>::kHalf) {
+        const uint2* a = (const uint2*)v.irr + t;
+        const uint2 h[4] = {__ldg(a), __ldg(a + 1), __ldg(a + row), __ldg(a + row + 1)};
+        float3* o[4] = {&q00, &q10, &q01, &q11};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 rg = __half22float2(*reinterpret_cast<const __half2*>(&h[k].x));
+            *o[k] = f3(rg.x, rg.y, __low2float(*reinterpret_cast<const __half2*>(&h[k].y)));
+        }
+    } else if constexpr (QueryForm<FORM>::kE5) {
+        const uint32_t* a = (const uint32_t*)v.irr + t;
+        const uint32_t h00 = __ldg(a), h10 = __ldg(a + 1), h01 = __ldg(a + row), h11 = __ldg(a + row + 1);
+        q00 = rgb9e5_decode(h00);
+        q10 = rgb9e5_decode(h10);
+        q01 = rgb9e5_decode(h01);
+        q11 = rgb9e5_decode(h11);
+    } else {
+        const float4* a = (const float4*)v.irr + t;
+        const float4 f00 = __ldg(a), f10 = __ldg(a + 1), f01 = __ldg(a + row), f11 = __ldg(a + row + 1);
+        q00 = f3(f00.x, f00.y, f00.z);
+        q10 = f3(f10.x, f10.y, f10.z);
+        q01 = f3(f01.x, f01.y, f01.z);
+        q11 = f3(f11.x, f11.y, f11.z);
+    }
+    uint64_t rg = f2_mul(f2_pack(w.w00, w.w00), f2_pack(q00.x, q00.y));
+    rg = f2_fma(f2_pack(w.w10, w.w10), f2_pack(q10.x, q10.y), rg);
+    rg = f2_fma(f2_pack(w.w01, w.w01), f2_pack(q01.x, q01.y), rg);
+    rg = f2_fma(f2_pack(w.w11, w.w11), f2_pack(q11.x, q11.y), rg);
+    eb = w.w00 * q00.z + w.w10 * q10.z + w.w01 * q01.z + w.w11 * q11.z;
+    return rg;
+}
+
+// The distance moments of a form's atlas at a footprint.
+template <int FORM>
+__device__ __forceinline__ float2 dist_taps(const VolView& v, int p, const Footprint& f) {
+    if constexpr (FORM == kQueryGeneral) return sample_dist_at(v, p, f);
+    if constexpr (!QueryForm<FORM>::kHalf) return sample_dist_fp32(v, p, f);
+    const int row = v.dist_n + 2;
+    const uint32_t* q = (const uint32_t*)v.dist + (int64_t)p * v.dist_tile + (int64_t)f.y0 * row + f.x0;
+    const uint32_t h[4] = {__ldg(q), __ldg(q + 1), __ldg(q + row), __ldg(q + row + 1)};
+    float2 a[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = __half22float2(*reinterpret_cast<const __half2*>(&h[k]));
+    const Bilerp w = bilerp_weights(f);
+    return make_float2(w.w00 * a[0].x + w.w10 * a[1].x + w.w01 * a[2].x + w.w11 * a[3].x,
+                       w.w00 * a[0].y + w.w10 * a[1].y + w.w01 * a[2].y + w.w11 * a[3].y);
+}
+
+// The eight-probe cage of a biased point: its base cell and, per axis, the
+// fraction and the two planes' physical index, x - x_p (high part) and
+// trilinear factor, so that a corner's values are registers.
+struct Cage {
+    int base[3];
+    int px[2], py[2], pz[2];
+    float ax[2], ay[2], az[2];
+    float tx[2], ty[2], tz[2];
+    __device__ __forceinline__ int probe(const VolView& v, int c) const {
+        return (c & 1 ? px[1] : px[0]) + v.counts.x * ((c & 2 ? py[1] : py[0]) + v.counts.y * (c & 4 ? pz[1] : pz[0]));
+    }
+};
+
+__device__ __forceinline__ Cage cage_of(const VolView& v, const LocalPoint& q) {
+    Cage k;
     const float g[3] = {(q.hi.x + q.lb.x) / v.spacing.x, (q.hi.y + q.lb.y) / v.spacing.y,
                         (q.hi.z + q.lb.z) / v.spacing.z};
     const int cnt[3] = {v.counts.x, v.counts.y, v.counts.z};
-    int base[3];
     float fr[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         float b = floorf(g[a]);
         b = fminf(fmaxf(b, 0.0f), (float)(cnt[a] - 2));
-        base[a] = (int)b;
+        k.base[a] = (int)b;
         fr[a] = fminf(fmaxf(g[a] - b, 0.0f), 1.0f);
     }
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+        k.px[o] = wrap_add(k.base[0] + o, v.shift.x, cnt[0]);
+        k.py[o] = wrap_add(k.base[1] + o, v.shift.y, cnt[1]);
+        k.pz[o] = wrap_add(k.base[2] + o, v.shift.z, cnt[2]);
+        k.ax[o] = q.hi.x - (float)(k.base[0] + o) * v.spacing.x;
+        k.ay[o] = q.hi.y - (float)(k.base[1] + o) * v.spacing.y;
+        k.az[o] = q.hi.z - (float)(k.base[2] + o) * v.spacing.z;
+        k.tx[o] = o ? fr[0] : 1.0f - fr[0];
+        k.ty[o] = o ? fr[1] : 1.0f - fr[1];
+        k.tz[o] = o ? fr[2] : 1.0f - fr[2];
+    }
+    return k;
+}
+
+// Weight of cage corner c (probe p) in a form's query: trilinear, backface
+// and Chebyshev factors, floored (query_M_look).  IEEE: the distance
+// and the lookup's coordinates by rounded square root and division instead of
+// the hardware reciprocals (the adjoint, where one point's weight can be a
+// whole texel's gradient: a Chebyshev weight near the depth it tests
+// magnifies their last bits).
+template <int FORM, bool IEEE = false>
+__device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoint& q, const Cage& k, int c, int p,
+                                               float3 n) {
+    const int o0 = c & 1, o1 = (c >> 1) & 1, o2 = c >> 2;
+    float3 a = f3(k.ax[o0], k.ay[o1], k.az[o2]);
+    if (QueryForm<FORM>::kMoved || (FORM == kQueryGeneral && v.offsets)) {
+        const float4 po = __ldg(v.offsets + p);   // the probe's own (moved) position; the cage stays on the grid
+        a = f3(a.x - po.x, a.y - po.y, a.z - po.z);
+    }
+    const float wt = k.tx[o0] * k.ty[o1] * k.tz[o2];
+    const float3 dp = f3(-(a.x + q.lo.x), -(a.y + q.lo.y), -(a.z + q.lo.z));   // probe - x
+    const float dd = dot(dp, dp);
+    const float cw = dd > 0.0f ? dot(n, dp) * rsqrtf(dd) : 1.0f;
+    const float hb = (1.0f + cw) * 0.5f;
+    const float wb = hb * hb + 0.2f;
+    const float3 pv = a + q.lb;                                                // biased point - probe
+    const float rr = dot(pv, pv);
+    float wc = 1.0f;
+    if (rr > 0.0f) {
+        const float r = IEEE ? sqrtf(rr) : rr * rsqrtf(rr);
+        const float ir = IEEE ? 1.0f / r : rsqrtf(rr);
+        const float2 u = IEEE ? oct_encode(ir * pv) : oct_encode_fast(ir * pv);
+        const float2 mom = dist_taps<FORM>(v, p, footprint(u, v.dist_n));
+        if (r > mom.x) {
+            const float var = fmaxf(mom.y - mom.x * mom.x, 0.0f);
+            const float dr = r - mom.x;
+            wc = __fdividef(var, var + dr * dr);
+        }
+    }
+    return wt * wb * fmaxf(wc, 1e-6f);
+}
+
+// The specialised query of query_M_look (FORM < kQueryGeneral): the same
+// operations in the same order, except the decode's zero test
+// (gamma_decode_g5_pair), with the eight cage corners unrolled, the storage
+// format, gamma and offsets fixed at compile time, and the red and green
+// channels of the irradiance taps and their decode carried as packed FP32
+// pairs (the blue channel scalar).  Bound by instruction issue for
+// neighbouring points: 1920 x 1080 of them on 16 x 8 x 16 probes take 118 us
+// with FP16 atlases (161 in the general form), 145 us with RGB9E5 (182),
+// 117 us with gamma 1 (142) and 118 us with probe offsets (140).  Points in
+// random order are bound by L2 sectors instead (222-300 us either way).
+template <int FORM>
+__device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, float3 n, float3 wo, float3 look) {
+    const LocalPoint q = local_point(v, x, n, wo);
+    const Cage k = cage_of(v, q);
     const Footprint fn = footprint(oct_encode(look), v.irr_n);
     const Bilerp wn = bilerp_weights(fn);
-    const uint64_t W00 = f2_pack(wn.w00, wn.w00), W10 = f2_pack(wn.w10, wn.w10);
-    const uint64_t W01 = f2_pack(wn.w01, wn.w01), W11 = f2_pack(wn.w11, wn.w11);
-    const int irow = v.irr_n + 2;
-    const int64_t itap = (int64_t)fn.y0 * irow + fn.x0;
-    // per axis, the cage's two planes: physical index, x - x_p (high part)
-    // and trilinear factor
-    const int px[2] = {wrap_add(base[0], v.shift.x, cnt[0]), wrap_add(base[0] + 1, v.shift.x, cnt[0])};
-    const int py[2] = {wrap_add(base[1], v.shift.y, cnt[1]), wrap_add(base[1] + 1, v.shift.y, cnt[1])};
-    const int pz[2] = {wrap_add(base[2], v.shift.z, cnt[2]), wrap_add(base[2] + 1, v.shift.z, cnt[2])};
-    const float ax[2] = {q.hi.x - (float)base[0] * v.spacing.x, q.hi.x - (float)(base[0] + 1) * v.spacing.x};
-    const float ay[2] = {q.hi.y - (float)base[1] * v.spacing.y, q.hi.y - (float)(base[1] + 1) * v.spacing.y};
-    const float az[2] = {q.hi.z - (float)base[2] * v.spacing.z, q.hi.z - (float)(base[2] + 1) * v.spacing.z};
-    const float tx[2] = {1.0f - fr[0], fr[0]}, ty[2] = {1.0f - fr[1], fr[1]}, tz[2] = {1.0f - fr[2], fr[2]};
     int pc[8];
     unsigned act = 0;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-        pc[c] = px[c & 1] + cnt[0] * (py[(c >> 1) & 1] + cnt[1] * pz[c >> 2]);
+        pc[c] = k.probe(v, c);
         act |= state_active(v.states[pc[c]]) ? 1u << c : 0u;
     }
     float sumw = 0.0f;
@@ -448,43 +574,21 @@ __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, 
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         if (!(act & (1u << c))) continue;
-        const int o0 = c & 1, o1 = (c >> 1) & 1, o2 = c >> 2;
-        const float3 a = f3(ax[o0], ay[o1], az[o2]);
-        const float wt = tx[o0] * ty[o1] * tz[o2];
-        const float3 dp = f3(-(a.x + q.lo.x), -(a.y + q.lo.y), -(a.z + q.lo.z));   // probe - x
-        const float dd = dot(dp, dp);
-        const float cw = dd > 0.0f ? dot(n, dp) * rsqrtf(dd) : 1.0f;
-        const float hb = (1.0f + cw) * 0.5f;
-        const float wb = hb * hb + 0.2f;
-        const float3 pv = a + q.lb;                                                // biased point - probe
-        const float rr = dot(pv, pv);
-        float wc = 1.0f;
-        if (rr > 0.0f) {
-            const float ir = rsqrtf(rr);
-            const float r = rr * ir;
-            const float2 mom = sample_dist_fp32(v, pc[c], footprint(oct_encode_fast(ir * pv), v.dist_n));
-            if (r > mom.x) {
-                const float var = fmaxf(mom.y - mom.x * mom.x, 0.0f);
-                const float dr = r - mom.x;
-                wc = __fdividef(var, var + dr * dr);
-            }
+        const float w = corner_weight<FORM>(v, q, k, c, pc[c], n);
+        float er, eg, eb;
+        f2_unpack(irr_taps<FORM>(v, pc[c], fn, wn, eb), er, eg);
+        if constexpr (QueryForm<FORM>::kGamma1) {
+            acc.x += w * gamma_decode_half_fast(er, 0.5f);
+            acc.y += w * gamma_decode_half_fast(eg, 0.5f);
+            acc.z += w * gamma_decode_half_fast(eb, 0.5f);
+        } else {
+            float dr_, dg_;
+            f2_unpack(gamma_decode_g5_pair(er, eg), dr_, dg_);
+            const float ebc = fmaxf(eb, 1e-30f);
+            acc.x += w * dr_;
+            acc.y += w * dg_;
+            acc.z += w * (ebc * ebc * (ebc * rsqrtf(ebc)));
         }
-        const float w = wt * wb * fmaxf(wc, 1e-6f);
-        const float4* ia = (const float4*)v.irr + ((int64_t)pc[c] * v.irr_tile + itap);
-        const float4 q00 = __ldg(ia), q10 = __ldg(ia + 1), q01 = __ldg(ia + irow), q11 = __ldg(ia + irow + 1);
-        uint64_t rg = f2_mul(W00, f2_pack(q00.x, q00.y));
-        rg = f2_fma(W10, f2_pack(q10.x, q10.y), rg);
-        rg = f2_fma(W01, f2_pack(q01.x, q01.y), rg);
-        rg = f2_fma(W11, f2_pack(q11.x, q11.y), rg);
-        const float eb = wn.w00 * q00.z + wn.w10 * q10.z + wn.w01 * q01.z + wn.w11 * q11.z;
-        float er, eg;
-        f2_unpack(rg, er, eg);
-        float dr_, dg_;
-        f2_unpack(gamma_decode_g5_pair(er, eg), dr_, dg_);
-        const float ebc = fmaxf(eb, 1e-30f);
-        acc.x += w * dr_;
-        acc.y += w * dg_;
-        acc.z += w * (ebc * ebc * (ebc * rsqrtf(ebc)));
         sumw += w;
     }
     if (!(sumw > 0.0f)) return f3(0.0f, 0.0f, 0.0f);
@@ -502,11 +606,11 @@ __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, 
 // `look` is the direction the irradiance tiles are read in: n for the
 // irradiance query, the mirror direction for a second-order glossy lookup
 // (Sec. 4.4); the bias and the backface weights use n either way.
-// FAST: the view is known to hold FP32 atlases, gamma 5 and no probe
-// offsets (query_fast_view); query_M_look_fast serves it.
-template <bool FAST = false>
+// FORM: the view's form (query_form); query_M_look_fast serves all but the
+// general one.
+template <int FORM = kQueryGeneral>
 __device__ __forceinline__ float3 query_M_look(const VolView& v, float3 x, float3 n, float3 wo, float3 look) {
-    if constexpr (FAST) return query_M_look_fast(v, x, n, wo, look);
+    if constexpr (FORM != kQueryGeneral) return query_M_look_fast<FORM>(v, x, n, wo, look);
     const LocalPoint q = local_point(v, x, n, wo);
     float g[3] = {(q.hi.x + q.lb.x) / v.spacing.x, (q.hi.y + q.lb.y) / v.spacing.y,
                   (q.hi.z + q.lb.z) / v.spacing.z};
@@ -578,9 +682,9 @@ __device__ __forceinline__ float3 query_M_look(const VolView& v, float3 x, float
     return f3(a.x * a.x, a.y * a.y, a.z * a.z);
 }
 
-template <bool FAST = false>
+template <int FORM = kQueryGeneral>
 __device__ __forceinline__ float3 query_M(const VolView& v, float3 x, float3 n, float3 wo) {
-    return query_M_look<FAST>(v, x, n, wo, n);
+    return query_M_look<FORM>(v, x, n, wo, n);
 }
 
 // Cascade value M at x (Sec. 7.3): volumes densest first; each volume's
@@ -594,7 +698,7 @@ __device__ __forceinline__ float volume_weight(const VolView& v, float3 x) {
     return wx * wy * wz;
 }
 
-template <bool FAST = false>
+template <int FORM = kQueryGeneral>
 __device__ __forceinline__ float3 cascade_M(const VolView* vols, int n, float3 x, float3 nrm, float3 wo) {
     float sum = 0.0f;
     float3 acc = f3(0.0f, 0.0f, 0.0f);
@@ -602,7 +706,7 @@ __device__ __forceinline__ float3 cascade_M(const VolView* vols, int n, float3 x
         const VolView& v = vols[k];
         float take = fminf(volume_weight(v, x), 1.0f - sum);
         if (!(take > 0.0f)) continue;
-        float3 M = query_M<FAST>(v, x, nrm, wo);
+        float3 M = query_M<FORM>(v, x, nrm, wo);
         acc = acc + take * M;
         sum += take;
         if (sum >= 1.0f) break;
