@@ -15,95 +15,222 @@
 
 namespace ddgi {
 
-// Reverse of query_M: M_c = A_c^2, A_c = sum_p w_p a_pc / sum_p w_p,
-// a_pc = b_pc^(gamma/2), b the bilinear sample of probe p's tile in
-// direction n.  Scatters dM into g_irr (float [P][tile][3]).
-__device__ void query_M_adjoint(const VolView& v, float3 x, float3 n, float3 wo, float3 dM, float* g_irr) {
-    const LocalPoint q = local_point(v, x, n, wo);
-    float g[3] = {(q.hi.x + q.lb.x) / v.spacing.x, (q.hi.y + q.lb.y) / v.spacing.y,
-                  (q.hi.z + q.lb.z) / v.spacing.z};
-    int cnt[3] = {v.counts.x, v.counts.y, v.counts.z};
-    int base[3];
-    float fr[3];
-    for (int a = 0; a < 3; ++a) {
-        float b = floorf(g[a]);
-        b = fminf(fmaxf(b, 0.0f), (float)(cnt[a] - 2));
-        base[a] = (int)b;
-        fr[a] = fminf(fmaxf(g[a] - b, 0.0f), 1.0f);
+// Per-warp scratch of the query adjoint: each point's eight corner gradients
+// (rows padded to 33 so the eight corners of one point lie on distinct
+// banks), its four bilinear weights, and one group's 96 sums.
+constexpr int kAdjWarps = 4;   // warps per block of the kernels that scatter
+struct AdjointScratch {
+    float4 d[8][33];
+    float4 bw[32];
+    float sum[96];
+};
+
+// The decode b^(gamma/2) of an encoded value and its slope without the
+// factor gamma/2, b^(gamma/2 - 1); both 0 for b <= 0.  The square roots are
+// b * rsqrt(b) (hardware reciprocal square root, about 2 ulp).
+template <int FORM>
+__device__ __forceinline__ float decode_slope(float b, float half_gamma, float& slope) {
+    if (!(b > 0.0f)) {
+        slope = 0.0f;
+        return 0.0f;
     }
-    float w8[8];
-    int p8[8];
-    float3 b8[8];
-    float sumw = 0.0f;
-    float3 acc = f3(0.0f, 0.0f, 0.0f);
-    Footprint fp = footprint(oct_encode(n), v.irr_n);
-    for (int c = 0; c < 8; ++c) {
-        int o0 = c & 1, o1 = (c >> 1) & 1, o2 = (c >> 2) & 1;
-        int p = probe_phys(v, base[0] + o0, base[1] + o1, base[2] + o2);
-        p8[c] = p;
-        w8[c] = 0.0f;
-        if (!state_active(v.states[p])) continue;
-        float3 a = local_to_probe(v, q, base[0] + o0, base[1] + o1, base[2] + o2);
-        if (v.offsets) {   // the probe's own (moved) position; the cage stays on the grid
-            const float4 po = v.offsets[p];
-            a = f3(a.x - po.x, a.y - po.y, a.z - po.z);
-        }
-        float wt = (o0 ? fr[0] : 1.0f - fr[0]) * (o1 ? fr[1] : 1.0f - fr[1]) * (o2 ? fr[2] : 1.0f - fr[2]);
-        float3 dp = f3(-(a.x + q.lo.x), -(a.y + q.lo.y), -(a.z + q.lo.z));   // probe - x
-        float ldp = length(dp);
-        float cw = ldp > 0.0f ? dot(n, dp) / ldp : 1.0f;
-        float hb = (1.0f + cw) * 0.5f;
-        float wb = hb * hb + 0.2f;
-        float3 pv = a + q.lb;                                                // biased point - probe
-        float r = length(pv);
-        float wc = 1.0f;
-        if (r > 0.0f) {
-            float2 mom = sample_dist(v, p, (1.0f / r) * pv);
-            if (r > mom.x) {
-                float var = fmaxf(mom.y - mom.x * mom.x, 0.0f);
-                float dr = r - mom.x;
-                wc = var / (var + dr * dr);
-            }
-        }
-        float w = wt * wb * fmaxf(wc, 1e-6f);
-        w8[c] = w;
-        float3 e = sample_irr(v, p, n);
-        b8[c] = e;
-        acc.x += w * gamma_decode_half(e.x, v.half_gamma);
-        acc.y += w * gamma_decode_half(e.y, v.half_gamma);
-        acc.z += w * gamma_decode_half(e.z, v.half_gamma);
-        sumw += w;
+    const bool general = FORM == kQueryGeneral;
+    if (QueryForm<FORM>::kGamma1 || (general && half_gamma == 0.5f)) {
+        slope = rsqrtf(b);
+        return b * slope;
     }
-    if (!(sumw > 0.0f)) return;
-    float inv = 1.0f / sumw;
-    float A[3] = {acc.x * inv, acc.y * inv, acc.z * inv};
-    float dMv[3] = {dM.x, dM.y, dM.z};
-    float bw[4] = {(1.0f - fp.tx) * (1.0f - fp.ty), fp.tx * (1.0f - fp.ty), (1.0f - fp.tx) * fp.ty, fp.tx * fp.ty};
-    int bx[4] = {fp.x0, fp.x0 + 1, fp.x0, fp.x0 + 1}, by[4] = {fp.y0, fp.y0, fp.y0 + 1, fp.y0 + 1};
-    const int N = v.irr_n + 2;
-    for (int c = 0; c < 8; ++c) {
-        if (!(w8[c] > 0.0f)) continue;
-        float bb[3] = {b8[c].x, b8[c].y, b8[c].z};
-        for (int ch = 0; ch < 3; ++ch) {
-            if (!(bb[ch] > 0.0f)) continue;
-            float d = dMv[ch] * 2.0f * A[ch] * w8[c] * inv * v.half_gamma * powf(bb[ch], v.half_gamma - 1.0f);
-            for (int j = 0; j < 4; ++j)
-                atomicAdd(g_irr + ((int64_t)p8[c] * v.irr_tile + by[j] * N + bx[j]) * 3 + ch, d * bw[j]);
-        }
+    if (!general || half_gamma == 2.5f) {
+        slope = b * (b * rsqrtf(b));
+        return b * slope;
+    }
+    slope = powf(b, half_gamma - 1.0f);
+    return powf(b, half_gamma);
+}
+
+// Six consecutive floats (a tap pair's two texels) added at p: pairs where
+// they are 8-byte aligned (tile rows start on odd words too).
+__device__ __forceinline__ void add_run6(float* p, float a0, float a1, float a2, float b0, float b1, float b2) {
+    if ((reinterpret_cast<uintptr_t>(p) & 7) == 0) {
+        atomicAdd(reinterpret_cast<float2*>(p), make_float2(a0, a1));
+        atomicAdd(reinterpret_cast<float2*>(p + 2), make_float2(a2, b0));
+        atomicAdd(reinterpret_cast<float2*>(p + 4), make_float2(b1, b2));
+    } else {
+        atomicAdd(p, a0);
+        atomicAdd(reinterpret_cast<float2*>(p + 1), make_float2(a1, a2));
+        atomicAdd(reinterpret_cast<float2*>(p + 3), make_float2(b0, b1));
+        atomicAdd(p + 5, b2);
     }
 }
 
-__global__ void k_query_adjoint(VolView v, const float* __restrict__ pos, const float* __restrict__ nrm, int64_t n,
-                                float3 cam, const float* __restrict__ dE, float* g_irr) {
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-        float3 x = f3(pos[3 * q], pos[3 * q + 1], pos[3 * q + 2]);
-        float3 nn = f3(nrm[3 * q], nrm[3 * q + 1], nrm[3 * q + 2]);
-        if (nn.x == 0.0f && nn.y == 0.0f && nn.z == 0.0f) continue;
-        float3 wo = cam - x;
-        float l = length(wo);
-        wo = l < 1e-6f ? nn : (1.0f / l) * wo;
-        const float pi = 3.14159265358979323846f;
-        query_M_adjoint(v, x, nn, wo, f3(pi * dE[3 * q], pi * dE[3 * q + 1], pi * dE[3 * q + 2]), g_irr);
+// Reverse of query_M for a warp's 32 points (all lanes call; valid: the lane
+// has one): M_c = A_c^2, A_c = sum_p w_p a_pc / sum_p w_p, a_pc =
+// b_pc^(gamma/2), b the bilinear sample of probe p's tile in direction n.
+// Adds dM's texel gradients to g_irr (float [P][tile][3]).
+//
+// A point touches 8 probes x 4 taps x 3 channels.  Bound by the atomics: one
+// float atomic for each of the 96 took 2068 us for a 1280 x 720 G-buffer (16 x
+// 8 x 16 probes), because neighbouring pixels share cage and footprint and so
+// all add to the same few words.  Here the lanes with the same cage and
+// footprint form a group; lane (corner, tap) sums the group's points through
+// shared memory, in lane order, and the 96 sums go out as three atomics a
+// lane on consecutive addresses (a tap pair's six floats are one run).  With
+// more than kAdjMaxGroups groups (scattered points) a group costs more than
+// it saves, and each lane adds its own 16 runs in pairs.  1920 x 1080 points
+// of a hall seen from inside: 4126 -> 249 us; the same points shuffled:
+// 1370 -> 785 us.
+constexpr int kAdjMaxGroups = 10;
+template <int FORM>
+__device__ __forceinline__ void query_M_adjoint_warp(const VolView& v, bool valid, float3 x, float3 n, float3 wo,
+                                                     float3 dM, float* g_irr, AdjointScratch& sh) {
+    constexpr int kUnroll = FORM == kQueryGeneral ? 1 : 8;
+    const int lane = threadIdx.x & 31;
+    const int N = v.irr_n + 2;
+    Cage cage{};
+    Footprint fp{0, 0, 0.0f, 0.0f};
+    Bilerp bw{};
+    if (valid) {
+        const LocalPoint q = local_point(v, x, n, wo);
+        cage = cage_of(v, q);
+        fp = footprint(oct_encode(n), v.irr_n);
+        bw = bilerp_weights(fp);
+        unsigned act = 0;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) act |= state_active(v.states[cage.probe(v, c)]) ? 1u << c : 0u;
+        float sumw = 0.0f;
+        float3 acc = f3(0.0f, 0.0f, 0.0f);
+        // w_c and the slopes of corner c in shared memory until the sums are known
+#pragma unroll kUnroll
+        for (int c = 0; c < 8; ++c) {
+            float4 d = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (act & (1u << c)) {
+                const int p = cage.probe(v, c);
+                const float w = corner_weight<FORM, true>(v, q, cage, c, p, n);
+                float er, eg, eb;
+                f2_unpack(irr_taps<FORM>(v, p, fp, bw, eb), er, eg);
+                acc.x += w * decode_slope<FORM>(er, v.half_gamma, d.x);
+                acc.y += w * decode_slope<FORM>(eg, v.half_gamma, d.y);
+                acc.z += w * decode_slope<FORM>(eb, v.half_gamma, d.z);
+                d.w = w;
+                sumw += w;
+            }
+            sh.d[c][lane] = d;
+        }
+        if (!(sumw > 0.0f)) {
+            valid = false;
+        } else {
+            // dM_c/db_pc = 2 A_c (w_p / sum w) gamma/2 b^(gamma/2 - 1)
+            const float inv = 1.0f / sumw;
+            const float k = 2.0f * v.half_gamma;
+            const float3 kA = f3(dM.x * (acc.x * inv) * k, dM.y * (acc.y * inv) * k, dM.z * (acc.z * inv) * k);
+#pragma unroll kUnroll
+            for (int c = 0; c < 8; ++c) {
+                const float4 d = sh.d[c][lane];
+                const float w = d.w > 0.0f ? d.w * inv : 0.0f;
+                // a zero slope (b <= 0) or weight gives 0, whatever dM is
+                sh.d[c][lane] = make_float4(w * d.x != 0.0f ? kA.x * (w * d.x) : 0.0f, w * d.y != 0.0f ? kA.y * (w * d.y) : 0.0f,
+                                            w * d.z != 0.0f ? kA.z * (w * d.z) : 0.0f, 0.0f);
+            }
+            sh.bw[lane] = make_float4(bw.w00, bw.w10, bw.w01, bw.w11);
+        }
+    }
+    // groups of equal cage and footprint (cells below 2^26, texel rows and
+    // columns below 2^6); the cell's probes differ with it
+    const unsigned long long cell = (unsigned)cage.base[0] + (unsigned long long)v.counts.x *
+                                        ((unsigned)cage.base[1] + (unsigned long long)v.counts.y * (unsigned)cage.base[2]);
+    const unsigned long long key = (cell << 12) | (unsigned)(fp.y0 << 6) | (unsigned)fp.x0;
+    unsigned left = __ballot_sync(0xffffffffu, valid);
+    const unsigned peers = __match_any_sync(0xffffffffu, valid ? key : ~0ull);
+    const unsigned leaders = __ballot_sync(0xffffffffu, valid && __ffs(peers) - 1 == lane);
+    __syncwarp();   // the corner gradients are in shared memory
+    if (__popc(leaders) > kAdjMaxGroups) {
+        if (valid) {
+#pragma unroll 1
+            for (int c = 0; c < 8; ++c) {
+                const float4 d = sh.d[c][lane];
+                if (d.x == 0.0f && d.y == 0.0f && d.z == 0.0f) continue;
+                float* g = g_irr + ((int64_t)cage.probe(v, c) * v.irr_tile + fp.y0 * N + fp.x0) * 3;
+                add_run6(g, d.x * bw.w00, d.y * bw.w00, d.z * bw.w00, d.x * bw.w10, d.y * bw.w10, d.z * bw.w10);
+                add_run6(g + 3 * N, d.x * bw.w01, d.y * bw.w01, d.z * bw.w01, d.x * bw.w11, d.y * bw.w11,
+                         d.z * bw.w11);
+            }
+        }
+        __syncwarp();
+        return;
+    }
+    const float* wp = reinterpret_cast<const float*>(sh.bw) + (lane & 3);
+    const float4* dp = sh.d[lane >> 2];
+    // of lane (corner, tap) and, for the atomics, of words lane + 32 k of the
+    // 96: corner, tap, channel = i / 12, i / 3 % 4, i % 3
+    while (left) {
+        const int leader = __ffs(left) - 1;
+        const unsigned group = __shfl_sync(0xffffffffu, peers, leader);
+        left &= ~group;
+        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+        if (group == 0xffffffffu) {
+#pragma unroll 8
+            for (int q = 0; q < 32; ++q) {
+                const float4 d = dp[q];
+                const float w = wp[4 * q];
+                s0 = fmaf(d.x, w, s0);
+                s1 = fmaf(d.y, w, s1);
+                s2 = fmaf(d.z, w, s2);
+            }
+        } else {
+            for (unsigned m = group; m; m &= m - 1) {
+                const int q = __ffs(m) - 1;
+                const float4 d = dp[q];
+                const float w = wp[4 * q];
+                s0 = fmaf(d.x, w, s0);
+                s1 = fmaf(d.y, w, s1);
+                s2 = fmaf(d.z, w, s2);
+            }
+        }
+        sh.sum[3 * lane] = s0;
+        sh.sum[3 * lane + 1] = s1;
+        sh.sum[3 * lane + 2] = s2;
+        // the leader's cage: physical planes of both sides of each axis, and its first tap
+        const int px0 = __shfl_sync(0xffffffffu, cage.px[0], leader), px1 = __shfl_sync(0xffffffffu, cage.px[1], leader);
+        const int py0 = __shfl_sync(0xffffffffu, cage.py[0], leader), py1 = __shfl_sync(0xffffffffu, cage.py[1], leader);
+        const int pz0 = __shfl_sync(0xffffffffu, cage.pz[0], leader), pz1 = __shfl_sync(0xffffffffu, cage.pz[1], leader);
+        const int tap0 = __shfl_sync(0xffffffffu, fp.y0 * N + fp.x0, leader);
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int i = lane + 32 * k;
+            const int t = i / 3, c = t >> 2;
+            const float s = sh.sum[i];
+            if (s != 0.0f) {
+                const int p = (c & 1 ? px1 : px0) + v.counts.x * ((c & 2 ? py1 : py0) + v.counts.y * (c & 4 ? pz1 : pz0));
+                const int tap = tap0 + ((t >> 1) & 1) * N + (t & 1);
+                atomicAdd(g_irr + ((int64_t)p * v.irr_tile + tap) * 3 + (i - 3 * t), s);
+            }
+        }
+        __syncwarp();   // the sums are read before the next group's are written
+    }
+}
+
+template <int FORM>
+__global__ void __launch_bounds__(32 * kAdjWarps) k_query_adjoint(VolView v, const float* __restrict__ pos,
+                                                                  const float* __restrict__ nrm, int64_t n, float3 cam,
+                                                                  const float* __restrict__ dE, float* g_irr) {
+    __shared__ AdjointScratch sh[kAdjWarps];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    // warp-uniform loop: 32 consecutive points per warp
+    for (int64_t q0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); q0 < n; q0 += stride) {
+        const int64_t q = q0 + (threadIdx.x & 31);
+        float3 x = f3(0.0f, 0.0f, 0.0f), nn = x, wo = x, dM = x;
+        bool valid = q < n;
+        if (valid) {
+            x = f3(pos[3 * q], pos[3 * q + 1], pos[3 * q + 2]);
+            nn = f3(nrm[3 * q], nrm[3 * q + 1], nrm[3 * q + 2]);
+            valid = nn.x != 0.0f || nn.y != 0.0f || nn.z != 0.0f;
+            wo = cam - x;
+            const float l = length(wo);
+            wo = l < 1e-6f ? nn : (1.0f / l) * wo;
+            const float pi = 3.14159265358979323846f;
+            dM = f3(pi * dE[3 * q], pi * dE[3 * q + 1], pi * dE[3 * q + 2]);
+        }
+        query_M_adjoint_warp<FORM>(v, valid, x, nn, wo, dM, g_irr, sh[threadIdx.x >> 5]);
     }
 }
 
@@ -171,7 +298,8 @@ __global__ void k_blend_adjoint(VolView v_after, const float* __restrict__ w_irr
 
 // Thread per (probe, ray) of frame f, re-traced against the scene.  v_before
 // is the atlas the frame's hit shading sampled (the previous frame's).
-__global__ void k_shade_adjoint(DevScene s, VolView v_before, Lights L, const float4* __restrict__ dirs, int P,
+template <int FORM>
+__global__ void __launch_bounds__(32 * kAdjWarps) k_shade_adjoint(DevScene s, VolView v_before, Lights L, const float4* __restrict__ dirs, int P,
                                 int R, const float4* __restrict__ gL, float* d_emit, float* d_albedo,
                                 float* g_prev, int with_prev) {
     const int64_t total = (int64_t)P * R;
@@ -179,6 +307,7 @@ __global__ void k_shade_adjoint(DevScene s, VolView v_before, Lights L, const fl
     const int lane = threadIdx.x & 31;
     const float3 tol = f3(-L.sun_dir.x, -L.sun_dir.y, -L.sun_dir.z);
     const RayPre r_sun = ray_pre(f3(0.0f, 0.0f, 0.0f), tol);
+    __shared__ AdjointScratch sh[kAdjWarps];
     int2 stack[kStackSize4];
     WwLane<kStackSize4, int2> w;
     w.stack = stack;
@@ -220,27 +349,28 @@ __global__ void k_shade_adjoint(DevScene s, VolView v_before, Lights L, const fl
             ww4_round<true>(s, sr, w);
         } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
         const bool lit = shadow && w.h.orig < 0;
-        if (!front) continue;
-        int2 at = __ldg(s.attr + h.orig);
-        if (at.y >= 0) {
-            atomicAdd(d_emit + 3 * at.y + 0, g4.x);
-            atomicAdd(d_emit + 3 * at.y + 1, g4.y);
-            atomicAdd(d_emit + 3 * at.y + 2, g4.z);
+        const float3 wo = f3(-d.x, -d.y, -d.z);
+        float3 dM = f3(0.0f, 0.0f, 0.0f);
+        if (front) {
+            int2 at = __ldg(s.attr + h.orig);
+            if (at.y >= 0) {
+                atomicAdd(d_emit + 3 * at.y + 0, g4.x);
+                atomicAdd(d_emit + 3 * at.y + 1, g4.y);
+                atomicAdd(d_emit + 3 * at.y + 2, g4.z);
+            }
+            float3 direct = f3(0.0f, 0.0f, 0.0f);
+            if (lit) {
+                float kk = cosl * 0.318309886183790672f;
+                direct = f3(L.sun_irr.x * kk, L.sun_irr.y * kk, L.sun_irr.z * kk);
+            }
+            float3 M = query_M<FORM>(v_before, x, n, wo);
+            atomicAdd(d_albedo + 3 * at.x + 0, g4.x * (direct.x + M.x));
+            atomicAdd(d_albedo + 3 * at.x + 1, g4.y * (direct.y + M.y));
+            atomicAdd(d_albedo + 3 * at.x + 2, g4.z * (direct.z + M.z));
+            const float4 rho = __ldg(s.albedo + at.x);
+            dM = f3(g4.x * rho.x, g4.y * rho.y, g4.z * rho.z);
         }
-        float3 direct = f3(0.0f, 0.0f, 0.0f);
-        if (lit) {
-            float kk = cosl * 0.318309886183790672f;
-            direct = f3(L.sun_irr.x * kk, L.sun_irr.y * kk, L.sun_irr.z * kk);
-        }
-        float3 wo = f3(-d.x, -d.y, -d.z);
-        float3 M = query_M(v_before, x, n, wo);
-        atomicAdd(d_albedo + 3 * at.x + 0, g4.x * (direct.x + M.x));
-        atomicAdd(d_albedo + 3 * at.x + 1, g4.y * (direct.y + M.y));
-        atomicAdd(d_albedo + 3 * at.x + 2, g4.z * (direct.z + M.z));
-        if (with_prev) {
-            float4 rho = __ldg(s.albedo + at.x);
-            query_M_adjoint(v_before, x, n, wo, f3(g4.x * rho.x, g4.y * rho.y, g4.z * rho.z), g_prev);
-        }
+        if (with_prev) query_M_adjoint_warp<FORM>(v_before, front, x, n, wo, dM, g_prev, sh[threadIdx.x >> 5]);
     }
 }
 
@@ -269,8 +399,11 @@ static int grid_for(int64_t n, int block) {
 cudaError_t launch_query_adjoint(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam,
                                  const float* dE, float* g_irr, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    k_query_adjoint<<<grid_for(n, 128), 128, 0, st>>>(v, pos, nrm, n, cam, dE, g_irr);
-    return cudaGetLastError();
+    return with_query_form(query_form(v), [&](auto f) {
+        k_query_adjoint<decltype(f)::value><<<grid_for(n, 32 * kAdjWarps), 32 * kAdjWarps, 0, st>>>(v, pos, nrm, n, cam,
+                                                                                                   dE, g_irr);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_border_fold(float* g_irr, int P, int n, cudaStream_t st) {
@@ -287,9 +420,11 @@ cudaError_t launch_blend_adjoint(const VolView& v_after, const float* w_irr, con
 cudaError_t launch_shade_adjoint(const DevScene& s, const VolView& v_before, const Lights& L, const float4* dirs,
                                  int P, int R, const float4* gL, float* d_emit, float* d_albedo, float* g_prev,
                                  int with_prev, cudaStream_t st) {
-    k_shade_adjoint<<<grid_for((int64_t)P * R, 128), 128, 0, st>>>(s, v_before, L, dirs, P, R, gL, d_emit,
-                                                                   d_albedo, g_prev, with_prev);
-    return cudaGetLastError();
+    return with_query_form(query_form(v_before), [&](auto f) {
+        k_shade_adjoint<decltype(f)::value><<<grid_for((int64_t)P * R, 32 * kAdjWarps), 32 * kAdjWarps, 0, st>>>(
+            s, v_before, L, dirs, P, R, gL, d_emit, d_albedo, g_prev, with_prev);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_set_materials(float4* albedo, int n_obj, const float* alb, float4* emit, int n_em, const float* em,
