@@ -1708,7 +1708,6 @@ ddgi_status ddgi_diff_backward(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
     float* g = v->g_irr;
     float* gp = v->g_prev;
     for (int f = n_frames - 1; f >= 0; --f) {
-        DDGI_CK(launch_border_fold(g, (int)v->P, d.irr_n, st));
         FrameRot rot = frame_rotation(d.seed, first_frame + f);
         DDGI_CK(launch_frame_setup(rot, v->R, d.irr_n, d.dist_n, d.dist_cos_power, v->sf64, v->dirs, v->w_irr,
                                    v->inv_s_irr, v->w_dist, v->inv_s_dist, nullptr, 0, st));

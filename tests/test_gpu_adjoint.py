@@ -220,3 +220,21 @@ def test_fp64_adjoint_matches_central_differences(g, gamma):
           f"emitter grad {rel_err(ge, g_em_ref).max():.2e}")
     assert worst <= 1e-5
     assert np.median(eE) <= 1e-5
+
+
+@pytest.mark.parametrize("irr_n, counts, rays", [(5, (3, 3, 2), 37), (28, (2, 2, 2), 16)])
+def test_blend_adjoint_tiles(g, irr_n, counts, rays):
+    """Probe counts that are no multiple of the adjoint's block of four, odd
+    ray counts, and the largest tiles (one probe a block), at the bound of
+    test_adjoint_matches_oracle_gradient."""
+    sc, L, desc, pos, nrm, G, cam = _setup(1.0)
+    desc.irr_n, desc.counts, desc.rays_per_probe = irr_n, counts, rays
+    desc.spacing = tuple(4.5 / (c - 1) for c in counts)
+    E_ref, g_em_ref, g_al_ref = oracle.diff(oracle.SceneHandle(sc), L, desc, pos, nrm, cam, G)
+    S, V = g.Scene.from_arrays(sc), g.Volume(desc)
+    albedo = torch.tensor(sc.object_albedo, dtype=torch.float32, device="cuda", requires_grad=True)
+    emit = torch.tensor(sc.emitter_radiance, dtype=torch.float32, device="cuda", requires_grad=True)
+    E = g.IrradianceField.apply(albedo, emit, V, S, L, to_dev(pos), to_dev(nrm), cam, 0, 2)
+    (E * to_dev(G)).sum().backward()
+    assert rel_err(albedo.grad.cpu().numpy(), g_al_ref).max() <= 1e-3
+    assert rel_err(emit.grad.cpu().numpy(), g_em_ref).max() <= 1e-3
