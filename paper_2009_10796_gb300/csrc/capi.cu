@@ -771,7 +771,7 @@ static ddgi_status update_impl(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
                                        v->counts + 4, kCounterInts - 4, st));
             DDGI_CK(launch_trace_wavefront(s->dev, view, make_lights(lights), v->conv_dirs, v->R, v->perm, v->lists,
                                            v->counts + 2, v->records, v->shadow_list, v->hit_list, v->shadow_count,
-                                           sms * 8, st, nullptr));
+                                           sms * 8, (end - begin) * v->R, st, nullptr));
             DDGI_CK(launch_converge_accum(v->R, d.irr_n, d.dist_n, v->conv_w_irr, v->conv_w_dist, v->records,
                                           v->counts + 2, v->conv_acc_irr, v->conv_acc_dist, v->conv_den, b == 0,
                                           sms * 8, st));
@@ -796,7 +796,7 @@ static ddgi_status update_impl(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
             for (auto& m : marks) DDGI_CK(cudaEventCreate(&m));
         DDGI_CK(launch_trace_wavefront(s->dev, view, make_lights(lights), v->dirs, v->R, v->perm, v->lists + v->P,
                                        v->counts + 1, v->records, v->shadow_list, v->hit_list, v->shadow_count, sms * 8,
-                                       st, v->timing ? marks : nullptr));
+                                       (end - begin) * v->R, st, v->timing ? marks : nullptr));
         if (v->timing) {
             v->stages[5].pending.emplace_back(marks[0], marks[1]);
             v->stages[6].pending.emplace_back(marks[1], marks[2]);
@@ -1226,7 +1226,7 @@ ddgi_status cascade_enqueue(ddgi_cascade_s* c, const DevScene& sc, const Lights&
     DDGI_CK(launch_build_list_multi(vs, (int)c->total, 1, c->lists + c->total, c->counts + 1, st));
     DDGI_CK(launch_trace_wavefront_multi(sc, vs, L, c->dirs, c->R, c->perm, c->lists + c->total, c->counts + 1,
                                          c->records, c->shadow_list, c->hit_list, c->shadow_count, sms * c->trace_mult,
-                                         st, query_form(c->h_params[slot]->views[0])));
+                                         c->total * c->R, st, query_form(c->h_params[slot]->views[0])));
     if (tensor)
         DDGI_CK(launch_blend_tc_set(vs, true, bp, precision, d0.irr_n, d0.dist_n, c->pack_w, c->inv_irr_r,
                                     c->inv_dist_r, c->records, c->lists + c->total, c->counts + 1, c->status, sms, st));

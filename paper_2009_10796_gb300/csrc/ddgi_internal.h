@@ -296,12 +296,13 @@ constexpr int kCounterInts = 10;
 // shadow pass, then shading of the front hits.  shadow_list and hit_list
 // hold one int32 per ray (active probes x R); shadow_count is 6 int32 of
 // device scratch, 8-byte aligned, zeroed by the caller: shadow rays, front
-// hits, the 64-bit work counters of the primary and the shadow pass.
+// hits, then the work counters of the primary ([2]) and the shadow pass
+// ([4]).  max_rays: an upper bound of active probes x R (it bounds the grids).
 // marks: 4 events recorded around the three passes, or nullptr.
 cudaError_t launch_trace_wavefront(const DevScene& s, const VolView& v, const Lights& L, const float4* dirs,
                                    int R, const int32_t* perm, const int32_t* active, const int32_t* count,
                                    float4* records, int32_t* shadow_list, int32_t* hit_list, int32_t* shadow_count,
-                                   int grid, cudaStream_t st, cudaEvent_t* marks);
+                                   int grid, int64_t max_rays, cudaStream_t st, cudaEvent_t* marks);
 // Measurement build of the primary and shadow passes: adds 4-wide node
 // visits and triangle tests to stats[1], [2] (primary) and [4], [5] (shadow);
 // the shadow-ray and front-hit counts are left in shadow_count[0], [1].
@@ -312,8 +313,8 @@ cudaError_t launch_trace_count(const DevScene& s, const VolView& v, const Lights
 cudaError_t launch_trace_wavefront_multi(const DevScene& s, const VolSet& vs, const Lights& L,
                                          const float4* dirs, int R, const int32_t* perm, const int32_t* active,
                                          const int32_t* count, float4* records, int32_t* shadow_list,
-                                         int32_t* hit_list, int32_t* shadow_count, int grid, cudaStream_t st,
-                                         int form);
+                                         int32_t* hit_list, int32_t* shadow_count, int grid, int64_t max_rays,
+                                         cudaStream_t st, int form);
 // Morton order of the octahedral positions of the unrotated spherical-
 // Fibonacci directions (host; a rotation keeps neighbouring directions together)
 std::vector<int32_t> ray_order_morton(int R);

@@ -8,6 +8,8 @@
 // spherical-Fibonacci pattern).  Kernels are persistent: the grid is sized to
 // the machine and threads stride over the device-side work count, so the host
 // never waits for the active-probe count.
+#include <algorithm>
+
 #include "traverse.cuh"
 
 namespace ddgi {
@@ -246,125 +248,106 @@ __device__ __forceinline__ void hit_frame(const DevScene& s, int k, float3& ng) 
     ng = cross(f3(p1.x - p0.x, p1.y - p0.y, p1.z - p0.z), f3(p2.x - p0.x, p2.y - p0.y, p2.z - p0.z));
 }
 
-// Persistent passes: each warp walks its lanes' rays in while-while rounds
-// and, once kRefillLanes lanes have finished, hands the idle lanes the next
-// work items from a global counter with one warp-aggregated atomic (Aila and
-// Laine 2009, persistent threads).  kRefillLanes = 32 (refill only when the
-// whole warp is idle) measured fastest on the city workload: 4, 8 and 16
-// cost more in lost ray coherence than they won back in busy lanes.
-constexpr int kRefillLanes = 32;
-
-// Hands idle lanes the next work items; returns the lane's item or -1.
-// Probe slot of work item (or record) idx = slot * R + ray.
-__device__ __forceinline__ int ray_slot(int64_t idx, int R, FastDiv dR) {
-    return idx <= INT32_MAX ? (int)fast_div((uint32_t)idx, dR) : (int)(idx / R);
+// Persistent passes: a warp walks its lanes' rays in while-while rounds and,
+// once every lane has finished, takes the next 32 work items (Aila and Laine
+// 2009, persistent threads; refilling at 4, 8 or 16 idle lanes measured
+// slower on the city workload, in lost ray coherence).  The first batch is
+// the warp's own index and only later ones come from the global counter,
+// which starts after them: with few rays, thousands of warps would
+// otherwise queue on one word to learn that nothing is left.  Work items are
+// below 2^31 (probes x rays is), a batch past the end below 2^32.
+constexpr unsigned kNoBatch = 0xffffffffu;
+__device__ __forceinline__ unsigned first_batch() { return (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; }
+__device__ __forceinline__ unsigned next_batch(uint32_t* next) {
+    unsigned base = 0;
+    if ((threadIdx.x & 31) == 0) base = gridDim.x * blockDim.x + atomicAdd(next, 32u);
+    return __shfl_sync(0xffffffffu, base, 0);
 }
 
-__device__ __forceinline__ int64_t refill(unsigned long long* next, int64_t total, bool idle_lane,
-                                          bool& exhausted) {
-    const unsigned idle = __ballot_sync(0xffffffffu, idle_lane);
-    if (exhausted || !(idle == 0xffffffffu || __popc(idle) >= kRefillLanes)) return -1;
-    const int lane = threadIdx.x & 31;
-    const int n = __popc(idle), leader = __ffs(idle) - 1;
-    unsigned long long base = 0;
-    if (lane == leader) base = atomicAdd(next, (unsigned long long)n);
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if ((int64_t)base + n >= total) exhausted = true;
-    if (!idle_lane) return -1;
-    int64_t w = (int64_t)base + __popc(idle & ((1u << lane) - 1u));
-    return w < total ? w : -1;
-}
+// CTAs per SM that both passes are built for (48 registers a thread).
+constexpr int kTraceCtas = 5;
 
 // COUNT: measurement build that adds its 4-wide node visits and triangle
 // tests to stats[1], stats[2] (otherwise identical).
 template <bool MULTI, bool COUNT = false>
-__global__ void __launch_bounds__(256, 5) k_trace_primary(DevScene s, VolSet vs, Lights L,
-                                                       const float4* __restrict__ dirs, int R, FastDiv dR,
-                                                       const int32_t* __restrict__ perm,
-                                                       const int32_t* __restrict__ active,
-                                                       const int32_t* __restrict__ count,
-                                                       float4* __restrict__ hits,
-                                                       int32_t* __restrict__ shadow_list,
-                                                       int32_t* __restrict__ hit_list,
-                                                       int32_t* shadow_count,
-                                                       unsigned long long* next,
-                                                       unsigned long long* stats = nullptr) {
+__global__ void __launch_bounds__(256, kTraceCtas) k_trace_primary(
+    DevScene s, VolSet vs, Lights L, const float4* __restrict__ dirs, int R, FastDiv dR,
+    const int32_t* __restrict__ perm, const int32_t* __restrict__ active, const int32_t* __restrict__ count,
+    float4* __restrict__ hits, int32_t* __restrict__ shadow_list, int32_t* __restrict__ hit_list, int32_t* shadow_count,
+    uint32_t* next, unsigned long long* stats) {
     pdl_wait();
     pdl_trigger();
     const int lane = threadIdx.x & 31;
-    const int64_t total = (int64_t)(*count) * R;
+    const unsigned total = (unsigned)(*count) * (unsigned)R;
     TraceCount tc;
-    const float3 tol = f3(-L.sun_dir.x, -L.sun_dir.y, -L.sun_dir.z);
-    int64_t rec = -1;   // record index of the lane's ray, -1 when idle
-    int entry = 0;      // its probe's list entry
-    bool exhausted = false;
-    RayPre r = ray_pre(f3(0.0f, 0.0f, 0.0f), f3(0.0f, 0.0f, 1.0f));   // the lane's ray (r.d its direction)
     int2 stack[kStackSize4];
     WwLane<kStackSize4, int2> w;
     w.stack = stack;
-    ww_start(s, w, false);
-    while (true) {
-        int64_t item = refill(next, total, rec < 0, exhausted);
-        if (item >= 0) {
-            // work item -> (probe slot, ray): consecutive items take a compact
-            // cone of directions; the record keeps its canonical ray index
-            int slot = ray_slot(item, R, dR);
-            int j = (int)(item - (int64_t)slot * R);
-            int i = perm ? __ldg(perm + j) : j;
-            rec = (int64_t)slot * R + i;
-            entry = __ldg(active + slot);
-            float3 o = probe_pos_phys(vol_of<MULTI>(vs, entry >> kEntryShift), entry & kEntryMask);
+    for (unsigned b = first_batch(); b < total; b = next_batch(next)) {
+        // work item -> (probe slot, ray): consecutive items take a compact
+        // cone of directions; the record keeps its canonical ray index
+        int rec;
+        RayPre r;
+        {
+            const int item = (int)min(b + lane, total - 1);
+            const int slot = (int)fast_div((uint32_t)item, dR);
+            const int j = item - slot * R;
+            const int i = perm ? __ldg(perm + j) : j;
+            rec = slot * R + i;
+            const int entry = __ldg(active + slot);
             const float4 d4 = __ldg(dirs + i);
-            r = ray_pre_packed(o, f3(d4.x, d4.y, d4.z), __ldg(dirs + R + 2 * i), __ldg(dirs + R + 2 * i + 1));
-            ww_start(s, w, true);
+            r = ray_pre_packed(probe_pos_phys(vol_of<MULTI>(vs, entry >> kEntryShift), entry & kEntryMask),
+                               f3(d4.x, d4.y, d4.z), __ldg(dirs + R + 2 * i), __ldg(dirs + R + 2 * i + 1));
         }
-        if (__ballot_sync(0xffffffffu, rec >= 0) == 0) break;
-        ww4_round<false, COUNT>(s, r, w, &tc);
+        const bool valid = b + lane < total;
+        ww_start(s, w, valid);
+        do {
+            ww4_round<false, COUNT>(s, r, w, &tc);
+        } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
         bool need = false, front = false;
-        int64_t done = -1;
-        if (rec >= 0 && w.node == kDone) {
+        if (valid) {
             // misses and back faces get their final record here; front hits
-            // keep (t, triangle) for the shading pass
+            // keep (t, triangle) for the shading pass.  The probe and the
+            // direction are read again (rec made opaque) rather than held
+            // across the walk, whose registers they would push out.
+            asm volatile("" : "+r"(rec));
+            const int slot = (int)fast_div((uint32_t)rec, dR);
+            const float4 d4 = __ldg(dirs + (rec - slot * R));
+            const float3 d = f3(d4.x, d4.y, d4.z);
             const Hit& h = w.h;
-            const float t_max = vol_of<MULTI>(vs, entry >> kEntryShift).t_max;
+            const float t_max = MULTI ? vol_of<MULTI>(vs, __ldg(active + slot) >> kEntryShift).t_max : vs.single.t_max;
             float4 out;
             if (h.orig < 0) {
-                float c = dot(r.d, L.sky_up);
+                float c = dot(d, L.sky_up);
                 out = make_float4(L.sky_a.x + L.sky_b.x * c, L.sky_a.y + L.sky_b.y * c, L.sky_a.z + L.sky_b.z * c,
                                   t_max);
             } else {
                 float3 ng;
                 hit_frame(s, h.k, ng);
-                if (dot(r.d, ng) > 0.0f) {
+                if (dot(d, ng) > 0.0f) {
                     out = make_float4(0.0f, 0.0f, 0.0f, fminf(0.2f * h.t, t_max));
                 } else {
                     front = true;
                     if (L.sun_on) {
                         float3 n = (1.0f / length(ng)) * ng;
-                        need = dot(n, tol) > 0.0f;
+                        need = dot(n, f3(-L.sun_dir.x, -L.sun_dir.y, -L.sun_dir.z)) > 0.0f;
                     }
                     out = make_float4(h.t, __int_as_float(h.k), 0.0f, 0.0f);
                 }
             }
             hits[rec] = out;
-            done = rec;
-            rec = -1;
         }
-        unsigned mask = __ballot_sync(0xffffffffu, need);
-        if (mask) {
-            int leader = __ffs(mask) - 1;
-            int off = 0;
-            if (lane == leader) off = atomicAdd(shadow_count, __popc(mask));
-            off = __shfl_sync(0xffffffffu, off, leader);
-            if (need) shadow_list[off + __popc(mask & ((1u << lane) - 1u))] = (int32_t)done;
-        }
-        mask = __ballot_sync(0xffffffffu, front);
-        if (mask) {
-            int leader = __ffs(mask) - 1;
-            int off = 0;
-            if (lane == leader) off = atomicAdd(shadow_count + 1, __popc(mask));
-            off = __shfl_sync(0xffffffffu, off, leader);
-            if (front) hit_list[off + __popc(mask & ((1u << lane) - 1u))] = (int32_t)done;
+        // both lists' places with one 64-bit atomic (shadow rays in the low word)
+        const unsigned mask_s = __ballot_sync(0xffffffffu, need), mask_f = __ballot_sync(0xffffffffu, front);
+        if (mask_f) {
+            unsigned long long off = 0;
+            if (lane == 0)
+                off = atomicAdd(reinterpret_cast<unsigned long long*>(shadow_count),
+                                ((unsigned long long)__popc(mask_f) << 32) | (unsigned)__popc(mask_s));
+            off = __shfl_sync(0xffffffffu, off, 0);
+            const unsigned below = (1u << lane) - 1u;
+            if (need) shadow_list[(unsigned)off + __popc(mask_s & below)] = rec;
+            if (front) hit_list[(unsigned)(off >> 32) + __popc(mask_f & below)] = rec;
         }
     }
     if (COUNT) {
@@ -375,53 +358,39 @@ __global__ void __launch_bounds__(256, 5) k_trace_primary(DevScene s, VolSet vs,
 
 // COUNT: adds 4-wide node visits and triangle tests to stats[4], stats[5].
 template <bool MULTI, bool COUNT = false>
-__global__ void __launch_bounds__(256) k_trace_shadow(DevScene s, VolSet vs, Lights L,
-                                                      const float4* __restrict__ dirs, int R, FastDiv dR,
-                                                      const int32_t* __restrict__ active,
-                                                      float4* __restrict__ hits,
-                                                      const int32_t* __restrict__ shadow_list,
-                                                      const int32_t* __restrict__ shadow_count,
-                                                      unsigned long long* next,
-                                                      unsigned long long* stats = nullptr) {
+__global__ void __launch_bounds__(256, kTraceCtas) k_trace_shadow(
+    DevScene s, VolSet vs, Lights L, const float4* __restrict__ dirs, int R, FastDiv dR,
+    const int32_t* __restrict__ active, float4* __restrict__ hits, const int32_t* __restrict__ shadow_list,
+    const int32_t* __restrict__ shadow_count, uint32_t* next, unsigned long long* stats) {
     pdl_wait();
     pdl_trigger();
-    const int64_t total = *shadow_count;
+    const int lane = threadIdx.x & 31;
+    const unsigned total = (unsigned)*shadow_count;
     TraceCount tc;
-    const float3 tol = f3(-L.sun_dir.x, -L.sun_dir.y, -L.sun_dir.z);
-    int64_t rec = -1;
-    bool exhausted = false;
-    const RayPre r_sun = ray_pre(f3(0.0f, 0.0f, 0.0f), tol);   // every shadow ray runs towards the sun
-    RayPre r = r_sun;
+    RayPre r = ray_pre(f3(0.0f, 0.0f, 0.0f), f3(-L.sun_dir.x, -L.sun_dir.y, -L.sun_dir.z));   // every shadow ray runs towards the sun
     int stack[kStackSize4];   // any-hit walk: plain references (no hit distance to prune by)
     WwLane<kStackSize4> w;
     w.stack = stack;
-    ww_start(s, w, false);
-    while (true) {
-        int64_t item = refill(next, total, rec < 0, exhausted);
-        if (item >= 0) {
-            rec = __ldg(shadow_list + item);
-            int slot = ray_slot(rec, R, dR);
-            int i = (int)(rec - (int64_t)slot * R);
-            int e = __ldg(active + slot);
-            float3 o = probe_pos_phys(vol_of<MULTI>(vs, e >> kEntryShift), e & kEntryMask);
-            float4 d4 = __ldg(dirs + i);
-            float3 d = f3(d4.x, d4.y, d4.z);
-            float4 hr = hits[rec];
-            float3 ng;
-            hit_frame(s, __float_as_int(hr.y), ng);
-            float3 nn = (1.0f / length(ng)) * ng;
-            float3 x = o + hr.x * d;
-            float off = 1e-4f * (1.0f + length(x));
-            r = r_sun;
-            ray_set_origin(r, x + off * nn);
-            ww_start(s, w, true);
-        }
-        if (__ballot_sync(0xffffffffu, rec >= 0) == 0) break;
-        ww4_round<true, COUNT>(s, r, w, &tc);
-        if (rec >= 0 && w.node == kDone) {
-            if (w.h.orig < 0) reinterpret_cast<float*>(hits)[4 * rec + 2] = 1.0f;
-            rec = -1;
-        }
+    for (unsigned b = first_batch(); b < total; b = next_batch(next)) {
+        const bool valid = b + lane < total;
+        const int rec = __ldg(shadow_list + (valid ? b + lane : b));
+        const int slot = (int)fast_div((uint32_t)rec, dR);
+        const int i = rec - slot * R;
+        const int e = __ldg(active + slot);
+        const float3 o = probe_pos_phys(vol_of<MULTI>(vs, e >> kEntryShift), e & kEntryMask);
+        const float4 d4 = __ldg(dirs + i);
+        const float4 hr = hits[rec];
+        float3 ng;
+        hit_frame(s, __float_as_int(hr.y), ng);
+        const float3 nn = (1.0f / length(ng)) * ng;
+        const float3 x = o + hr.x * f3(d4.x, d4.y, d4.z);
+        const float off = 1e-4f * (1.0f + length(x));
+        ray_set_origin(r, x + off * nn);
+        ww_start(s, w, valid);
+        do {
+            ww4_round<true, COUNT>(s, r, w, &tc);
+        } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
+        if (valid && w.h.orig < 0) reinterpret_cast<float*>(hits)[4 * (int64_t)rec + 2] = 1.0f;
     }
     if (COUNT) {
         atomicAdd(stats + 4, (unsigned long long)tc.nodes);
@@ -440,9 +409,9 @@ __global__ void __launch_bounds__(256, 4) k_shade(DevScene s, VolSet vs, Lights 
     pdl_trigger();
     const int n_hits = *hit_count;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n_hits; q += gridDim.x * blockDim.x) {
-        const int64_t idx = __ldg(hit_list + q);
-        const int slot = ray_slot(idx, R, dR);
-        const int i = (int)(idx - (int64_t)slot * R);
+        const int idx = __ldg(hit_list + q);
+        const int slot = (int)fast_div((uint32_t)idx, dR);
+        const int i = idx - slot * R;
         float4 d4 = __ldg(dirs + i);
         float3 d = f3(d4.x, d4.y, d4.z);
         float4 hr = records[idx];
@@ -650,15 +619,25 @@ cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights
     return cudaGetLastError();
 }
 
+// Blocks of 256 threads for at most max_items of them, no more than `grid`
+// nor, for the persistent passes, than are resident at once (a block of a
+// later wave would start its own first batch when the others are done).
+static int bounded_grid(int grid, int64_t max_items) {
+    const int64_t need = (max_items + 255) / 256;
+    return need < grid ? (need > 0 ? (int)need : 1) : grid;
+}
+
 template <bool MULTI>
 static cudaError_t trace_wavefront(const DevScene& s, const VolSet& vs, const Lights& L, const float4* dirs, int R,
                                    const int32_t* perm, const int32_t* active, const int32_t* count,
                                    float4* records, int32_t* shadow_list, int32_t* hit_list, int32_t* shadow_count,
-                                   int grid, cudaStream_t st, cudaEvent_t* marks, int form) {
+                                   int grid, int64_t max_rays, cudaStream_t st, cudaEvent_t* marks, int form) {
     // shadow_count (zeroed by the caller): [0] shadow rays, [1] front hits,
-    // [2..3] and [4..5] the 64-bit work counters of the two persistent passes
-    unsigned long long* next = reinterpret_cast<unsigned long long*>(shadow_count + 2);
-    unsigned long long* next_shadow = reinterpret_cast<unsigned long long*>(shadow_count + 4);
+    // [2] and [4] the work counters of the two persistent passes
+    uint32_t* next = reinterpret_cast<uint32_t*>(shadow_count + 2);
+    uint32_t* next_shadow = reinterpret_cast<uint32_t*>(shadow_count + 4);
+    const int shade_grid = bounded_grid(grid, max_rays);
+    grid = bounded_grid(std::min(grid, kTraceCtas * sm_count()), max_rays);
     cudaError_t e = cudaSuccess;
     if (marks && (e = cudaEventRecord(marks[0], st)) != cudaSuccess) return e;
     const FastDiv dR = make_fast_div((uint32_t)R);
@@ -671,7 +650,7 @@ static cudaError_t trace_wavefront(const DevScene& s, const VolSet& vs, const Li
         return e;
     if (marks && (e = cudaEventRecord(marks[2], st)) != cudaSuccess) return e;
     e = with_query_form(form, [&](auto f) {
-        return launch_pdl(k_shade<MULTI, decltype(f)::value>, grid, 256, 0, st, s, vs, L, dirs, R, dR, active, hit_list,
+        return launch_pdl(k_shade<MULTI, decltype(f)::value>, shade_grid, 256, 0, st, s, vs, L, dirs, R, dR, active, hit_list,
                           shadow_count + 1, records);
     });
     if (e != cudaSuccess) return e;
@@ -684,8 +663,9 @@ cudaError_t launch_trace_count(const DevScene& s, const VolView& v, const Lights
                                int32_t* shadow_list, int32_t* hit_list, int32_t* shadow_count,
                                unsigned long long* stats, int grid, cudaStream_t st) {
     const VolSet vs = single_set(v);
-    unsigned long long* next = reinterpret_cast<unsigned long long*>(shadow_count + 2);
-    unsigned long long* next_shadow = reinterpret_cast<unsigned long long*>(shadow_count + 4);
+    uint32_t* next = reinterpret_cast<uint32_t*>(shadow_count + 2);
+    uint32_t* next_shadow = reinterpret_cast<uint32_t*>(shadow_count + 4);
+    grid = std::min(grid, kTraceCtas * sm_count());
     cudaError_t e = cudaMemsetAsync(shadow_count, 0, 6 * sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     const FastDiv dR = make_fast_div((uint32_t)R);
@@ -700,18 +680,18 @@ cudaError_t launch_trace_count(const DevScene& s, const VolView& v, const Lights
 cudaError_t launch_trace_wavefront(const DevScene& s, const VolView& v, const Lights& L, const float4* dirs,
                                    int R, const int32_t* perm, const int32_t* active, const int32_t* count,
                                    float4* records, int32_t* shadow_list, int32_t* hit_list, int32_t* shadow_count,
-                                   int grid, cudaStream_t st, cudaEvent_t* marks) {
+                                   int grid, int64_t max_rays, cudaStream_t st, cudaEvent_t* marks) {
     return trace_wavefront<false>(s, single_set(v), L, dirs, R, perm, active, count, records, shadow_list, hit_list,
-                                  shadow_count, grid, st, marks, query_form(v));
+                                  shadow_count, grid, max_rays, st, marks, query_form(v));
 }
 
 cudaError_t launch_trace_wavefront_multi(const DevScene& s, const VolSet& vs, const Lights& L,
                                          const float4* dirs, int R, const int32_t* perm, const int32_t* active,
                                          const int32_t* count, float4* records, int32_t* shadow_list,
-                                         int32_t* hit_list, int32_t* shadow_count, int grid, cudaStream_t st,
-                                         int form) {
+                                         int32_t* hit_list, int32_t* shadow_count, int grid, int64_t max_rays,
+                                         cudaStream_t st, int form) {
     return trace_wavefront<true>(s, vs, L, dirs, R, perm, active, count, records, shadow_list, hit_list,
-                                 shadow_count, grid, st, nullptr, form);
+                                 shadow_count, grid, max_rays, st, nullptr, form);
 }
 
 cudaError_t launch_trace_rays(const DevScene& s, const float* orig, const float* dir, int64_t n,
