@@ -160,6 +160,7 @@ struct ddgi_volume_s {
     int3 shift{0, 0, 0};
     float4* offsets = nullptr;             // [P] probe offsets (position optimizer)
     float4* opt_dirs = nullptr;            // [3R] rays (and their constants) of an optimizer iteration
+    OptimizeScratch* opt_scratch = nullptr;   // [P] an iteration's reductions (zeroed between uses)
     bool uninit_possible = true;           // some probe may still be UNINIT
     float* dyn_boxes = nullptr;            // [DDGI_MAX_DYNAMIC_BOXES][6] extended boxes (device)
     int32_t n_dyn = 0;
@@ -499,7 +500,7 @@ void ddgi_volume_destroy(ddgi_volume v) {
     for (void* p : v->snap_dist) cudaFree(p);
     cudaFree(v->g_irr); cudaFree(v->g_prev);
     cudaFree(v->pack_w); cudaFree(v->inv_irr_r); cudaFree(v->inv_dist_r);
-    cudaFree(v->offsets); cudaFree(v->opt_dirs); cudaFree(v->dyn_boxes);
+    cudaFree(v->offsets); cudaFree(v->opt_dirs); cudaFree(v->opt_scratch); cudaFree(v->dyn_boxes);
     for (double* q : v->snap64_irr) cudaFree(q);
     for (double* q : v->snap64_dist) cudaFree(q);
     cudaFree(v->rec64); cudaFree(v->g64); cudaFree(v->g64_prev); cudaFree(v->gL64); cudaFree(v->sw64);
@@ -557,6 +558,8 @@ ddgi_status ddgi_volume_create(const ddgi_volume_desc* desc, ddgi_volume* out) {
     A((void**)&v->offsets, sizeof(float4) * (size_t)v->P);
     if (desc->optimizer_iters > 0) {
         A((void**)&v->opt_dirs, sizeof(float4) * 3 * v->R);
+        A((void**)&v->opt_scratch, sizeof(OptimizeScratch) * (size_t)v->P);
+        if (e == cudaSuccess) e = cudaMemset(v->opt_scratch, 0, sizeof(OptimizeScratch) * (size_t)v->P);
     }
     if (desc->converge_batches > 0) {
         const size_t ti = (size_t)desc->irr_n * desc->irr_n, td = (size_t)desc->dist_n * desc->dist_n;
@@ -741,11 +744,12 @@ static ddgi_status update_impl(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
         for (int k = 0; k < d.optimizer_iters; ++k) {
             // iteration k traces the rays of frame + k, as if spread over frames
             DDGI_CK(launch_frame_dirs(frame_rotation(d.seed, params->frame + k), v->R, d.irr_n, d.dist_n, v->sf64,
-                                      v->opt_dirs, st));
-            DDGI_CK(launch_optimize(s->dev, view, v->opt_dirs, v->R, v->lists, v->counts + 0, sms * 8, st));
+                                      v->opt_dirs, v->counts + 3, 1, st));
+            DDGI_CK(launch_optimize(s->dev, view, v->opt_dirs, v->R, v->perm, v->lists, v->counts + 0, v->opt_scratch,
+                                    reinterpret_cast<uint32_t*>(v->counts + 3), st));
         }
         DDGI_CK(launch_classify(s->dev, view, v->dirs, v->R, v->perm, v->lists, v->counts + 0, v->class_scratch,
-                                sms * 8, st));
+                                reinterpret_cast<uint32_t*>(v->counts + 9), sms * 8, st));
         if (begin == 0 && end == v->P) v->uninit_possible = false;
     }
     // dynamic objects wake sleeping probes (and awake probes fall asleep
@@ -1222,7 +1226,7 @@ ddgi_status cascade_enqueue(ddgi_cascade_s* c, const DevScene& sc, const Lights&
                                     c->inv_irr_r, c->inv_dist_r, st));
     DDGI_CK(launch_build_list_multi(vs, (int)c->total, 0, c->lists, c->counts + 0, st));
     DDGI_CK(launch_classify_multi(sc, vs, c->dirs, c->R, c->perm, c->lists, c->counts + 0, c->class_scratch,
-                                  sms * 8, st));
+                                  reinterpret_cast<uint32_t*>(c->counts + 9), st));
     DDGI_CK(launch_build_list_multi(vs, (int)c->total, 1, c->lists + c->total, c->counts + 1, st));
     DDGI_CK(launch_trace_wavefront_multi(sc, vs, L, c->dirs, c->R, c->perm, c->lists + c->total, c->counts + 1,
                                          c->records, c->shadow_list, c->hit_list, c->shadow_count, sms * c->trace_mult,
@@ -1776,7 +1780,7 @@ ddgi_status ddgi_diff_forward_f64(ddgi_volume v, ddgi_scene s, const ddgi_lights
     DDGI_CK(cudaMemsetAsync(v->snap64_dist[0], 0, dist64_bytes(v), st));
     for (int f = 0; f < n_frames; ++f) {
         DDGI_CK(launch_frame_dirs(frame_rotation(d.seed, first_frame + f), v->R, d.irr_n, d.dist_n, v->sf64, v->dirs,
-                                  st));
+                                  nullptr, 0, st));
         // a texel no ray reaches keeps its value: start from the previous atlas
         DDGI_CK(cudaMemcpyAsync(v->snap64_irr[f + 1], v->snap64_irr[f], irr64_bytes(v), cudaMemcpyDeviceToDevice, st));
         DDGI_CK(cudaMemcpyAsync(v->snap64_dist[f + 1], v->snap64_dist[f], dist64_bytes(v), cudaMemcpyDeviceToDevice,
@@ -1824,7 +1828,7 @@ ddgi_status ddgi_diff_backward_f64(ddgi_volume v, ddgi_scene s, const ddgi_light
     double* gp = v->g64_prev;
     for (int f = n_frames - 1; f >= 0; --f) {
         DDGI_CK(launch_frame_dirs(frame_rotation(d.seed, first_frame + f), v->R, d.irr_n, d.dist_n, v->sf64, v->dirs,
-                                  st));
+                                  nullptr, 0, st));
         DDGI_CK(cudaMemsetAsync(gp, 0, irr64_bytes(v), st));
         DDGI_CK(launch_diff64_frame_adjoint(dv, s->dev, L, v->dirs, albedo_dev, v->snap64_irr[f], v->snap64_dist[f],
                                             v->snap64_irr[f + 1], f > 0, v->sw64, g, v->gL64, d_emit_dev,

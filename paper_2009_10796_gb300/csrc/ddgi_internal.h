@@ -268,27 +268,38 @@ cudaError_t launch_build_list_multi(const VolSet& vs, int total, int which, int3
                                     cudaStream_t st);
 // perm (may be NULL = identity): ray order of a probe's warps, a permutation
 // of [0, R) that groups nearby directions (ray_order_morton)
-// One position-optimizer iteration (Sec. 5) over the UNINIT list, rays `dirs`.
-cudaError_t launch_optimize(const DevScene& s, const VolView& v, const float4* dirs, int R, const int32_t* list,
-                            const int32_t* count, int grid, cudaStream_t st);
+// One position-optimizer iteration (Sec. 5) over the UNINIT list, rays `dirs`
+// taken in the order perm.  scratch: one zeroed entry per list entry, left
+// zeroed; next: a zeroed work counter.
+struct OptimizeScratch {
+    unsigned long long near_back, near_front, far_front;
+    int32_t back, done;
+};
+cudaError_t launch_optimize(const DevScene& s, const VolView& v, const float4* dirs, int R, const int32_t* perm,
+                            const int32_t* list, const int32_t* count, OptimizeScratch* scratch, uint32_t* next,
+                            cudaStream_t st);
 // Frame ray directions only (float4 for the trace, double for the weights).
 // The frame directions and ray constants alone (position-optimizer rays).
 cudaError_t launch_frame_dirs(const FrameRot& rot, int R, int irr_n, int dist_n, const double* sf64, float4* dirs,
-                              cudaStream_t st);
+                              int32_t* zero, int n_zero, cudaStream_t st);
 // Classification of the listed (uninitialised) probes.  scratch: one zeroed
-// int4 per list entry, left zeroed (batch-split kernel), or nullptr (one
-// warp per probe, no scratch: the allocation-free update).
+// int4 per list entry, left zeroed, and next a zeroed work counter
+// (batch-split kernel), or nullptr (one warp per probe on `grid` blocks: the
+// allocation-free update).
 cudaError_t launch_classify(const DevScene& s, const VolView& v, const float4* dirs, int R, const int32_t* perm,
-                            const int32_t* list, const int32_t* count, int4* scratch, int grid, cudaStream_t st);
+                            const int32_t* list, const int32_t* count, int4* scratch, uint32_t* next, int grid,
+                            cudaStream_t st);
 cudaError_t launch_classify_multi(const DevScene& s, const VolSet& vs, const float4* dirs, int R,
                                   const int32_t* perm, const int32_t* list, const int32_t* count, int4* scratch,
-                                  int grid, cudaStream_t st);
+                                  uint32_t* next, cudaStream_t st);
 cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights& L,
                                const float4* dirs, int R, const int32_t* active,
                                const int32_t* count, float4* records, int grid, cudaStream_t st);
 // Per-volume device counters, one block cleared by one memset per frame:
-// [0] uninitialised-list count, [1] active-list count, [4..9] the trace's
-// counters (shadow_count below).
+// [0] uninitialised-list count, [1] active-list count, [2] new-probe count,
+// [3] the optimizer's work counter (zeroed by each of its direction
+// launches), [4..8] the trace's counters (shadow_count below), [9] the
+// classification's work counter.
 constexpr int kCounterInts = 10;
 
 // Wavefront trace: persistent primary pass (closest hits; final records of

@@ -691,10 +691,10 @@ cudaError_t launch_converge_finish(const VolView& v, const int32_t* list, const 
 }
 
 cudaError_t launch_frame_dirs(const FrameRot& rot, int R, int irr_n, int dist_n, const double* sf64, float4* dirs,
-                              cudaStream_t st) {
+                              int32_t* zero, int n_zero, cudaStream_t st) {
     // the direction blocks of k_frame_setup alone
     k_frame_setup<false><<<(R + 255) / 256, 256, 0, st>>>(rot, nullptr, R, irr_n, dist_n, 0.0, sf64, dirs, nullptr,
-                                                           nullptr, nullptr, nullptr, nullptr, 0,
+                                                           nullptr, nullptr, nullptr, zero, n_zero,
                                                            irr_n * irr_n + dist_n * dist_n);
     return cudaGetLastError();
 }

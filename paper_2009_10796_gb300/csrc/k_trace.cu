@@ -70,6 +70,25 @@ __global__ void __launch_bounds__(256) k_classify(DevScene s, VolSet vs, const f
     }
 }
 
+// Persistent passes: a warp walks its lanes' rays in while-while rounds and,
+// once every lane has finished, takes the next 32 work items (Aila and Laine
+// 2009, persistent threads; refilling at 4, 8 or 16 idle lanes measured
+// slower on the city workload, in lost ray coherence).  The first batch is
+// the warp's own index and only later ones come from the global counter,
+// which starts after them: with few rays, thousands of warps would
+// otherwise queue on one word to learn that nothing is left.  Work items are
+// below 2^31 (probes x rays is), a batch past the end below 2^32.
+__device__ __forceinline__ unsigned first_batch() { return (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; }
+__device__ __forceinline__ unsigned next_batch(uint32_t* next) {
+    unsigned base = 0;
+    if ((threadIdx.x & 31) == 0) base = gridDim.x * blockDim.x + atomicAdd(next, 32u);
+    return __shfl_sync(0xffffffffu, base, 0);
+}
+
+// CTAs per SM that classification and the optimizer are built for (64
+// registers a thread: their reductions spill at 48).
+constexpr int kClassCtas = 4;
+
 // Classification in 32-ray batches: one work item per (list entry, batch),
 // so the R rays of the few probes a frame classifies (the planes a tracking
 // window scrolls in) spread over all warps instead of R / 32 sequential
@@ -81,20 +100,21 @@ __global__ void __launch_bounds__(256) k_classify(DevScene s, VolSet vs, const f
 // minima do not depend on the order the batches run in, so the states are
 // k_classify's.  scratch: one zeroed int4 per list entry.
 template <bool MULTI>
-__global__ void __launch_bounds__(256) k_classify_split(DevScene s, VolSet vs, const float4* __restrict__ dirs,
-                                                        int R, const int32_t* __restrict__ perm,
-                                                        const int32_t* __restrict__ list,
-                                                        const int32_t* __restrict__ count, int4* scratch) {
+__global__ void __launch_bounds__(256, kClassCtas) k_classify_split(DevScene s, VolSet vs,
+                                                                    const float4* __restrict__ dirs, int R,
+                                                                    const int32_t* __restrict__ perm,
+                                                                    const int32_t* __restrict__ list,
+                                                                    const int32_t* __restrict__ count, int4* scratch,
+                                                                    uint32_t* next) {
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int nb = (R + 31) / 32;
-    const int64_t items = (int64_t)(*count) * nb;
+    const unsigned nb = (unsigned)(R + 31) / 32;
+    const unsigned total = (unsigned)(*count) * nb * 32u;   // below 2^32: probes x R is below 2^31, probes 2^26
     int2 stack[kStackSize4];
     WwLane<kStackSize4, int2> w;
     w.stack = stack;
-    for (int64_t it = warp; it < items; it += nwarps) {
-        const int q = (int)(it / nb), b = (int)(it - (int64_t)q * nb);
+    for (unsigned at = first_batch(); at < total; at = next_batch(next)) {
+        const unsigned it = at >> 5;
+        const int q = (int)(it / nb), b = (int)(it - (unsigned)q * nb);
         const int e = list[q];
         const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
         const int p = e & kEntryMask;
@@ -126,7 +146,7 @@ __global__ void __launch_bounds__(256) k_classify_split(DevScene s, VolSet vs, c
             if (bf) atomicAdd(&sc->x, bf);
             atomicMax(&sc->y, 0x7f800000 - __float_as_int(dmin));
             __threadfence();   // this batch's sums before its done count
-            if (atomicAdd(&sc->z, 1) == nb - 1) {
+            if (atomicAdd(&sc->z, 1) == (int)nb - 1) {
                 __threadfence();
                 const int bft = atomicAdd(&sc->x, 0);
                 const float dm = __int_as_float(0x7f800000 - atomicAdd(&sc->y, 0));
@@ -246,22 +266,6 @@ __device__ __forceinline__ void hit_frame(const DevScene& s, int k, float3& ng) 
     const float4* T = s.tris + 3 * (int64_t)k;
     float4 p0 = __ldg(T), p1 = __ldg(T + 1), p2 = __ldg(T + 2);
     ng = cross(f3(p1.x - p0.x, p1.y - p0.y, p1.z - p0.z), f3(p2.x - p0.x, p2.y - p0.y, p2.z - p0.z));
-}
-
-// Persistent passes: a warp walks its lanes' rays in while-while rounds and,
-// once every lane has finished, takes the next 32 work items (Aila and Laine
-// 2009, persistent threads; refilling at 4, 8 or 16 idle lanes measured
-// slower on the city workload, in lost ray coherence).  The first batch is
-// the warp's own index and only later ones come from the global counter,
-// which starts after them: with few rays, thousands of warps would
-// otherwise queue on one word to learn that nothing is left.  Work items are
-// below 2^31 (probes x rays is), a batch past the end below 2^32.
-constexpr unsigned kNoBatch = 0xffffffffu;
-__device__ __forceinline__ unsigned first_batch() { return (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; }
-__device__ __forceinline__ unsigned next_batch(uint32_t* next) {
-    unsigned base = 0;
-    if ((threadIdx.x & 31) == 0) base = gridDim.x * blockDim.x + atomicAdd(next, 32u);
-    return __shfl_sync(0xffffffffu, base, 0);
 }
 
 // CTAs per SM that both passes are built for (48 registers a thread).
@@ -521,75 +525,80 @@ __global__ void __launch_bounds__(256, kTraceCtas) k_gbuffer(DevScene s, float3 
     }
 }
 
-// One iteration of the probe position optimizer (Sec. 5 and its listing),
-// one warp per UNINIT probe: the lanes trace the iteration's rays from the
-// probe's current position and reduce, as (t bits << 32 | ray) keys, the
-// closest backface, the closest front face and the farthest front face
-// (ties: smaller ray index for closest, larger for farthest); lane 0 moves
-// the offset:
+// One iteration of the probe position optimizer (Sec. 5 and its listing):
+// the iteration's rays from the probe's current position reduced, as
+// (t bits << 32 | ray) keys, to the closest backface, the closest front face
+// and the farthest front face (ties: smaller ray index for closest, larger
+// for farthest); then the offset moves:
 //   more than 25% backfaces: along t * w of the closest backface, by the
 //     largest scale keeping every component within +-limit (less 1 mm),
 //     only when that scale exceeds 1 (the move goes through the backface);
 //   otherwise, unless the farthest front face lies within 60 degrees of the
 //     closest: min(0.2, t) along the farthest front face, clamped to +-limit.
-__global__ void __launch_bounds__(256) k_optimize(DevScene s, VolView v, const float4* __restrict__ dirs, int R,
-                                                  const int32_t* __restrict__ list,
-                                                  const int32_t* __restrict__ count) {
+// As in k_classify_split, a work item is a batch of 32 rays in the order
+// `perm` (a compact cone), a batch joins the entry's scratch (zeroed; the
+// closest keys as maxima of their complements) and counts itself done, and
+// the warp that completes an entry moves the probe and zeroes the scratch.
+// Counts, minima and maxima do not depend on the order of the batches.  With
+// a warp to a probe, its batches one after another over all directions, an
+// iteration of 6912 probes x 128 rays took 106-138 us against 91-122 us here
+// (and the classification's trace 123 us against 108 us with batches from
+// a counter on one resident wave).
+__global__ void __launch_bounds__(256, kClassCtas) k_optimize(DevScene s, VolView v, const float4* __restrict__ dirs,
+                                                              int R, const int32_t* __restrict__ perm,
+                                                              const int32_t* __restrict__ list,
+                                                              const int32_t* __restrict__ count,
+                                                              OptimizeScratch* scratch, uint32_t* next) {
     const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int n = *count;
-    const DevScene& sc = s;
+    const unsigned nb = (unsigned)(R + 31) / 32;
+    const unsigned total = (unsigned)(*count) * nb * 32u;   // below 2^32, as in k_classify_split
     int2 stack[kStackSize4];
-    WwLane<kStackSize4, int2> w;
-    w.stack = stack;
-    for (int q = warp; q < n; q += nwarps) {
-        const int p = list[q];
-        const float3 o = probe_pos_phys(v, p);
-        int bf = 0;
+    for (unsigned at = first_batch(); at < total; at = next_batch(next)) {
+        const unsigned it = at >> 5;
+        const int q = (int)(it / nb), j = 32 * (int)(it - (unsigned)q * nb) + lane;
+        const bool valid = j < R;
+        const int i = valid ? __ldg(perm + j) : 0;
+        const float4 d4 = __ldg(dirs + i);
+        const float3 d = f3(d4.x, d4.y, d4.z);
+        // coherent loads: the offsets are written by other launches' warps only
+        const Hit h = closest_hit_warp(s, ray_pre_packed(probe_pos_phys(v, list[q]), d, __ldg(dirs + R + 2 * i),
+                                                         __ldg(dirs + R + 2 * i + 1)), stack, valid);
+        bool back = false;
         unsigned long long cb = ~0ull, cf = ~0ull, ff = 0ull;
-        // 32 rays at a time through the warp-cooperative 4-wide walk (lanes
-        // past R take part without a ray)
-        for (int i0 = 0; i0 < R; i0 += 32) {
-            const int i = i0 + lane;
-            const bool valid = i < R;
-            const int ii = valid ? i : 0;
-            const float4 d4 = __ldg(dirs + ii);
-            const float3 d = f3(d4.x, d4.y, d4.z);
-            const RayPre r = ray_pre_packed(o, d, __ldg(dirs + R + 2 * ii), __ldg(dirs + R + 2 * ii + 1));
-            ww_start(sc, w, valid);
-            do {
-                ww4_round<false>(sc, r, w);
-            } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
-            const Hit h = w.h;
-            if (!valid || h.orig < 0) continue;
-            const float4* T = s.tris + 3 * (int64_t)h.k;
-            float4 p0 = __ldg(T), p1 = __ldg(T + 1), p2 = __ldg(T + 2);
-            float3 ng = cross(f3(p1.x - p0.x, p1.y - p0.y, p1.z - p0.z), f3(p2.x - p0.x, p2.y - p0.y, p2.z - p0.z));
+        if (valid && h.orig >= 0) {
+            float3 ng;
+            hit_frame(s, h.k, ng);
             const unsigned long long key = ((unsigned long long)__float_as_uint(h.t) << 32) | (unsigned)i;
-            if (dot(d, ng) > 0.0f) {
-                bf++;
-                cb = key < cb ? key : cb;
-            } else {
-                cf = key < cf ? key : cf;
-                ff = key > ff ? key : ff;
-            }
+            back = dot(d, ng) > 0.0f;
+            if (back) cb = key;
+            else cf = ff = key;
         }
+        const int bf = __popc(__ballot_sync(0xffffffffu, back));
         for (int off = 16; off > 0; off >>= 1) {
-            bf += __shfl_xor_sync(0xffffffffu, bf, off);
-            const unsigned long long a = __shfl_xor_sync(0xffffffffu, cb, off);
-            const unsigned long long b = __shfl_xor_sync(0xffffffffu, cf, off);
-            const unsigned long long c = __shfl_xor_sync(0xffffffffu, ff, off);
-            cb = a < cb ? a : cb;
-            cf = b < cf ? b : cf;
-            ff = c > ff ? c : ff;
+            cb = min(cb, __shfl_xor_sync(0xffffffffu, cb, off));
+            cf = min(cf, __shfl_xor_sync(0xffffffffu, cf, off));
+            ff = max(ff, __shfl_xor_sync(0xffffffffu, ff, off));
         }
         if (lane != 0) continue;
+        OptimizeScratch* sc = scratch + q;
+        if (bf) atomicAdd(&sc->back, bf);
+        if (cb != ~0ull) atomicMax(&sc->near_back, ~cb);
+        if (cf != ~0ull) atomicMax(&sc->near_front, ~cf);
+        if (ff != 0ull) atomicMax(&sc->far_front, ff);
+        __threadfence();   // this batch's part before its done count
+        if (atomicAdd(&sc->done, 1) != (int)nb - 1) continue;
+        __threadfence();
+        const int bft = atomicAdd(&sc->back, 0);
+        cb = ~atomicMax(&sc->near_back, 0ull);
+        cf = ~atomicMax(&sc->near_front, 0ull);
+        ff = atomicMax(&sc->far_front, 0ull);
+        *sc = OptimizeScratch{};   // no other batch of this entry is left
+        const int p = list[q];
         const float4 c4 = v.offsets[p];
         float3 cur = f3(c4.x, c4.y, c4.z);
         const float3 lim = f3(v.offset_limit * v.spacing.x, v.offset_limit * v.spacing.y,
                               v.offset_limit * v.spacing.z);
-        if (4 * bf > R) {
+        if (4 * bft > R) {
             const float4 w = __ldg(dirs + (int)(cb & 0xffffffffu));
             const float tb = __uint_as_float((unsigned)(cb >> 32));
             const float3 vec = f3(tb * w.x, tb * w.y, tb * w.z);
@@ -612,16 +621,28 @@ __global__ void __launch_bounds__(256) k_optimize(DevScene s, VolView v, const f
     }
 }
 
-cudaError_t launch_optimize(const DevScene& s, const VolView& v, const float4* dirs, int R, const int32_t* list,
-                            const int32_t* count, int grid, cudaStream_t st) {
-    k_optimize<<<grid, 256, 0, st>>>(s, v, dirs, R, list, count);
+// Blocks of 256 threads for at most max_items of them, no more than `grid`
+// nor, for the persistent passes, than are resident at once (a block of a
+// later wave would start its own first batch when the others are done).
+static int bounded_grid(int grid, int64_t max_items) {
+    const int64_t need = (max_items + 255) / 256;
+    return need < grid ? (need > 0 ? (int)need : 1) : grid;
+}
+
+cudaError_t launch_optimize(const DevScene& s, const VolView& v, const float4* dirs, int R, const int32_t* perm,
+                            const int32_t* list, const int32_t* count, OptimizeScratch* scratch, uint32_t* next,
+                            cudaStream_t st) {
+    const int grid = bounded_grid(kClassCtas * sm_count(), (int64_t)v.n_probes * ((R + 31) / 32) * 32);
+    k_optimize<<<grid, 256, 0, st>>>(s, v, dirs, R, perm, list, count, scratch, next);
     return cudaGetLastError();
 }
 
 cudaError_t launch_classify(const DevScene& s, const VolView& v, const float4* dirs, int R, const int32_t* perm,
-                            const int32_t* list, const int32_t* count, int4* scratch, int grid, cudaStream_t st) {
+                            const int32_t* list, const int32_t* count, int4* scratch, uint32_t* next, int grid,
+                            cudaStream_t st) {
     if (scratch)
-        k_classify_split<false><<<grid, 256, 0, st>>>(s, single_set(v), dirs, R, perm, list, count, scratch);
+        k_classify_split<false><<<bounded_grid(kClassCtas * sm_count(), (int64_t)v.n_probes * ((R + 31) / 32) * 32), 256,
+                                  0, st>>>(s, single_set(v), dirs, R, perm, list, count, scratch, next);
     else
         k_classify<false><<<grid, 256, 0, st>>>(s, single_set(v), dirs, R, perm, list, count);
     return cudaGetLastError();
@@ -629,11 +650,8 @@ cudaError_t launch_classify(const DevScene& s, const VolView& v, const float4* d
 
 cudaError_t launch_classify_multi(const DevScene& s, const VolSet& vs, const float4* dirs, int R,
                                   const int32_t* perm, const int32_t* list, const int32_t* count, int4* scratch,
-                                  int grid, cudaStream_t st) {
-    if (scratch)
-        k_classify_split<true><<<grid, 256, 0, st>>>(s, vs, dirs, R, perm, list, count, scratch);
-    else
-        k_classify<true><<<grid, 256, 0, st>>>(s, vs, dirs, R, perm, list, count);
+                                  uint32_t* next, cudaStream_t st) {
+    k_classify_split<true><<<kClassCtas * sm_count(), 256, 0, st>>>(s, vs, dirs, R, perm, list, count, scratch, next);
     return cudaGetLastError();
 }
 
@@ -642,14 +660,6 @@ cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights
                                int grid, cudaStream_t st) {
     k_trace_shade<<<grid, 128, 0, st>>>(s, v, L, dirs, R, active, count, records);
     return cudaGetLastError();
-}
-
-// Blocks of 256 threads for at most max_items of them, no more than `grid`
-// nor, for the persistent passes, than are resident at once (a block of a
-// later wave would start its own first batch when the others are done).
-static int bounded_grid(int grid, int64_t max_items) {
-    const int64_t need = (max_items + 255) / 256;
-    return need < grid ? (need > 0 ? (int)need : 1) : grid;
 }
 
 template <bool MULTI>
