@@ -268,13 +268,14 @@ __device__ __forceinline__ void hit_frame(const DevScene& s, int k, float3& ng) 
     ng = cross(f3(p1.x - p0.x, p1.y - p0.y, p1.z - p0.z), f3(p2.x - p0.x, p2.y - p0.y, p2.z - p0.z));
 }
 
-// CTAs per SM that both passes are built for (48 registers a thread).
-constexpr int kTraceCtas = 5;
+// CTAs per SM that the passes are built for: four with the 64-register walk
+// for a single volume, five (48 registers) for a cascade (ww4_round).
+constexpr int trace_ctas(bool multi) { return multi ? 5 : 4; }
 
 // COUNT: measurement build that adds its 4-wide node visits and triangle
 // tests to stats[1], stats[2] (otherwise identical).
 template <bool MULTI, bool COUNT = false>
-__global__ void __launch_bounds__(256, kTraceCtas) k_trace_primary(
+__global__ void __launch_bounds__(256, trace_ctas(MULTI)) k_trace_primary(
     DevScene s, VolSet vs, Lights L, const float4* __restrict__ dirs, int R, FastDiv dR,
     const int32_t* __restrict__ perm, const int32_t* __restrict__ active, const int32_t* __restrict__ count,
     float4* __restrict__ hits, int32_t* __restrict__ shadow_list, int32_t* __restrict__ hit_list, int32_t* shadow_count,
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(256, kTraceCtas) k_trace_primary(
         const bool valid = b + lane < total;
         ww_start(s, w, valid);
         do {
-            ww4_round<false, COUNT>(s, r, w, &tc);
+            ww4_round<false, COUNT, !MULTI>(s, r, w, &tc);
         } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
         bool need = false, front = false;
         if (valid) {
@@ -362,7 +363,7 @@ __global__ void __launch_bounds__(256, kTraceCtas) k_trace_primary(
 
 // COUNT: adds 4-wide node visits and triangle tests to stats[4], stats[5].
 template <bool MULTI, bool COUNT = false>
-__global__ void __launch_bounds__(256, kTraceCtas) k_trace_shadow(
+__global__ void __launch_bounds__(256, trace_ctas(MULTI)) k_trace_shadow(
     DevScene s, VolSet vs, Lights L, const float4* __restrict__ dirs, int R, FastDiv dR,
     const int32_t* __restrict__ active, float4* __restrict__ hits, const int32_t* __restrict__ shadow_list,
     const int32_t* __restrict__ shadow_count, uint32_t* next, unsigned long long* stats) {
@@ -392,7 +393,7 @@ __global__ void __launch_bounds__(256, kTraceCtas) k_trace_shadow(
         ray_set_origin(r, x + off * nn);
         ww_start(s, w, valid);
         do {
-            ww4_round<true, COUNT>(s, r, w, &tc);
+            ww4_round<true, COUNT, !MULTI>(s, r, w, &tc);
         } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
         if (valid && w.h.orig < 0) reinterpret_cast<float*>(hits)[4 * (int64_t)rec + 2] = 1.0f;
     }
@@ -452,18 +453,19 @@ __global__ void __launch_bounds__(256, 4) k_shade(DevScene s, VolSet vs, Lights 
 
 // Closest hit of a warp's 32 rays over the 4-wide hierarchy (all lanes call;
 // valid: the lane has a ray).
+template <bool WIDE>
 __device__ __forceinline__ Hit closest_hit_warp(const DevScene& s, const RayPre& r, int2* stack, bool valid) {
     WwLane<kStackSize4, int2> w;
     w.stack = stack;
     ww_start(s, w, valid);
     do {
-        ww4_round<false>(s, r, w);
+        ww4_round<false, false, WIDE>(s, r, w);
     } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
     return w.h;
 }
 
 // Closest hits of arbitrary rays, a warp for 32 consecutive ones.
-__global__ void __launch_bounds__(256, kTraceCtas) k_trace_rays(DevScene s, const float* __restrict__ orig,
+__global__ void __launch_bounds__(256, 4) k_trace_rays(DevScene s, const float* __restrict__ orig,
                                                                 const float* __restrict__ dir, int64_t n,
                                                                 float* __restrict__ t_out,
                                                                 int32_t* __restrict__ tri_out,
@@ -474,7 +476,7 @@ __global__ void __launch_bounds__(256, kTraceCtas) k_trace_rays(DevScene s, cons
         const int64_t q = min(q0 + (threadIdx.x & 31), n - 1);
         const bool valid = q0 + (threadIdx.x & 31) < n;
         const float3 d = f3(dir[3 * q], dir[3 * q + 1], dir[3 * q + 2]);
-        const Hit h = closest_hit_warp(s, ray_pre(f3(orig[3 * q], orig[3 * q + 1], orig[3 * q + 2]), d), stack, valid);
+        const Hit h = closest_hit_warp<true>(s, ray_pre(f3(orig[3 * q], orig[3 * q + 1], orig[3 * q + 2]), d), stack, valid);
         if (!valid) continue;
         t_out[q] = h.t;
         tri_out[q] = h.orig;
@@ -493,9 +495,9 @@ __global__ void __launch_bounds__(256, kTraceCtas) k_trace_rays(DevScene s, cons
 // Camera G-buffer, a warp for a tile of 8 x 4 pixels, whose rays stay together
 // further down the hierarchy than a row of 32.  Bound by the walk's
 // instruction issue, as the probe rays are: 1920 x 1080 over 196,610 city
-// triangles take 149 us, 199 us with one ray a thread over the binary
+// triangles take 139 us, 199 us with one ray a thread over the binary
 // hierarchy.
-__global__ void __launch_bounds__(256, kTraceCtas) k_gbuffer(DevScene s, float3 cpos, float3 fwd, float3 right,
+__global__ void __launch_bounds__(256, 4) k_gbuffer(DevScene s, float3 cpos, float3 fwd, float3 right,
                                                              float3 up, float tan_half, float aspect, int w, int h,
                                                              float* __restrict__ out_pos,
                                                              float* __restrict__ out_nrm) {
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(256, kTraceCtas) k_gbuffer(DevScene s, float3 
         float sy = (1.0f - (y + 0.5f) / h * 2.0f) * tan_half;
         float3 d = fwd + sx * right + sy * up;
         d = (1.0f / length(d)) * d;
-        const Hit hh = closest_hit_warp(s, ray_pre(cpos, d), stack, valid);
+        const Hit hh = closest_hit_warp<true>(s, ray_pre(cpos, d), stack, valid);
         if (!valid) continue;
         float3 p = f3(0.0f, 0.0f, 0.0f), nn = f3(0.0f, 0.0f, 0.0f);
         if (hh.orig >= 0) {
@@ -561,7 +563,7 @@ __global__ void __launch_bounds__(256, kClassCtas) k_optimize(DevScene s, VolVie
         const float4 d4 = __ldg(dirs + i);
         const float3 d = f3(d4.x, d4.y, d4.z);
         // coherent loads: the offsets are written by other launches' warps only
-        const Hit h = closest_hit_warp(s, ray_pre_packed(probe_pos_phys(v, list[q]), d, __ldg(dirs + R + 2 * i),
+        const Hit h = closest_hit_warp<false>(s, ray_pre_packed(probe_pos_phys(v, list[q]), d, __ldg(dirs + R + 2 * i),
                                                          __ldg(dirs + R + 2 * i + 1)), stack, valid);
         bool back = false;
         unsigned long long cb = ~0ull, cf = ~0ull, ff = 0ull;
@@ -672,7 +674,7 @@ static cudaError_t trace_wavefront(const DevScene& s, const VolSet& vs, const Li
     uint32_t* next = reinterpret_cast<uint32_t*>(shadow_count + 2);
     uint32_t* next_shadow = reinterpret_cast<uint32_t*>(shadow_count + 4);
     const int shade_grid = bounded_grid(grid, max_rays);
-    grid = bounded_grid(std::min(grid, kTraceCtas * sm_count()), max_rays);
+    grid = bounded_grid(std::min(grid, trace_ctas(MULTI) * sm_count()), max_rays);
     cudaError_t e = cudaSuccess;
     if (marks && (e = cudaEventRecord(marks[0], st)) != cudaSuccess) return e;
     const FastDiv dR = make_fast_div((uint32_t)R);
@@ -700,7 +702,7 @@ cudaError_t launch_trace_count(const DevScene& s, const VolView& v, const Lights
     const VolSet vs = single_set(v);
     uint32_t* next = reinterpret_cast<uint32_t*>(shadow_count + 2);
     uint32_t* next_shadow = reinterpret_cast<uint32_t*>(shadow_count + 4);
-    grid = std::min(grid, kTraceCtas * sm_count());
+    grid = std::min(grid, trace_ctas(false) * sm_count());
     cudaError_t e = cudaMemsetAsync(shadow_count, 0, 6 * sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     const FastDiv dR = make_fast_div((uint32_t)R);

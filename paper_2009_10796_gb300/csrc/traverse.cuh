@@ -156,26 +156,66 @@ __device__ __forceinline__ float box_enter_oct(const RayPre& r, float nx, float 
 // box_enter_oct for the four children of a 4-wide node at once: the slab
 // distances of children (0, 1) and (2, 3) in packed pairs, the same IEEE
 // operations lane by lane, so each k_c equals box_enter_oct's result.
-__device__ __forceinline__ void box4_enter_oct(const RayPre& r, float4 nx, float4 fx, float4 ny, float4 fy, float4 nz,
+//
+// FUSED evaluates each plane's distance as p r + c in one multiply-add, r the
+// reciprocal direction and c = -o r moved outward by 1.8e-7 |o r| (SlabRay).
+// c carries a rounding error of at most 2^-24 |o r| and moving it another one,
+// less together than the move, so no near distance is above and no far one
+// below the exact (p - o) r by more than the fused operation's own rounding,
+// which the widened exit distance covers with the reciprocal's: the test
+// stays conservative and the closest hit the same.
+struct SlabRay {
+    float3 cn, cf;   // near and far planes' c
+};
+
+__device__ __forceinline__ SlabRay slab_ray(const RayPre& r) {
+    SlabRay q;
+    const float3 p = f3(__fmul_rn(-r.o.x, r.idir.x), __fmul_rn(-r.o.y, r.idir.y), __fmul_rn(-r.o.z, r.idir.z));
+    const float k = 1.8e-7f;   // above 1.5 2^-23
+    q.cn = f3(fmaf(-k, fabsf(p.x), p.x), fmaf(-k, fabsf(p.y), p.y), fmaf(-k, fabsf(p.z), p.z));
+    q.cf = f3(fmaf(k, fabsf(p.x), p.x), fmaf(k, fabsf(p.y), p.y), fmaf(k, fabsf(p.z), p.z));
+    return q;
+}
+
+template <bool FUSED>
+__device__ __forceinline__ void box4_enter_oct(const RayPre& r, const SlabRay& q, float4 nx, float4 fx, float4 ny, float4 fy, float4 nz,
                                                float4 fz, float tmax, float& k0, float& k1, float& k2, float& k3) {
     float tnx[4], tfx[4], tny[4], tfy[4], tnz[4], tfz[4];
-    // the doubled operands are built per visit: holding them across the walk
-    // cost more in registers (spills) than the moves cost here
-    const uint64_t o2x = f2_pack(r.o.x, r.o.x), o2y = f2_pack(r.o.y, r.o.y), o2z = f2_pack(r.o.z, r.o.z);
-    const uint64_t i2x = f2_pack(r.idir.x, r.idir.x), i2y = f2_pack(r.idir.y, r.idir.y),
-                   i2z = f2_pack(r.idir.z, r.idir.z);
-    f2_unpack(f2_mul(f2_sub(f2_pack(nx.x, nx.y), o2x), i2x), tnx[0], tnx[1]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(nx.z, nx.w), o2x), i2x), tnx[2], tnx[3]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(fx.x, fx.y), o2x), i2x), tfx[0], tfx[1]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(fx.z, fx.w), o2x), i2x), tfx[2], tfx[3]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(ny.x, ny.y), o2y), i2y), tny[0], tny[1]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(ny.z, ny.w), o2y), i2y), tny[2], tny[3]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(fy.x, fy.y), o2y), i2y), tfy[0], tfy[1]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(fy.z, fy.w), o2y), i2y), tfy[2], tfy[3]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(nz.x, nz.y), o2z), i2z), tnz[0], tnz[1]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(nz.z, nz.w), o2z), i2z), tnz[2], tnz[3]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(fz.x, fz.y), o2z), i2z), tfz[0], tfz[1]);
-    f2_unpack(f2_mul(f2_sub(f2_pack(fz.z, fz.w), o2z), i2z), tfz[2], tfz[3]);
+    if constexpr (FUSED) {
+        const uint64_t i2x = f2_pack(r.idir.x, r.idir.x), i2y = f2_pack(r.idir.y, r.idir.y), i2z = f2_pack(r.idir.z, r.idir.z);
+        const uint64_t cnx = f2_pack(q.cn.x, q.cn.x), cny = f2_pack(q.cn.y, q.cn.y), cnz = f2_pack(q.cn.z, q.cn.z);
+        const uint64_t cfx = f2_pack(q.cf.x, q.cf.x), cfy = f2_pack(q.cf.y, q.cf.y), cfz = f2_pack(q.cf.z, q.cf.z);
+        f2_unpack(f2_fma(f2_pack(nx.x, nx.y), i2x, cnx), tnx[0], tnx[1]);
+        f2_unpack(f2_fma(f2_pack(nx.z, nx.w), i2x, cnx), tnx[2], tnx[3]);
+        f2_unpack(f2_fma(f2_pack(fx.x, fx.y), i2x, cfx), tfx[0], tfx[1]);
+        f2_unpack(f2_fma(f2_pack(fx.z, fx.w), i2x, cfx), tfx[2], tfx[3]);
+        f2_unpack(f2_fma(f2_pack(ny.x, ny.y), i2y, cny), tny[0], tny[1]);
+        f2_unpack(f2_fma(f2_pack(ny.z, ny.w), i2y, cny), tny[2], tny[3]);
+        f2_unpack(f2_fma(f2_pack(fy.x, fy.y), i2y, cfy), tfy[0], tfy[1]);
+        f2_unpack(f2_fma(f2_pack(fy.z, fy.w), i2y, cfy), tfy[2], tfy[3]);
+        f2_unpack(f2_fma(f2_pack(nz.x, nz.y), i2z, cnz), tnz[0], tnz[1]);
+        f2_unpack(f2_fma(f2_pack(nz.z, nz.w), i2z, cnz), tnz[2], tnz[3]);
+        f2_unpack(f2_fma(f2_pack(fz.x, fz.y), i2z, cfz), tfz[0], tfz[1]);
+        f2_unpack(f2_fma(f2_pack(fz.z, fz.w), i2z, cfz), tfz[2], tfz[3]);
+    } else {
+        // the doubled operands are built per visit: holding them across the walk
+        // cost more in registers (spills) than the moves cost here
+        const uint64_t o2x = f2_pack(r.o.x, r.o.x), o2y = f2_pack(r.o.y, r.o.y), o2z = f2_pack(r.o.z, r.o.z);
+        const uint64_t i2x = f2_pack(r.idir.x, r.idir.x), i2y = f2_pack(r.idir.y, r.idir.y),
+                       i2z = f2_pack(r.idir.z, r.idir.z);
+        f2_unpack(f2_mul(f2_sub(f2_pack(nx.x, nx.y), o2x), i2x), tnx[0], tnx[1]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(nx.z, nx.w), o2x), i2x), tnx[2], tnx[3]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(fx.x, fx.y), o2x), i2x), tfx[0], tfx[1]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(fx.z, fx.w), o2x), i2x), tfx[2], tfx[3]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(ny.x, ny.y), o2y), i2y), tny[0], tny[1]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(ny.z, ny.w), o2y), i2y), tny[2], tny[3]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(fy.x, fy.y), o2y), i2y), tfy[0], tfy[1]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(fy.z, fy.w), o2y), i2y), tfy[2], tfy[3]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(nz.x, nz.y), o2z), i2z), tnz[0], tnz[1]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(nz.z, nz.w), o2z), i2z), tnz[2], tnz[3]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(fz.x, fz.y), o2z), i2z), tfz[0], tfz[1]);
+        f2_unpack(f2_mul(f2_sub(f2_pack(fz.z, fz.w), o2z), i2z), tfz[2], tfz[3]);
+    }
     float tn[4], tf[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -404,9 +444,29 @@ __device__ __forceinline__ void cx(float& ka, int& va, float& kb, int& vb) {
 // farthest first (for shadow rays too: near occluders are found first, and
 // any hit ends them).  Leaves found among the children are parked or pushed
 // as leaf codes exactly as in the binary walk.
-template <bool ANY, bool COUNT = false, typename E = int>
+// WIDE is the form for kernels with 64 registers a thread: fused slab
+// distances, and a pointer per axis whose low bit 4 the ray's direction has
+// chosen, so that a near plane is one widening multiply-add away and the far
+// one differs in that bit (a node is 128-byte aligned).  At four CTAs per SM
+// it took the city's primary pass from 130.6 to 127.5 us, the G-buffer from
+// 146 to 139 us; at 48 registers and five CTAs it spills (139 us), which is
+// what the cascade passes keep: 2570 us a frame against 2590.
+template <bool ANY, bool COUNT = false, bool WIDE = false, typename E = int>
 __device__ __forceinline__ void ww4_round(const DevScene& s, const RayPre& r, WwLane<kStackSize4, E>& w,
                                           TraceCount* tc = nullptr) {
+    SlabRay q{};
+    const char *bx = nullptr, *by = nullptr, *bz = nullptr;
+    if constexpr (WIDE) {
+        q = slab_ray(r);
+        bx = reinterpret_cast<const char*>(s.nodes4) + ((r.oct & 1) << 4);
+        by = reinterpret_cast<const char*>(s.nodes4) + 32 + ((r.oct & 2) << 3);
+        bz = reinterpret_cast<const char*>(s.nodes4) + 64 + ((r.oct & 4) << 2);
+    }
+    // plane row `base` of a node; flip = 16: the axis's other row
+    auto row = [](const char* base, int node, unsigned flip) {
+        const unsigned long long a = (unsigned long long)reinterpret_cast<uintptr_t>(base) + (unsigned long long)(unsigned)node * 128ull;
+        return reinterpret_cast<const float4*>((uintptr_t)((a & 0xffffffff00000000ull) | ((unsigned)a ^ flip)));
+    };
     while (true) {
         if (w.node >= 0) {
             if (COUNT) tc->nodes++;
@@ -414,12 +474,12 @@ __device__ __forceinline__ void ww4_round(const DevScene& s, const RayPre& r, Ww
             // near / far planes per axis by the ray's octant: lo and hi swap for
             // an axis the ray runs down
             const int ax = r.oct & 1, ay = (r.oct >> 1) & 1, az = (r.oct >> 2) & 1;
-            const float4 nx = __ldg(N + ax), fx = __ldg(N + (ax ^ 1));
-            const float4 ny = __ldg(N + 2 + ay), fy = __ldg(N + 2 + (ay ^ 1));
-            const float4 nz = __ldg(N + 4 + az), fz = __ldg(N + 4 + (az ^ 1));
+            const float4 nx = __ldg(WIDE ? row(bx, w.node, 0) : N + ax), fx = __ldg(WIDE ? row(bx, w.node, 16) : N + (ax ^ 1));
+            const float4 ny = __ldg(WIDE ? row(by, w.node, 0) : N + 2 + ay), fy = __ldg(WIDE ? row(by, w.node, 16) : N + 2 + (ay ^ 1));
+            const float4 nz = __ldg(WIDE ? row(bz, w.node, 0) : N + 4 + az), fz = __ldg(WIDE ? row(bz, w.node, 16) : N + 4 + (az ^ 1));
             const int4 ref = __ldg(reinterpret_cast<const int4*>(N + 6));
             float k0, k1, k2, k3;
-            box4_enter_oct(r, nx, fx, ny, fy, nz, fz, w.h.t, k0, k1, k2, k3);
+            box4_enter_oct<WIDE>(r, q, nx, fx, ny, fy, nz, fz, w.h.t, k0, k1, k2, k3);
             int v0 = ref.x, v1 = ref.y, v2 = ref.z, v3 = ref.w;
             cx(k0, v0, k1, v1);
             cx(k2, v2, k3, v3);
