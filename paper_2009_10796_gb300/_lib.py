@@ -131,6 +131,9 @@ class DDGIError(RuntimeError):
 def load(path: str = LIB_PATH):
     """Load libddgi.so (raise if it is missing) and declare every entry point."""
     global _lib
+    lib = _lib
+    if lib is not None:
+        return lib
     with _lock:
         if _lib is not None:
             return _lib

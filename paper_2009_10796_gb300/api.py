@@ -20,9 +20,13 @@ __all__ = ["Scene", "Volume", "Cascade", "IrradianceField", "trace", "lights_str
 
 
 def _stream(stream):
+    """The stream's handle as an integer (None: torch's current stream of the
+    current device, read without building a Stream object)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _ptr(t: torch.Tensor):
@@ -32,21 +36,33 @@ def _ptr(t: torch.Tensor):
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _np(a, dtype):
     return np.ascontiguousarray(np.asarray(a, dtype=dtype))
 
 
+def _xyz(v):
+    """Three floats of a tuple, list, array or tensor of three numbers."""
+    try:
+        x, y, z = v.tolist() if hasattr(v, "tolist") else v
+        return float(x), float(y), float(z)
+    except (TypeError, ValueError):   # other shapes and element types
+        return tuple(float(x) for x in np.asarray(v, dtype=np.float64).reshape(3))
+
+
 def _f3(v):
-    return _lib.F3(*[float(x) for x in np.asarray(v, dtype=np.float64).reshape(3)])
+    return _lib.F3(*_xyz(v))
+
+
+_F15 = C.c_float * 15
 
 
 def lights_struct(lights) -> _lib.Lights:
     """Any object with sun_dir, sun_irradiance, sky_a, sky_b, sky_up."""
-    return _lib.Lights(_f3(lights.sun_dir), _f3(lights.sun_irradiance), _f3(lights.sky_a),
-                       _f3(lights.sky_b), _f3(lights.sky_up))
+    return _lib.Lights.from_buffer(_F15(*_xyz(lights.sun_dir), *_xyz(lights.sun_irradiance), *_xyz(lights.sky_a),
+                                        *_xyz(lights.sky_b), *_xyz(lights.sky_up)))
 
 
 def bvh_check(verts, tris) -> dict:
@@ -557,7 +573,7 @@ class ProbeQuery(torch.autograd.Function):
     def backward(ctx, dE):
         volume, pos, nrm, camera = ctx.args
         g = volume.query_backward(pos, nrm, camera, dE)
-        return torch.nn.functional.pad(g, (0, 1)), None, None, None, None
+        return torch.constant_pad_nd(g, (0, 1)), None, None, None, None
 
 
 class IrradianceField(torch.autograd.Function):

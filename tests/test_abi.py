@@ -119,3 +119,24 @@ def test_descriptor_limits_without_gpu(lib):
         d = api.desc_struct(synth.room_volume(**kw))
         assert L.ddgi_volume_create(C.byref(d), C.byref(out)) == 1
         assert msg in L.ddgi_last_error(), (kw, L.ddgi_last_error())
+
+
+def test_vector_arguments_convert_alike():
+    """Three numbers as a tuple, list, array, tensor or row of one give the same
+    floats; anything else is refused."""
+    import pytest
+    import torch
+
+    from paper_2009_10796_gb300 import api
+    want = [0.5, -1.0, 3.0]
+    for v in ((0.5, -1, 3), [0.5, -1.0, 3.0], np.array(want), np.array([want], np.float32), torch.tensor(want)):
+        assert list(api._f3(v)) == want
+
+    class L:
+        sun_dir, sun_irradiance, sky_a, sky_b, sky_up = want, np.array(want), [want], (0, 1, 0), torch.tensor(want)
+    s = api.lights_struct(L)
+    assert list(s.sun_dir) == list(s.sun_irradiance) == list(s.sky_a) == list(s.sky_up) == want
+    assert list(s.sky_b) == [0.0, 1.0, 0.0]
+    for bad in ([1.0, 2.0], None, "abc", np.zeros((2, 3))):
+        with pytest.raises((ValueError, TypeError)):
+            api._f3(bad)
