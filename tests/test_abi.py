@@ -124,7 +124,7 @@ def test_descriptor_limits_without_gpu(lib):
 def test_vector_arguments_convert_alike():
     """Three numbers as a tuple, list, array, tensor or row of one give the same
     floats; anything else is refused."""
-    import pytest
+    import numpy as np
     import torch
 
     from paper_2009_10796_gb300 import api
