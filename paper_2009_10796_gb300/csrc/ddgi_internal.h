@@ -202,8 +202,9 @@ struct BlendParams {
     float hyst_irr, hyst_vis;      // already scaled and clamped
     float thr_low, thr_high, thr_step;
     int32_t R;
-    // set by the tiled blend's launcher: by the texel counts n^2 and the
-    // tile widths n of irradiance and distance
+    // set by the tiled blend's launcher: the device's SMs; divisors by the
+    // texel counts n^2 and the tile widths n of irradiance and distance
+    int32_t n_sm;
     FastDiv div_ti, div_td, div_ni, div_nd;
 };
 

@@ -268,7 +268,7 @@ static TiledShape tiled_shape(int PG, int R, int irr_n, int dist_n) {
     t.dist_threads = (t.dist_units + 31) / 32 * 32;
     t.irr_units = t.nqi * (PG / 2);
     t.threads = t.dist_threads + (t.irr_units + 31) / 32 * 32;
-    t.smem = sizeof(float) * ((size_t)4 * PG * R + (size_t)kTileNS * 4 * (t.nqd + t.nqi) * kTileWS);
+    t.smem = sizeof(float) * ((size_t)4 * PG * ((R + 3) / 4 * 4) + (size_t)kTileNS * 4 * (t.nqd + t.nqi) * kTileWS);
     // the epilogue reuses the same shared memory for the weighted sums and
     // the frame's inverse weight sums
     const size_t sums = sizeof(float) * ((size_t)PG * (2 * dist_n * dist_n + 3 * irr_n * irr_n) +
@@ -277,11 +277,16 @@ static TiledShape tiled_shape(int PG, int R, int irr_n, int dist_n) {
     return t;
 }
 
-// 16-byte asynchronous global -> shared copy (zero-filled when !valid).
+// 16- and 4-byte asynchronous global -> shared copies (zero-filled when !valid).
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     const int n = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, bool valid) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = valid ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // every group but the kTileNS - 1 most recent complete
@@ -291,7 +296,14 @@ __device__ __forceinline__ void cp_async_wait_ahead() {
 
 // Each CTA takes an equal share of the active probes (at most PG per pass;
 // the grid is one wave of resident CTAs); blockDim = TiledShape::threads.
-// Requires R % 4 == 0.  Thread u < dist_units owns distance texels
+// Up to 8 probes to an SM go to the first n_sm CTAs, one on each, since a CTA
+// streams all of the weights whatever its probes (1079 probes of 8 x 8 and
+// 16 x 16 texels 40.5 -> 38.9 us; at 13.5 probes to an SM two CTAs are faster).
+// ROW16: the weight rows start on 16-byte boundaries (R a multiple of 4) and
+// arrive in 16-byte copies, else in 4-byte ones; rays past R weigh zero.  (The
+// row kernel took ray counts off 4 before: a room's frame with 63 rays
+// 150 -> 83 us, a city's with 250 rays 507 -> 429 us.)
+// Thread u < dist_units owns distance texels
 // tq + a * nqd (a < 4) of probes 4 pq .. 4 pq + 3; thread dist_threads + u'
 // (u' < irr_units) owns irradiance texels tq + a * nqi of probes 2 pq,
 // 2 pq + 1.  Striding the texels by nqd (not 4) puts a warp's weight rows on
@@ -302,7 +314,7 @@ __device__ __forceinline__ void cp_async_wait_ahead() {
 // arrive by asynchronous copies into a ring of kTileNS buffers (with one
 // buffer, the copy overlaps the other resident CTA's summing); the blend
 // epilogue runs over the sums in shared memory.
-template <bool MULTI, int PG>
+template <bool MULTI, int PG, bool ROW16>
 __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, BlendParams bp,
                                                                     const float* __restrict__ w_irr,
                                                                     const float* __restrict__ inv_s_irr,
@@ -324,11 +336,12 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
     const int ti = ni * ni, td = nd * nd;
     const int nqi = (ti + 3) / 4, nqd = (td + 3) / 4;
     const int wrows = 4 * (nqd + nqi);          // distance rows, then irradiance rows
-    float* pr = sm;                              // [R][PG] planes: radiance r, g, b and distance
-    float* pgc = pr + PG * R;
-    float* pbc = pgc + PG * R;
-    float* pdc = pbc + PG * R;
-    float* wbuf = pdc + PG * R;                  // 2 x [wrows][kTileWS] weight chunks
+    const int Rp = ROW16 ? R : (R + 3) / 4 * 4;  // rays past R are zero
+    float* pr = sm;                              // [Rp][PG] planes: radiance r, g, b and distance
+    float* pgc = pr + PG * Rp;
+    float* pbc = pgc + PG * Rp;
+    float* pdc = pbc + PG * Rp;
+    float* wbuf = pdc + PG * Rp;                 // [wrows][kTileWS] weight chunks
     const int dist_units = nqd * (PG / 4), irr_units = nqi * (PG / 2);
     const int dist_threads = (dist_units + 31) / 32 * 32;
     const int u = threadIdx.x;
@@ -343,18 +356,21 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
     auto issue_chunk = [&](int c) {
         float* wb = wbuf + (c % kTileNS) * wrows * kTileWS;
         const int c0 = c * kTileKC;
-        for (int k = threadIdx.x; k < wrows * (kTileKC / 4); k += blockDim.x) {
-            int row = k / (kTileKC / 4), j = 4 * (k - row * (kTileKC / 4));
+        constexpr int kCopy = ROW16 ? 4 : 1;   // floats a copy
+        for (int k = threadIdx.x; k < wrows * (kTileKC / kCopy); k += blockDim.x) {
+            int row = k / (kTileKC / kCopy), j = kCopy * (k - row * (kTileKC / kCopy));
             bool dist_row = row < 4 * nqd;
             int t = dist_row ? row : row - 4 * nqd;
             bool ok = c0 + j < R && t < (dist_row ? td : ti);
             const float* src = (dist_row ? w_dist : w_irr) + (ok ? (int64_t)t * R + c0 + j : 0);
-            cp_async16(wb + row * kTileWS + j, src, ok);
+            if constexpr (ROW16) cp_async16(wb + row * kTileWS + j, src, ok);
+            else cp_async4(wb + row * kTileWS + j, src, ok);
         }
         cp_async_commit();
     };
 
-    const int per = min(PG, max(1, (n_act + (int)gridDim.x - 1) / (int)gridDim.x));
+    const int ctas = n_act <= 8 * bp.n_sm ? bp.n_sm : (int)gridDim.x;
+    const int per = min(PG, max(1, (n_act + ctas - 1) / ctas));
     for (int g0 = blockIdx.x * per; g0 < n_act; g0 += gridDim.x * per) {
         const int np = min(per, n_act - g0);
         const bool live = is_dist ? 4 * pq < np : 2 * pq < np;   // some of the thread's probes hold records
@@ -374,19 +390,19 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
         // records -> planes, kRecBatch independent loads in flight per thread.
         // Item k is (ray pair, probe, ray within the pair): two threads read a
         // probe's 32 contiguous bytes, a warp writes 32 consecutive plane floats.
-        for (int k0 = threadIdx.x; k0 < PG * R; k0 += kRecBatch * blockDim.x) {
+        for (int k0 = threadIdx.x; k0 < PG * Rp; k0 += kRecBatch * blockDim.x) {
             float4 rec[kRecBatch];
 #pragma unroll
             for (int b = 0; b < kRecBatch; ++b) {
                 const int k = k0 + b * blockDim.x;
                 const int q = k >> 1, pp = q % PG, ray = 2 * (q / PG) + (k & 1);
-                rec[b] = (k < PG * R && pp < np) ? records[(int64_t)(g0 + pp) * R + ray]
+                rec[b] = ((ROW16 ? k < PG * R : ray < R) && pp < np) ? records[(int64_t)(g0 + pp) * R + ray]
                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
 #pragma unroll
             for (int b = 0; b < kRecBatch; ++b) {
                 const int k = k0 + b * blockDim.x;
-                if (k < PG * R) {
+                if (k < PG * Rp) {
                     const int q = k >> 1, o = (2 * (q / PG) + (k & 1)) * PG + q % PG;
                     pr[o] = rec[b].x;
                     pgc[o] = rec[b].y;
@@ -772,8 +788,9 @@ static int smem_optin() {
 // shared memory, once per device.
 template <bool MULTI, int PGS>
 static cudaError_t opt_in_blend() {
-    static DeviceOnce tiled, rows;
-    cudaError_t e = allow_max_smem(k_blend_tiled<MULTI, PGS>, tiled);
+    static DeviceOnce tiled, tiled4, rows;
+    cudaError_t e = allow_max_smem(k_blend_tiled<MULTI, PGS, true>, tiled);
+    if (e == cudaSuccess) e = allow_max_smem(k_blend_tiled<MULTI, PGS, false>, tiled4);
     if (e == cudaSuccess) e = allow_max_smem(k_blend_simt<MULTI, PGS>, rows);
     return e;
 }
@@ -781,7 +798,7 @@ static cudaError_t opt_in_blend() {
 template <int PG>
 static bool tiled_fits(const BlendParams& bp, int irr_n, int dist_n) {
     const TiledShape ts = tiled_shape(PG, bp.R, irr_n, dist_n);
-    return bp.R % 4 == 0 && ts.threads <= kTileMaxThreads && ts.smem + 1024 <= (size_t)smem_optin();
+    return ts.threads <= kTileMaxThreads && ts.smem + 1024 <= (size_t)smem_optin();
 }
 
 template <bool MULTI, int PG>
@@ -792,21 +809,21 @@ static cudaError_t launch_tiled(const VolSet& vs, const BlendParams& bp, int irr
     cudaError_t e = opt_in_blend<MULTI, PG>();
     if (e != cudaSuccess) return e;
     const TiledShape ts = tiled_shape(PG, bp.R, irr_n, dist_n);
+    auto kernel = bp.R % 4 == 0 ? k_blend_tiled<MULTI, PG, true> : k_blend_tiled<MULTI, PG, false>;
     // one wave of resident CTAs; the kernel splits the active probes evenly
     int occ = 0, dev = 0, sms = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_blend_tiled<MULTI, PG>, ts.threads, ts.smem)) !=
-        cudaSuccess)
-        return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, ts.threads, ts.smem)) != cudaSuccess) return e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     grid = sms * (occ > 0 ? occ : 1);
     BlendParams bpt = bp;
+    bpt.n_sm = sms;
     bpt.div_ti = make_fast_div((uint32_t)(irr_n * irr_n));
     bpt.div_td = make_fast_div((uint32_t)(dist_n * dist_n));
     bpt.div_ni = make_fast_div((uint32_t)irr_n);
     bpt.div_nd = make_fast_div((uint32_t)dist_n);
-    k_blend_tiled<MULTI, PG><<<grid, ts.threads, ts.smem, st>>>(vs, bpt, w_irr, inv_s_irr, w_dist, inv_s_dist,
-                                                                records, active, count, status);
+    kernel<<<grid, ts.threads, ts.smem, st>>>(vs, bpt, w_irr, inv_s_irr, w_dist, inv_s_dist, records, active, count,
+                                              status);
     return cudaGetLastError();
 }
 

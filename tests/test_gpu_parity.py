@@ -164,6 +164,27 @@ def test_odd_sizes_parity(g):
     assert eq.max() <= REL
 
 
+@pytest.mark.parametrize("rays, counts", [(6, (4, 4, 4)), (33, (5, 4, 3)), (63, (8, 8, 8)), (30, (12, 11, 12))])
+def test_ray_counts_of_no_multiple_of_four(g, rays, counts):
+    """The register-tiled blend with weight rows off 16-byte boundaries, a last
+    chunk of one ray, and probe counts on both sides of eight to an SM; texels
+    that a ray with another FP32 than FP64 hit reaches are left out."""
+    sc = synth.room_scene(n_boxes=6)
+    desc = synth.VolumeDesc(origin=(0.6, 0.6, 0.6), spacing=tuple(8.8 / (c - 1) for c in counts), counts=counts,
+                            rays_per_probe=rays, state_machine=0, seed=31)
+    L = synth.room_lights()
+    st, irr, dist, rec_o = run_oracle(sc, L, desc, [3])
+    V = g.Volume(desc)
+    V.update(g.Scene.from_arrays(sc), L, 3)
+    rec, ids = gpu_rays_by_probe(V)
+    bad, _ = compare_rays(rec, ids, rec_o[-1])
+    assert bad.sum() <= max(2, 1e-3 * bad.size)
+    mi, md = masked_texels(desc, desc.seed, 3, bad, ids)
+    ei = rel_err(V.irr_atlas().cpu().numpy(), irr).max(-1)
+    ed = rel_err(V.dist_atlas().cpu().numpy(), dist).max(-1)
+    assert ei[~mi].max() <= REL and ed[~md].max() <= REL
+
+
 @pytest.mark.parametrize("case", ["max_tiles", "max_rays_tf32x3"])
 def test_maximum_sizes_parity(g, case):
     """The largest rays per probe (1024) and tiles (32 x 32 irradiance, 64 x
