@@ -9,16 +9,13 @@ namespace ddgi {
 // (16-byte stores when the run is aligned), so each warp writes whole lines,
 // for page-locked host memory written across the host link; otherwise each
 // thread stores its own three floats (device memory).
-// Five CTAs per SM (48 registers, a short spill) measured 1 us faster on the
-// 1080p query than four in the specialised forms; the general form keeps four,
-// and so do the gamma 1 and moved forms, whose points are often in random
-// order (281 and 300 us for 1080p of them, 290 and 312 us at five).
+// Four CTAs per SM (64 registers): 1920 x 1080 points of a hall take 70.0 us,
+// 72.2 us at five (48 registers, spills).
 constexpr int kQueryThreads = 256;
-constexpr int query_ctas(int form) { return form == kQueryGeneral || form == kQueryGamma1 || form == kQueryMoved ? 4 : 5; }
 template <bool STAGE_OUT, int FORM>
-__global__ void __launch_bounds__(kQueryThreads, query_ctas(FORM)) k_query(VolView v, const float* __restrict__ pos,
-                                                         const float* __restrict__ nrm, int64_t n, float3 cam,
-                                                         float* __restrict__ out) {
+__global__ void __launch_bounds__(kQueryThreads, 4) k_query(VolView v, const float* __restrict__ pos,
+                                                            const float* __restrict__ nrm, int64_t n, float3 cam,
+                                                            float* __restrict__ out) {
     pdl_wait();
     pdl_trigger();
     __shared__ __align__(16) float s_out[3 * kQueryThreads];
@@ -66,7 +63,7 @@ __global__ void __launch_bounds__(kQueryThreads, query_ctas(FORM)) k_query(VolVi
 // dirs are the unit directions the hits were reached along.  Output is the
 // prefiltered radiance M read in the mirror direction (no factor pi).
 template <int FORM>
-__global__ void __launch_bounds__(256) k_query_glossy(VolView v, const float* __restrict__ pos,
+__global__ void __launch_bounds__(256, 4) k_query_glossy(VolView v, const float* __restrict__ pos,
                                                       const float* __restrict__ nrm, const float* __restrict__ dirs,
                                                       int64_t n, float* __restrict__ out) {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n;
