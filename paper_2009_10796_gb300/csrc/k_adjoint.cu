@@ -105,7 +105,7 @@ __device__ __forceinline__ void query_M_adjoint_warp(const VolView& v, bool vali
             float4 d = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (act & (1u << c)) {
                 const int p = cage.probe(v, c);
-                const float w = corner_weight<FORM, kIeee>(v, q, cage, c, p, n);
+                const float w = corner_weight<FORM, true>(v, q, cage, c, p, n);
                 float er, eg, eb;
                 f2_unpack(irr_taps<FORM>(v, p, fp, bw, eb), er, eg);
                 acc.x += w * decode_slope<FORM>(er, v.half_gamma, d.x);
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(32 * kAdjWarps) k_shade_adjoint(DevScene s, Vo
                 float kk = cosl * 0.318309886183790672f;
                 direct = f3(L.sun_irr.x * kk, L.sun_irr.y * kk, L.sun_irr.z * kk);
             }
-            float3 M = query_M<FORM, true, kSteady>(v_before, x, n, wo);
+            float3 M = query_M<FORM>(v_before, x, n, wo);
             atomicAdd(d_albedo + 3 * at.x + 0, g4.x * (direct.x + M.x));
             atomicAdd(d_albedo + 3 * at.x + 1, g4.y * (direct.y + M.y));
             atomicAdd(d_albedo + 3 * at.x + 2, g4.z * (direct.z + M.z));

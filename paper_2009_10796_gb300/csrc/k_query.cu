@@ -9,8 +9,8 @@ namespace ddgi {
 // (16-byte stores when the run is aligned), so each warp writes whole lines,
 // for page-locked host memory written across the host link; otherwise each
 // thread stores its own three floats (device memory).
-// Four CTAs per SM (64 registers): 1920 x 1080 points of a hall take 70.0 us,
-// 72.2 us at five (48 registers, spills).
+// Four CTAs per SM (64 registers): 1920 x 1080 points of a hall take 72 us; at
+// five (48 registers, spills) the time was 3 % longer.
 constexpr int kQueryThreads = 256;
 template <bool STAGE_OUT, int FORM>
 __global__ void __launch_bounds__(kQueryThreads, 4) k_query(VolView v, const float* __restrict__ pos,

@@ -436,9 +436,8 @@ __global__ void __launch_bounds__(256, 4) k_shade(DevScene s, VolSet vs, Lights 
         const float3 tol = f3(-L.sun_dir.x, -L.sun_dir.y, -L.sun_dir.z);
         const float kk = hr.z != 0.0f ? dot(n, tol) * 0.318309886183790672f : 0.0f;   // 1/pi
         const int orig = __float_as_int(__ldg(&s.tris[3 * (int64_t)k].w));
-        constexpr CornerMode kMode = FORM == kQueryHalf || FORM == kQueryE5 ? kIssue : kSteady;
-        float3 M = MULTI ? cascade_M<FORM, kMode>(vs.table, vs.n, x, n, f3(-d.x, -d.y, -d.z))
-                         : query_M<FORM, true, kMode>(v, x, n, f3(-d.x, -d.y, -d.z));
+        float3 M = MULTI ? cascade_M<FORM>(vs.table, vs.n, x, n, f3(-d.x, -d.y, -d.z))
+                         : query_M<FORM>(v, x, n, f3(-d.x, -d.y, -d.z));
         int2 at = __ldg(s.attr + orig);
         float4 rho = __ldg(s.albedo + at.x);
         float3 Le = f3(0.0f, 0.0f, 0.0f);

@@ -151,14 +151,14 @@ __device__ __forceinline__ Footprint footprint(float2 u, int n) {
     return f;
 }
 
-// The same footprint in the specialised queries, whose instruction issue
-// bounds them: the texel position as one multiply-add, and its floor by adding
-// 2^23 rounded down (positions lie in [0.5, n + 0.5], n <= 64, so the sum's
-// low bits are the texel).  The clamp keeps a NaN position (a point on a
-// probe: no direction) inside the tile.
+// The same footprint, value for value, in the specialised queries, whose
+// instruction issue bounds them: the floor by adding 2^23 rounded down (texel
+// positions lie in [0.5, n + 0.5], n <= 64, so the sum's low bits are the
+// texel) instead of conversions and clamps.  The one clamp left keeps a NaN
+// position (a point on a probe: no direction) inside the tile.
 __device__ __forceinline__ Footprint footprint_issue(float2 u, int n) {
-    const float h = 0.5f * (float)n;
-    const float sx = fmaf(u.x, h, h + 0.5f), sy = fmaf(u.y, h, h + 0.5f);
+    const float sx = 1.0f + (u.x + 1.0f) * 0.5f * (float)n - 0.5f;
+    const float sy = 1.0f + (u.y + 1.0f) * 0.5f * (float)n - 0.5f;
     const float kx = __fadd_rd(sx, 8388608.0f), ky = __fadd_rd(sy, 8388608.0f);
     Footprint f;
     f.x0 = min(__float_as_int(kx) & 0x7f, n);
@@ -468,25 +468,12 @@ __device__ __forceinline__ uint64_t irr_taps(const VolView& v, int p, const Foot
     return rg;
 }
 
-// The distance moments of a form's atlas at a footprint with the bilinear
-// weights of sample_dist_at.
-template <int FORM>
-__device__ __forceinline__ float2 dist_taps_weighted(const VolView& v, int p, const Footprint& f) {
-    if constexpr (FORM == kQueryGeneral) return sample_dist_at(v, p, f);
-    if constexpr (!QueryForm<FORM>::kHalf) return sample_dist_fp32(v, p, f);
-    const int row = v.dist_n + 2;
-    const uint32_t* q = (const uint32_t*)v.dist + (int64_t)p * v.dist_tile + (int64_t)f.y0 * row + f.x0;
-    const uint32_t h[4] = {__ldg(q), __ldg(q + 1), __ldg(q + row), __ldg(q + row + 1)};
-    float2 a[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) a[k] = __half22float2(*reinterpret_cast<const __half2*>(&h[k]));
-    const Bilerp w = bilerp_weights(f);
-    return make_float2(w.w00 * a[0].x + w.w10 * a[1].x + w.w01 * a[2].x + w.w11 * a[3].x,
-                       w.w00 * a[0].y + w.w10 * a[1].y + w.w01 * a[2].y + w.w11 * a[3].y);
-}
-
-// The same as three lerps of packed (mean, mean square) pairs.
-template <int FORM>
+// The distance moments of a form's atlas at a footprint as packed (mean, mean
+// square) pairs.  A Chebyshev weight takes the variance, a difference, from
+// these sums, so their order is kept as it was in each direction: the second
+// tap's product first in queries, the first's in the adjoint (ADJOINT).  With
+// the other order points near an occluder moved by up to 0.3 %.
+template <int FORM, bool ADJOINT = false>
 __device__ __forceinline__ float2 dist_taps(const VolView& v, int p, const Footprint& f) {
     if constexpr (FORM == kQueryGeneral) return sample_dist_at(v, p, f);
     const int row = v.dist_n + 2;
@@ -508,11 +495,14 @@ __device__ __forceinline__ float2 dist_taps(const VolView& v, int p, const Footp
         c = __ldg(q + row);
         d = __ldg(q + row + 1);
     }
-    const uint64_t tx = f2_pack(f.tx, f.tx), ty = f2_pack(f.ty, f.ty);
-    const uint64_t top = f2_fma(tx, f2_sub(b, a), a), bottom = f2_fma(tx, f2_sub(d, c), c);
-    float2 m;
-    f2_unpack(f2_fma(ty, f2_sub(bottom, top), top), m.x, m.y);
-    return m;
+    const Bilerp w = bilerp_weights(f);
+    const uint64_t W00 = f2_pack(w.w00, w.w00), W10 = f2_pack(w.w10, w.w10);
+    uint64_t m = ADJOINT ? f2_fma(W10, b, f2_mul(W00, a)) : f2_fma(W00, a, f2_mul(W10, b));
+    m = f2_fma(f2_pack(w.w01, w.w01), c, m);
+    m = f2_fma(f2_pack(w.w11, w.w11), d, m);
+    float2 r;
+    f2_unpack(m, r.x, r.y);
+    return r;
 }
 
 // The eight-probe cage of a biased point: its base cell and, per axis, the
@@ -560,19 +550,17 @@ __device__ __forceinline__ Cage cage_of(const VolView& v, const LocalPoint& q) {
     return k;
 }
 
-// How a corner's depth lookup is evaluated.  kIssue: the fewest instructions
-// (the queries of points).  kSteady: the hit shading's arithmetic, whose
-// results feed the next frame's: where a Chebyshev weight is near the depth it
-// tests, its last bits reach the atlas and every later frame, so they stay as
-// they are (FP16 and RGB9E5 atlases round far coarser, and take kIssue).
-// kIeee: the distance and the lookup's coordinates by rounded square root and
-// division (the adjoint, where one point's weight can be a whole texel's
-// gradient).
-enum CornerMode { kIssue, kSteady, kIeee };
-
 // Weight of cage corner c (probe p) in a form's query: trilinear, backface
-// and Chebyshev factors, floored (query_M_look).
-template <int FORM, CornerMode MODE>
+// and Chebyshev factors, floored (query_M_look).  Where a Chebyshev weight is
+// near the depth it tests, the last bits of the distance and of the lookup
+// decide it, and hit shading carries them into the atlas and every later
+// frame: the operations are those of the general form.  BRANCH keeps the
+// general form's branches, which the cascade kernels are faster with (2567 us a
+// frame against 2580); a single volume's are slower (city frame with FP16
+// atlases 504 us against 498).  IEEE: the distance and the lookup's
+// coordinates by rounded square root and division (the adjoint, where one
+// point's weight can be a whole texel's gradient).
+template <int FORM, bool IEEE = false, bool BRANCH = false>
 __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoint& q, const Cage& k, int c, int p,
                                                float3 n) {
     const int o0 = c & 1, o1 = (c >> 1) & 1, o2 = c >> 2;
@@ -590,22 +578,20 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
     const float3 pv = a + q.lb;                                                // biased point - probe
     const float rr = dot(pv, pv);
     float wc = 1.0f;
-    if constexpr (MODE == kIssue) {
-        // rr = 0 makes r a NaN, which is not beyond any mean: wc = 1
-        const float r = rr * rsqrtf(rr);
-        const float2 mom = dist_taps<FORM>(v, p, footprint_issue(oct_encode_fast(pv), v.dist_n));
-        const float var = fmaxf(mom.y - mom.x * mom.x, 0.0f);
-        const float dr = r - mom.x;
-        wc = r > mom.x ? __fdividef(var, var + dr * dr) : 1.0f;
-    } else if (rr > 0.0f) {
-        const float r = MODE == kIeee ? sqrtf(rr) : rr * rsqrtf(rr);
-        const float ir = MODE == kIeee ? 1.0f / r : rsqrtf(rr);
-        const float2 u = MODE == kIeee ? oct_encode(ir * pv) : oct_encode_fast(ir * pv);
-        const float2 mom = dist_taps_weighted<FORM>(v, p, footprint(u, v.dist_n));
-        if (r > mom.x) {
+    if (!BRANCH || rr > 0.0f) {   // without the branch rr = 0 makes a NaN of r, beyond no mean
+        const float r = IEEE ? sqrtf(rr) : rr * rsqrtf(rr);
+        const float2 u = IEEE ? oct_encode((1.0f / r) * pv) : oct_encode_fast(rsqrtf(rr) * pv);
+        const float2 mom = dist_taps<FORM, IEEE>(v, p, footprint_issue(u, v.dist_n));
+        auto chebyshev = [&]() {
             const float var = fmaxf(mom.y - mom.x * mom.x, 0.0f);
             const float dr = r - mom.x;
-            wc = __fdividef(var, var + dr * dr);
+            return __fdividef(var, var + dr * dr);
+        };
+        if constexpr (BRANCH) {
+            if (r > mom.x) wc = chebyshev();
+        } else {
+            const float c = chebyshev();
+            wc = rr > 0.0f && r > mom.x ? c : 1.0f;
         }
     }
     return wt * wb * fmaxf(wc, 1e-6f);
@@ -618,20 +604,20 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
 // channels of the irradiance taps and their decode carried as packed FP32
 // pairs (the blue channel scalar).  Bound by instruction issue for
 // neighbouring points: 1920 x 1080 of them on 16 x 8 x 16 probes, beyond the
-// grid planes on one axis, take 70 us (general form: 142-182 us by the
-// storage format and gamma).  Points in random order are bound by L2 sectors
-// instead (137-168 us).
+// grid planes on one axis, take 72-83 us by the storage format (general form:
+// 142-182 us).  Points in random order are bound by L2 sectors instead
+// (124-165 us).
 // EDGES: corners of zero trilinear weight are passed over (no lookup, the
 // same sums), which a volume's points on and beyond its grid planes gain
 // from: the glossy lookup of 960 x 540 such points 33.6 -> 22.6 us, a
 // city frame's hit shading 74 -> 72 us.  Cascades leave it out: a volume of
 // weight 0 at its edges is not read there, and their kernels spill more with
 // the test (2852 -> 2912 us a frame).
-template <int FORM, bool EDGES, CornerMode MODE>
+template <int FORM, bool EDGES>
 __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, float3 n, float3 wo, float3 look) {
     const LocalPoint q = local_point(v, x, n, wo);
     const Cage k = cage_of(v, q);
-    const Footprint fn = MODE == kIssue ? footprint_issue(oct_encode(look), v.irr_n) : footprint(oct_encode(look), v.irr_n);
+    const Footprint fn = footprint_issue(oct_encode(look), v.irr_n);
     const Bilerp wn = bilerp_weights(fn);
     int pc[8];
     unsigned act = 0;
@@ -645,7 +631,7 @@ __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, 
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         if (!(act & (1u << c)) || (EDGES && k.trilinear(c) == 0.0f)) continue;
-        const float w = corner_weight<FORM, MODE>(v, q, k, c, pc[c], n);
+        const float w = corner_weight<FORM, false, !EDGES>(v, q, k, c, pc[c], n);
         float er, eg, eb;
         f2_unpack(irr_taps<FORM>(v, pc[c], fn, wn, eb), er, eg);
         if constexpr (QueryForm<FORM>::kGamma1) {
@@ -679,9 +665,9 @@ __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, 
 // (Sec. 4.4); the bias and the backface weights use n either way.
 // FORM: the view's form (query_form); query_M_look_fast serves all but the
 // general one.
-template <int FORM = kQueryGeneral, bool EDGES = true, CornerMode MODE = kIssue>
+template <int FORM = kQueryGeneral, bool EDGES = true>
 __device__ __forceinline__ float3 query_M_look(const VolView& v, float3 x, float3 n, float3 wo, float3 look) {
-    if constexpr (FORM != kQueryGeneral) return query_M_look_fast<FORM, EDGES, MODE>(v, x, n, wo, look);
+    if constexpr (FORM != kQueryGeneral) return query_M_look_fast<FORM, EDGES>(v, x, n, wo, look);
     const LocalPoint q = local_point(v, x, n, wo);
     float g[3] = {(q.hi.x + q.lb.x) / v.spacing.x, (q.hi.y + q.lb.y) / v.spacing.y,
                   (q.hi.z + q.lb.z) / v.spacing.z};
@@ -753,9 +739,9 @@ __device__ __forceinline__ float3 query_M_look(const VolView& v, float3 x, float
     return f3(a.x * a.x, a.y * a.y, a.z * a.z);
 }
 
-template <int FORM = kQueryGeneral, bool EDGES = true, CornerMode MODE = kIssue>
+template <int FORM = kQueryGeneral, bool EDGES = true>
 __device__ __forceinline__ float3 query_M(const VolView& v, float3 x, float3 n, float3 wo) {
-    return query_M_look<FORM, EDGES, MODE>(v, x, n, wo, n);
+    return query_M_look<FORM, EDGES>(v, x, n, wo, n);
 }
 
 // Cascade value M at x (Sec. 7.3): volumes densest first; each volume's
@@ -769,7 +755,7 @@ __device__ __forceinline__ float volume_weight(const VolView& v, float3 x) {
     return wx * wy * wz;
 }
 
-template <int FORM = kQueryGeneral, CornerMode MODE = kIssue>
+template <int FORM = kQueryGeneral>
 __device__ __forceinline__ float3 cascade_M(const VolView* vols, int n, float3 x, float3 nrm, float3 wo) {
     float sum = 0.0f;
     float3 acc = f3(0.0f, 0.0f, 0.0f);
@@ -777,7 +763,7 @@ __device__ __forceinline__ float3 cascade_M(const VolView* vols, int n, float3 x
         const VolView& v = vols[k];
         float take = fminf(volume_weight(v, x), 1.0f - sum);
         if (!(take > 0.0f)) continue;
-        float3 M = query_M<FORM, false, MODE>(v, x, nrm, wo);
+        float3 M = query_M<FORM, false>(v, x, nrm, wo);
         acc = acc + take * M;
         sum += take;
         if (sum >= 1.0f) break;
