@@ -772,7 +772,7 @@ static ddgi_status update_impl(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
             const FrameRot rb = frame_rotation(d.seed + 0xD1B54A32D192ED03ULL * (uint64_t)(b + 1), params->frame);
             DDGI_CK(launch_frame_setup(rb, v->R, d.irr_n, d.dist_n, d.dist_cos_power, v->sf64, v->conv_dirs,
                                        v->conv_w_irr, v->conv_inv_irr, v->conv_w_dist, v->conv_inv_dist,
-                                       v->counts + 4, kCounterInts - 4, st));
+                                       v->counts + 4, kCounterInts - 4, nullptr, st));
             DDGI_CK(launch_trace_wavefront(s->dev, view, make_lights(lights), v->conv_dirs, v->R, v->perm, v->lists,
                                            v->counts + 2, v->records, v->shadow_list, v->hit_list, v->shadow_count,
                                            sms * 8, (end - begin) * v->R, st, nullptr));
@@ -822,7 +822,7 @@ static ddgi_status update_impl(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
                                     v->records, v->lists + v->P, v->counts + 1, v->status, sms, st));
         else
             DDGI_CK(launch_blend(view, bp, v->w_irr, v->inv_s_irr, v->w_dist, v->inv_s_dist, v->records,
-                                 v->lists + v->P, v->counts + 1, v->status, sms * 4, st));
+                                 v->lists + v->P, v->counts + 1, v->status, sms * 4, false, st));
     }
     v->updates++;
     return DDGI_OK;
@@ -1714,7 +1714,7 @@ ddgi_status ddgi_diff_backward(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
     for (int f = n_frames - 1; f >= 0; --f) {
         FrameRot rot = frame_rotation(d.seed, first_frame + f);
         DDGI_CK(launch_frame_setup(rot, v->R, d.irr_n, d.dist_n, d.dist_cos_power, v->sf64, v->dirs, v->w_irr,
-                                   v->inv_s_irr, v->w_dist, v->inv_s_dist, nullptr, 0, st));
+                                   v->inv_s_irr, v->w_dist, v->inv_s_dist, nullptr, 0, nullptr, st));
         DDGI_CK(launch_blend_adjoint(snap_view(f + 1), v->w_irr, v->inv_s_irr, g, (int)v->P, v->R, v->records, st));
         DDGI_CK(cudaMemsetAsync(gp, 0, gbytes, st));
         DDGI_CK(launch_shade_adjoint(s->dev, snap_view(f), L, v->dirs, (int)v->P, v->R, v->records, d_emit_dev,

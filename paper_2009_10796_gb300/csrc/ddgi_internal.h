@@ -237,7 +237,8 @@ FrameRot frame_rotation(uint64_t seed, int64_t frame);
 // then for ray i the two packed ray constants of dir_pre_pack at R + 2i.
 // Frame ray pattern and texel weights in one launch.  sf64: [R][3] double,
 // the unrotated pattern written once by launch_sf_table; the first n_zero
-// ints at zero (counters) are cleared by the same launch.
+// ints at zero (counters) are cleared by the same launch, and the ray order
+// (ray_order_morton) written to perm [R] unless that is nullptr.
 cudaError_t launch_sf_table(int R, double* sf64, cudaStream_t st);
 // Optional converge pass for new probes (Sec. 6.3): one batch's weighted
 // sums per list slot (init: first batch), then the texels and state advance.
@@ -250,7 +251,7 @@ cudaError_t launch_converge_finish(const VolView& v, const int32_t* list, const 
                                    int grid, cudaStream_t st);
 cudaError_t launch_frame_setup(const FrameRot& rot, int R, int irr_n, int dist_n, float cos_power,
                                const double* sf64, float4* dirs, float* w_irr, float* inv_s_irr, float* w_dist,
-                               float* inv_s_dist, int32_t* zero, int n_zero, cudaStream_t st);
+                               float* inv_s_dist, int32_t* zero, int n_zero, int32_t* perm, cudaStream_t st);
 // The same as two launches: the texel weights on st_weights, the directions
 // (and the counter clear) on st_dirs, so the weights can overlap the trace.
 cudaError_t launch_frame_setup_split(const FrameRot& rot, int R, int irr_n, int dist_n, float cos_power,
@@ -293,9 +294,9 @@ cudaError_t launch_classify(const DevScene& s, const VolView& v, const float4* d
 cudaError_t launch_classify_multi(const DevScene& s, const VolSet& vs, const float4* dirs, int R,
                                   const int32_t* perm, const int32_t* list, const int32_t* count, int4* scratch,
                                   uint32_t* next, cudaStream_t st);
-cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights& L,
-                               const float4* dirs, int R, const int32_t* active,
-                               const int32_t* count, float4* records, int grid, cudaStream_t st);
+cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights& L, const float4* dirs,
+                               int R, const int32_t* perm, const int32_t* active, const int32_t* count,
+                               float4* records, int grid, cudaStream_t st);
 // Per-volume device counters, one block cleared by one memset per frame:
 // [0] uninitialised-list count, [1] active-list count, [2] new-probe count,
 // [3] the optimizer's work counter (zeroed by each of its direction
@@ -330,10 +331,12 @@ cudaError_t launch_trace_wavefront_multi(const DevScene& s, const VolSet& vs, co
 // Morton order of the octahedral positions of the unrotated spherical-
 // Fibonacci directions (host; a rotation keeps neighbouring directions together)
 std::vector<int32_t> ray_order_morton(int R);
+// pdl: a programmatic dependent launch (nothing but a kernel before it on the
+// stream; the volume update waits for the side stream's weights there).
 cudaError_t launch_blend(const VolView& v, const BlendParams& bp, const float* w_irr,
                          const float* inv_s_irr, const float* w_dist, const float* inv_s_dist,
                          const float4* records, const int32_t* active, const int32_t* count,
-                         uint32_t* status, int grid, cudaStream_t st);
+                         uint32_t* status, int grid, bool pdl, cudaStream_t st);
 // blend over a volume set sharing irr_n / dist_n; probes_per_cta in
 // {4, 8, 16} (autotuned)
 cudaError_t launch_blend_set(const VolSet& vs, bool multi, const BlendParams& bp, int irr_n, int dist_n,

@@ -98,6 +98,30 @@ __global__ void k_sf_table(int R, double* sf64) {
     if (i < R) sf_dir(i, R, sf64 + 3 * i);
 }
 
+// The order in which a probe's warps take its rays (ray_order_morton, here in
+// FP32 and on the device for the allocation-free update): perm[rank of ray i's
+// key] = i.  Called by every thread of a block; i may be past R.
+__device__ void order_rays(const double* __restrict__ sf64, int R, int i, int32_t* perm) {
+    __shared__ uint32_t key[1024];
+    auto spread = [](uint32_t v) {
+        v = (v | (v << 8)) & 0x00ff00ffu;
+        v = (v | (v << 4)) & 0x0f0f0f0fu;
+        v = (v | (v << 2)) & 0x33333333u;
+        return (v | (v << 1)) & 0x55555555u;
+    };
+    for (int k = threadIdx.x; k < R; k += blockDim.x) {
+        const float2 u = oct_encode(f3((float)sf64[3 * k], (float)sf64[3 * k + 1], (float)sf64[3 * k + 2]));
+        key[k] = spread((uint32_t)fminf(1023.0f, (u.x + 1.0f) * 512.0f)) |
+                 (spread((uint32_t)fminf(1023.0f, (u.y + 1.0f) * 512.0f)) << 1);
+    }
+    __syncthreads();
+    if (i >= R) return;
+    const uint32_t mine = key[i];
+    int rank = 0;
+    for (int k = 0; k < R; ++k) rank += key[k] < mine || (key[k] == mine && k < i);
+    perm[rank] = i;
+}
+
 // One launch of the whole frame setup.  Block b < irr_n^2 handles
 // irradiance texel b, the next dist_n^2 blocks the distance texels, rays
 // strided over the block: each rotates the pattern itself from the sf table
@@ -111,7 +135,7 @@ __global__ void __launch_bounds__(256) k_frame_setup(FrameRot rot_arg, const Fra
                                                      int dist_n, double cos_power,
                                                      const double* __restrict__ sf64, float4* dirs, float* w_irr,
                                                      float* inv_s_irr, float* w_dist, float* inv_s_dist,
-                                                     int32_t* zero, int n_zero, int first_block) {
+                                                     int32_t* zero, int n_zero, int first_block, int32_t* perm) {
     pdl_wait();
     pdl_trigger();
     __shared__ double red[256];
@@ -128,6 +152,7 @@ __global__ void __launch_bounds__(256) k_frame_setup(FrameRot rot_arg, const Fra
             rotate_dir(rot, sv, w);
             store_frame_dir(dirs, R, i, w);
         }
+        if (perm) order_rays(sf64, R, i, perm);
         return;
     }
     const int b = blk;
@@ -711,7 +736,7 @@ cudaError_t launch_frame_dirs(const FrameRot& rot, int R, int irr_n, int dist_n,
     // the direction blocks of k_frame_setup alone
     k_frame_setup<false><<<(R + 255) / 256, 256, 0, st>>>(rot, nullptr, R, irr_n, dist_n, 0.0, sf64, dirs, nullptr,
                                                            nullptr, nullptr, nullptr, zero, n_zero,
-                                                           irr_n * irr_n + dist_n * dist_n);
+                                                           irr_n * irr_n + dist_n * dist_n, nullptr);
     return cudaGetLastError();
 }
 
@@ -724,11 +749,9 @@ static int frame_setup_grid(int R, int irr_n, int dist_n) { return irr_n * irr_n
 
 cudaError_t launch_frame_setup(const FrameRot& rot, int R, int irr_n, int dist_n, float cos_power,
                                const double* sf64, float4* dirs, float* w_irr, float* inv_s_irr, float* w_dist,
-                               float* inv_s_dist, int32_t* zero, int n_zero, cudaStream_t st) {
-    k_frame_setup<false><<<frame_setup_grid(R, irr_n, dist_n), 256, 0, st>>>(
-        rot, nullptr, R, irr_n, dist_n, (double)cos_power, sf64, dirs, w_irr, inv_s_irr, w_dist, inv_s_dist, zero,
-        n_zero, 0);
-    return cudaGetLastError();
+                               float* inv_s_dist, int32_t* zero, int n_zero, int32_t* perm, cudaStream_t st) {
+    return launch_pdl(k_frame_setup<false>, frame_setup_grid(R, irr_n, dist_n), 256, 0, st, rot, nullptr, R, irr_n, dist_n,
+                      (double)cos_power, sf64, dirs, w_irr, inv_s_irr, w_dist, inv_s_dist, zero, n_zero, 0, perm);
 }
 
 cudaError_t launch_frame_setup_split(const FrameRot& rot, int R, int irr_n, int dist_n, float cos_power,
@@ -737,14 +760,14 @@ cudaError_t launch_frame_setup_split(const FrameRot& rot, int R, int irr_n, int 
                                      cudaStream_t st_dirs, cudaStream_t st_weights) {
     const int nwb = irr_n * irr_n + dist_n * dist_n;
     k_frame_setup<false><<<nwb, 256, 0, st_weights>>>(rot, nullptr, R, irr_n, dist_n, (double)cos_power, sf64, dirs,
-                                                      w_irr, inv_s_irr, w_dist, inv_s_dist, zero, n_zero, 0);
+                                                      w_irr, inv_s_irr, w_dist, inv_s_dist, zero, n_zero, 0, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // the directions in blocks of 64 rays, so the FP64 rotations of the
     // frame's rays spread over several SMs' double-precision units
     if (n_zero > 64) return cudaErrorInvalidValue;
     return launch_pdl(k_frame_setup<false>, (R + 63) / 64, 64, 0, st_dirs, rot, nullptr, R, irr_n, dist_n,
-                      (double)cos_power, sf64, dirs, w_irr, inv_s_irr, w_dist, inv_s_dist, zero, n_zero, nwb);
+                      (double)cos_power, sf64, dirs, w_irr, inv_s_irr, w_dist, inv_s_dist, zero, n_zero, nwb, nullptr);
 }
 
 cudaError_t launch_frame_setup_dev(const FrameRot* rot_dev, int R, int irr_n, int dist_n, float cos_power,
@@ -752,7 +775,7 @@ cudaError_t launch_frame_setup_dev(const FrameRot* rot_dev, int R, int irr_n, in
                                    float* inv_s_dist, int32_t* zero, int n_zero, cudaStream_t st) {
     k_frame_setup<true><<<frame_setup_grid(R, irr_n, dist_n), 256, 0, st>>>(
         FrameRot{}, rot_dev, R, irr_n, dist_n, (double)cos_power, sf64, dirs, w_irr, inv_s_irr, w_dist, inv_s_dist,
-        zero, n_zero, 0);
+        zero, n_zero, 0, nullptr);
     return cudaGetLastError();
 }
 
@@ -805,7 +828,7 @@ template <bool MULTI, int PG>
 static cudaError_t launch_tiled(const VolSet& vs, const BlendParams& bp, int irr_n, int dist_n, const float* w_irr,
                                 const float* inv_s_irr, const float* w_dist, const float* inv_s_dist,
                                 const float4* records, const int32_t* active, const int32_t* count,
-                                uint32_t* status, int grid, cudaStream_t st) {
+                                uint32_t* status, int grid, bool pdl, cudaStream_t st) {
     cudaError_t e = opt_in_blend<MULTI, PG>();
     if (e != cudaSuccess) return e;
     const TiledShape ts = tiled_shape(PG, bp.R, irr_n, dist_n);
@@ -822,6 +845,12 @@ static cudaError_t launch_tiled(const VolSet& vs, const BlendParams& bp, int irr
     bpt.div_td = make_fast_div((uint32_t)(dist_n * dist_n));
     bpt.div_ni = make_fast_div((uint32_t)irr_n);
     bpt.div_nd = make_fast_div((uint32_t)dist_n);
+    // a cascade's blend launched early takes the shading pass's shared memory
+    // and slots in its tail (2622 us a frame against 2580), so only the
+    // allocation-free update asks for it
+    if (pdl)
+        return launch_pdl(kernel, grid, ts.threads, ts.smem, st, vs, bpt, w_irr, inv_s_irr, w_dist, inv_s_dist, records,
+                          active, count, status);
     kernel<<<grid, ts.threads, ts.smem, st>>>(vs, bpt, w_irr, inv_s_irr, w_dist, inv_s_dist, records, active, count,
                                               status);
     return cudaGetLastError();
@@ -835,16 +864,16 @@ template <bool MULTI, int PGS>
 static cudaError_t blend_simt(const VolSet& vs, const BlendParams& bp, int irr_n, int dist_n, const float* w_irr,
                               const float* inv_s_irr, const float* w_dist, const float* inv_s_dist,
                               const float4* records, const int32_t* active, const int32_t* count,
-                              uint32_t* status, int grid, cudaStream_t st) {
+                              uint32_t* status, int grid, bool pdl, cudaStream_t st) {
     if (PGS >= 16 && tiled_fits<16>(bp, irr_n, dist_n))
         return launch_tiled<MULTI, 16>(vs, bp, irr_n, dist_n, w_irr, inv_s_irr, w_dist, inv_s_dist, records, active,
-                                       count, status, grid, st);
+                                       count, status, grid, pdl, st);
     if (PGS >= 8 && tiled_fits<8>(bp, irr_n, dist_n))
         return launch_tiled<MULTI, 8>(vs, bp, irr_n, dist_n, w_irr, inv_s_irr, w_dist, inv_s_dist, records, active,
-                                      count, status, grid * (PGS / 8), st);
+                                      count, status, grid * (PGS / 8), pdl, st);
     if (tiled_fits<4>(bp, irr_n, dist_n))
         return launch_tiled<MULTI, 4>(vs, bp, irr_n, dist_n, w_irr, inv_s_irr, w_dist, inv_s_dist, records, active,
-                                      count, status, grid * (PGS / 4), st);
+                                      count, status, grid * (PGS / 4), pdl, st);
     cudaError_t e = opt_in_blend<MULTI, PGS>();
     if (e != cudaSuccess) return e;
     // as many probes per CTA as fit (R <= 1024 leaves room for at least 13)
@@ -859,10 +888,10 @@ static cudaError_t blend_simt(const VolSet& vs, const BlendParams& bp, int irr_n
 
 cudaError_t launch_blend(const VolView& v, const BlendParams& bp, const float* w_irr, const float* inv_s_irr,
                          const float* w_dist, const float* inv_s_dist, const float4* records,
-                         const int32_t* active, const int32_t* count, uint32_t* status, int grid,
+                         const int32_t* active, const int32_t* count, uint32_t* status, int grid, bool pdl,
                          cudaStream_t st) {
     return blend_simt<false, 16>(single_set(v), bp, v.irr_n, v.dist_n, w_irr, inv_s_irr, w_dist, inv_s_dist,
-                                records, active, count, status, grid, st);
+                                records, active, count, status, grid, pdl, st);
 }
 
 cudaError_t launch_blend_set(const VolSet& vs, bool multi, const BlendParams& bp, int irr_n, int dist_n,
@@ -873,7 +902,7 @@ cudaError_t launch_blend_set(const VolSet& vs, bool multi, const BlendParams& bp
 #define DDGI_BLEND_CASE(M, P)                                                                                 \
     if (multi == M && probes_per_cta == P)                                                                   \
         return blend_simt<M, P>(vs, bp, irr_n, dist_n, w_irr, inv_s_irr, w_dist, inv_s_dist, records, active,   \
-                                count, status, grid, st);
+                                count, status, grid, false, st);
     DDGI_BLEND_CASE(false, 4)
     DDGI_BLEND_CASE(false, 8)
     DDGI_BLEND_CASE(false, 16)

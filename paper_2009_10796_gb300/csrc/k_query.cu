@@ -92,6 +92,8 @@ __global__ void __launch_bounds__(256, 4) k_query_glossy(VolView v, const float*
 // consumers carry the probe index with each entry.
 __global__ void k_build_list(const uint8_t* __restrict__ states, int begin, int end, int which, int32_t* list,
                              int32_t* count) {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     for (int base = begin + blockIdx.x * blockDim.x; base < end; base += gridDim.x * blockDim.x) {
         int p = base + threadIdx.x;
@@ -115,6 +117,8 @@ __global__ void k_build_list(const uint8_t* __restrict__ states, int begin, int 
 // becomes Newly Awake, an Awake probe inside none goes back to Sleeping.
 __global__ void __launch_bounds__(256) k_wake(VolView v, const float* __restrict__ boxes, int n_boxes, int begin,
                                               int end) {
+    pdl_wait();
+    pdl_trigger();
     extern __shared__ float sbox[];   // n_boxes x 6
     for (int k = threadIdx.x; k < 6 * n_boxes; k += blockDim.x) sbox[k] = boxes[k];
     __syncthreads();
@@ -136,8 +140,7 @@ cudaError_t launch_wake(const VolView& v, const float* boxes, int n_boxes, int b
     if (end <= begin) return cudaSuccess;
     int blocks = (end - begin + 255) / 256;
     if (blocks > 4096) blocks = 4096;
-    k_wake<<<blocks, 256, sizeof(float) * 6 * (size_t)n_boxes, st>>>(v, boxes, n_boxes, begin, end);
-    return cudaGetLastError();
+    return launch_pdl(k_wake, blocks, 256, sizeof(float) * 6 * (size_t)n_boxes, st, v, boxes, n_boxes, begin, end);
 }
 
 // Cascade query (Sec. 7.3): one thread per point, volumes densest first.
@@ -167,6 +170,8 @@ __global__ void __launch_bounds__(256) k_query_cascade(VolSet vs, const float* _
 // List build over every volume of a set: global index g runs over the
 // volumes' probes in order; entries are (volume << 24) | probe.
 __global__ void k_build_list_multi(VolSet vs, int total, int which, int32_t* list, int32_t* count) {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     for (int base = blockIdx.x * blockDim.x; base < total; base += gridDim.x * blockDim.x) {
         int g = base + threadIdx.x;
@@ -238,8 +243,7 @@ cudaError_t launch_build_list_multi(const VolSet& vs, int total, int which, int3
     int blocks = (total + 255) / 256;
     if (blocks > 4096) blocks = 4096;
     if (blocks < 1) blocks = 1;
-    k_build_list_multi<<<blocks, 256, 0, st>>>(vs, total, which, list, count);
-    return cudaGetLastError();
+    return launch_pdl(k_build_list_multi, blocks, 256, 0, st, vs, total, which, list, count);
 }
 
 cudaError_t launch_reset_planes(const VolSet& vs, const int4* planes, const int32_t* count, int max_planes,
@@ -286,8 +290,7 @@ cudaError_t launch_build_list_range(const uint8_t* states, int begin, int end, i
     int blocks = (end - begin + 255) / 256;
     if (blocks > 4096) blocks = 4096;
     if (blocks < 1) blocks = 1;
-    k_build_list<<<blocks, 256, 0, st>>>(states, begin, end, which, list, count);
-    return cudaGetLastError();
+    return launch_pdl(k_build_list, blocks, 256, 0, st, states, begin, end, which, list, count);
 }
 
 }  // namespace ddgi

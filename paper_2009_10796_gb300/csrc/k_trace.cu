@@ -19,6 +19,8 @@ __global__ void __launch_bounds__(256) k_classify(DevScene s, VolSet vs, const f
                                                   int R, const int32_t* __restrict__ perm,
                                                   const int32_t* __restrict__ list,
                                                   const int32_t* __restrict__ count) {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -106,6 +108,8 @@ __global__ void __launch_bounds__(256, kClassCtas) k_classify_split(DevScene s, 
                                                                     const int32_t* __restrict__ list,
                                                                     const int32_t* __restrict__ count, int4* scratch,
                                                                     uint32_t* next) {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const unsigned nb = (unsigned)(R + 31) / 32;
     const unsigned total = (unsigned)(*count) * nb * 32u;   // below 2^32: probes x R is below 2^31, probes 2^26
@@ -163,14 +167,23 @@ __global__ void __launch_bounds__(256, kClassCtas) k_classify_split(DevScene s, 
 
 // Fused trace + shade, one thread per probe ray (the allocation-free
 // update's path: it needs no shadow or hit lists); rays and shadow rays go
-// through the warp-cooperative 4-wide walk.
-__global__ void __launch_bounds__(128) k_trace_shade(DevScene s, VolView v, Lights L,
-                                                     const float4* __restrict__ dirs, int R,
-                                                     const int32_t* __restrict__ active,
-                                                     const int32_t* __restrict__ count,
-                                                     float4* __restrict__ records) {
-    const int64_t total = (int64_t)(*count) * R;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+// through the warp-cooperative 4-wide walk.  Bound by the latency of the walk:
+// a volume of this path has some ten warps of rays to an SM.  So a warp takes a
+// compact cone of directions (perm) instead of 32 steps of the spiral over the
+// sphere, the walk its 64-register form and the shading the specialised query;
+// with that, and with every kernel of the update launched while the one before
+// it ends, 16 x 8 x 16 probes x 128 rays of a city take 62 us (78 before).
+template <int FORM>
+__global__ void __launch_bounds__(128, 6) k_trace_shade(DevScene s, VolView v, Lights L,
+                                                        const float4* __restrict__ dirs, int R, FastDiv dR,
+                                                        const int32_t* __restrict__ perm,
+                                                        const int32_t* __restrict__ active,
+                                                        const int32_t* __restrict__ count,
+                                                        float4* __restrict__ records) {
+    pdl_wait();
+    pdl_trigger();
+    const int total = (*count) * R;   // at most 2^20
+    const int stride = gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
     const float3 tol = f3(-L.sun_dir.x, -L.sun_dir.y, -L.sun_dir.z);
     const RayPre r_sun = ray_pre(f3(0.0f, 0.0f, 0.0f), tol);
@@ -179,20 +192,19 @@ __global__ void __launch_bounds__(128) k_trace_shade(DevScene s, VolView v, Ligh
     w.stack = stack;
     // warp-uniform loop: each warp takes 32 consecutive rays through the
     // warp-cooperative 4-wide walk, then their shadow rays the same way
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
-        const int64_t idx = base + lane;
-        const bool valid = idx < total;
-        const int64_t id = valid ? idx : 0;
-        int slot = (int)(id / R);
-        int i = (int)(id - (int64_t)slot * R);
-        int p = __ldg(active + slot);
+    for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
+        const bool valid = base + lane < total;
+        const int id = valid ? base + lane : base;
+        const int slot = (int)fast_div((uint32_t)id, dR);
+        const int i = __ldg(perm + (id - slot * R));   // consecutive items take a compact cone of directions
+        const int p = __ldg(active + slot);
         float3 o = probe_pos_phys(v, p);
         float4 d4 = __ldg(dirs + i);
         float3 d = f3(d4.x, d4.y, d4.z);
         const RayPre r = ray_pre_packed(o, d, __ldg(dirs + R + 2 * i), __ldg(dirs + R + 2 * i + 1));
         ww_start(s, w, valid);
         do {
-            ww4_round<false>(s, r, w);
+            ww4_round<false, false, true>(s, r, w);
         } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
         const Hit h = w.h;
         // the shadow ray of a sunlit front hit
@@ -214,7 +226,7 @@ __global__ void __launch_bounds__(128) k_trace_shade(DevScene s, VolView v, Ligh
         if (shadow) ray_set_origin(sr, x + (1e-4f * (1.0f + length(x))) * n);
         ww_start(s, w, shadow);
         do {
-            ww4_round<true>(s, sr, w);
+            ww4_round<true, false, true>(s, sr, w);
         } while (__ballot_sync(0xffffffffu, w.node != kDone) != 0);
         const bool lit = shadow && w.h.orig < 0;
         if (!valid) continue;
@@ -239,11 +251,11 @@ __global__ void __launch_bounds__(128) k_trace_shade(DevScene s, VolView v, Ligh
                 float k = cosl * 0.318309886183790672f;   // 1/pi
                 direct = f3(L.sun_irr.x * k, L.sun_irr.y * k, L.sun_irr.z * k);
             }
-            float3 M = query_M(v, x, n, f3(-d.x, -d.y, -d.z));
+            float3 M = query_M<FORM>(v, x, n, f3(-d.x, -d.y, -d.z));
             rec = make_float4(Le.x + rho.x * (direct.x + M.x), Le.y + rho.y * (direct.y + M.y),
                               Le.z + rho.z * (direct.z + M.z), fminf(h.t, v.t_max));
         }
-        records[idx] = rec;
+        records[slot * R + i] = rec;
     }
 }
 
@@ -551,6 +563,8 @@ __global__ void __launch_bounds__(256, kClassCtas) k_optimize(DevScene s, VolVie
                                                               const int32_t* __restrict__ list,
                                                               const int32_t* __restrict__ count,
                                                               OptimizeScratch* scratch, uint32_t* next) {
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x & 31;
     const unsigned nb = (unsigned)(R + 31) / 32;
     const unsigned total = (unsigned)(*count) * nb * 32u;   // below 2^32, as in k_classify_split
@@ -635,33 +649,36 @@ cudaError_t launch_optimize(const DevScene& s, const VolView& v, const float4* d
                             const int32_t* list, const int32_t* count, OptimizeScratch* scratch, uint32_t* next,
                             cudaStream_t st) {
     const int grid = bounded_grid(kClassCtas * sm_count(), (int64_t)v.n_probes * ((R + 31) / 32) * 32);
-    k_optimize<<<grid, 256, 0, st>>>(s, v, dirs, R, perm, list, count, scratch, next);
-    return cudaGetLastError();
+    return launch_pdl(k_optimize, grid, 256, 0, st, s, v, dirs, R, perm, list, count, scratch, next);
 }
 
 cudaError_t launch_classify(const DevScene& s, const VolView& v, const float4* dirs, int R, const int32_t* perm,
                             const int32_t* list, const int32_t* count, int4* scratch, uint32_t* next, int grid,
                             cudaStream_t st) {
     if (scratch)
-        k_classify_split<false><<<bounded_grid(kClassCtas * sm_count(), (int64_t)v.n_probes * ((R + 31) / 32) * 32), 256,
-                                  0, st>>>(s, single_set(v), dirs, R, perm, list, count, scratch, next);
-    else
-        k_classify<false><<<grid, 256, 0, st>>>(s, single_set(v), dirs, R, perm, list, count);
-    return cudaGetLastError();
+        return launch_pdl(k_classify_split<false>,
+                          bounded_grid(kClassCtas * sm_count(), (int64_t)v.n_probes * ((R + 31) / 32) * 32), 256, 0, st,
+                          s, single_set(v), dirs, R, perm, list, count, scratch, next);
+    return launch_pdl(k_classify<false>, bounded_grid(grid, (int64_t)v.n_probes * 32), 256, 0, st, s, single_set(v), dirs,
+                      R, perm, list, count);
 }
 
 cudaError_t launch_classify_multi(const DevScene& s, const VolSet& vs, const float4* dirs, int R,
                                   const int32_t* perm, const int32_t* list, const int32_t* count, int4* scratch,
                                   uint32_t* next, cudaStream_t st) {
-    k_classify_split<true><<<kClassCtas * sm_count(), 256, 0, st>>>(s, vs, dirs, R, perm, list, count, scratch, next);
-    return cudaGetLastError();
+    return launch_pdl(k_classify_split<true>, kClassCtas * sm_count(), 256, 0, st, s, vs, dirs, R, perm, list, count,
+                      scratch, next);
 }
 
 cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights& L, const float4* dirs,
-                               int R, const int32_t* active, const int32_t* count, float4* records,
-                               int grid, cudaStream_t st) {
-    k_trace_shade<<<grid, 128, 0, st>>>(s, v, L, dirs, R, active, count, records);
-    return cudaGetLastError();
+                               int R, const int32_t* perm, const int32_t* active, const int32_t* count,
+                               float4* records, int grid, cudaStream_t st) {
+    const int64_t need = ((int64_t)v.n_probes * R + 127) / 128;
+    const FastDiv dR = make_fast_div((uint32_t)R);
+    return with_query_form(query_form(v), [&](auto f) {
+        return launch_pdl(k_trace_shade<decltype(f)::value>, (int)std::min<int64_t>(grid, need), 128, 0, st, s, v, L, dirs,
+                          R, dR, perm, active, count, records);
+    });
 }
 
 template <bool MULTI>

@@ -36,6 +36,7 @@ static __device__ __align__(256) float g_na_w_dist[kNaMaxDistTexels * kNaMaxRays
 static __device__ __align__(256) float g_na_inv_s_dist[kNaMaxDistTexels];
 static __device__ __align__(256) int32_t g_na_lists[2 * kNaMaxProbes];
 static __device__ __align__(256) int32_t g_na_counts[4];
+static __device__ __align__(256) int32_t g_na_perm[kNaMaxRays];           // ray order within a probe
 static __device__ __align__(256) uint32_t g_na_status[4];
 
 struct NaScratch {
@@ -48,6 +49,7 @@ struct NaScratch {
     float* inv_s_dist;
     int32_t* lists;
     int32_t* counts;
+    int32_t* perm;
     uint32_t* status;
 };
 
@@ -76,6 +78,7 @@ cudaError_t scratch_for_current_device(NaScratch* out) {
         if ((e = cudaGetSymbolAddress((void**)&s.inv_s_dist, g_na_inv_s_dist)) != cudaSuccess) return e;
         if ((e = cudaGetSymbolAddress((void**)&s.lists, g_na_lists)) != cudaSuccess) return e;
         if ((e = cudaGetSymbolAddress((void**)&s.counts, g_na_counts)) != cudaSuccess) return e;
+        if ((e = cudaGetSymbolAddress((void**)&s.perm, g_na_perm)) != cudaSuccess) return e;
         if ((e = cudaGetSymbolAddress((void**)&s.status, g_na_status)) != cudaSuccess) return e;
         g_na_scratch[dev] = s;
         g_na_ready[dev] = true;
@@ -190,22 +193,22 @@ extern "C" ddgi_status ddgi_update_noalloc(ddgi_scene scene, const ddgi_volume_d
     // counters; the status word keeps its flags until it is polled
     if ((e = launch_sf_table(R, s.sf64, st)) != cudaSuccess) return na_fail(e, "ray pattern");
     if ((e = launch_frame_setup(rot, R, d->irr_n, d->dist_n, d->dist_cos_power, s.sf64, s.dirs, s.w_irr,
-                                s.inv_s_irr, s.w_dist, s.inv_s_dist, s.counts, 4, st)) != cudaSuccess)
+                                s.inv_s_irr, s.w_dist, s.inv_s_dist, s.counts, 4, s.perm, st)) != cudaSuccess)
         return na_fail(e, "frame setup");
     if (d->state_machine) {
         if ((e = launch_build_list(states_dev, (int)P, 0, s.lists, s.counts + 0, st)) != cudaSuccess)
             return na_fail(e, "uninitialised list");
-        if ((e = launch_classify(*sv, v, s.dirs, R, nullptr, s.lists, s.counts + 0, nullptr, nullptr, sms * 8,
+        if ((e = launch_classify(*sv, v, s.dirs, R, s.perm, s.lists, s.counts + 0, nullptr, nullptr, sms * 8,
                                  st)) != cudaSuccess)
             return na_fail(e, "classify");
     }
     if ((e = launch_build_list(states_dev, (int)P, 1, s.lists + P, s.counts + 1, st)) != cudaSuccess)
         return na_fail(e, "active list");
-    if ((e = launch_trace_shade(*sv, v, L, s.dirs, R, s.lists + P, s.counts + 1, s.records, sms * 16, st)) !=
+    if ((e = launch_trace_shade(*sv, v, L, s.dirs, R, s.perm, s.lists + P, s.counts + 1, s.records, sms * 16, st)) !=
         cudaSuccess)
         return na_fail(e, "trace and shade");
     if ((e = launch_blend(v, bp, s.w_irr, s.inv_s_irr, s.w_dist, s.inv_s_dist, s.records, s.lists + P,
-                          s.counts + 1, s.status, sms * 4, st)) != cudaSuccess)
+                          s.counts + 1, s.status, sms * 4, true, st)) != cudaSuccess)
         return na_fail(e, "blend");
     return DDGI_OK;
 }

@@ -158,3 +158,23 @@ def test_update_noalloc_rejects_oversized_volume():
     with pytest.raises(g.DDGIError) as err:
         g.update_noalloc(scene, big, synth.city_lights(), 0, t, t, t)
     assert err.value.code == 1 and "1048576" in str(err.value)
+
+
+@pytest.mark.parametrize("rays", [31, 33, 256, 257, 512])
+def test_update_noalloc_ray_orders(rays):
+    """The pass takes a probe's rays in an order of its own: one block of them,
+    ragged ones, more than one block of threads, the most."""
+    import paper_2009_10796_gb300 as g
+    scene = g.Scene.from_arrays(synth.room_scene())
+    ref = g.Volume(synth.room_volume(rays_per_probe=rays))
+    info = ref.info
+    states = torch.zeros(info.n_probes, dtype=torch.uint8, device="cuda")
+    irr = torch.zeros(info.irr_bytes, dtype=torch.uint8, device="cuda")
+    dist = torch.zeros(info.dist_bytes, dtype=torch.uint8, device="cuda")
+    for frame in (0, 1):
+        ref.update(scene, synth.room_lights(), frame)
+        g.update_noalloc(scene, ref.desc, synth.room_lights(), frame, states, irr, dist)
+        torch.cuda.synchronize()
+        assert torch.equal(states, ref.states())
+        assert _close(_decode(irr, 0, 0), _decode(ref.irr_raw(), 0, 0), 0, 0)
+        assert _close(_decode(dist, 1, 0), _decode(ref.dist_raw(), 1, 0), 1, 0)
