@@ -1617,8 +1617,8 @@ cudaError_t launch_border_fold(float* g_irr, int P, int n, cudaStream_t st);
 cudaError_t launch_blend_adjoint(const VolView& v_after, const float* w_irr, const float* inv_s, const float* g_irr,
                                  int P, int R, float4* gL, cudaStream_t st);
 cudaError_t launch_shade_adjoint(const DevScene& s, const VolView& v_before, const Lights& L, const float4* dirs,
-                                 int P, int R, const float4* gL, float* d_emit, float* d_albedo, float* g_prev,
-                                 int with_prev, cudaStream_t st);
+                                 int P, int R, const int32_t* perm, const float4* gL, float* d_emit,
+                                 float* d_albedo, float* g_prev, int with_prev, cudaStream_t st);
 cudaError_t launch_set_materials(float4* albedo, int n_obj, const float* alb, float4* emit, int n_em, const float* em,
                                  cudaStream_t st);
 }  // namespace ddgi
@@ -1717,8 +1717,8 @@ ddgi_status ddgi_diff_backward(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
                                    v->inv_s_irr, v->w_dist, v->inv_s_dist, nullptr, 0, nullptr, st));
         DDGI_CK(launch_blend_adjoint(snap_view(f + 1), v->w_irr, v->inv_s_irr, g, (int)v->P, v->R, v->records, st));
         DDGI_CK(cudaMemsetAsync(gp, 0, gbytes, st));
-        DDGI_CK(launch_shade_adjoint(s->dev, snap_view(f), L, v->dirs, (int)v->P, v->R, v->records, d_emit_dev,
-                                     d_albedo_dev, gp, f > 0, st));
+        DDGI_CK(launch_shade_adjoint(s->dev, snap_view(f), L, v->dirs, (int)v->P, v->R, v->perm, v->records,
+                                     d_emit_dev, d_albedo_dev, gp, f > 0, st));
         float* t = g;
         g = gp;
         gp = t;

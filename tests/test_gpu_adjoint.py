@@ -238,3 +238,30 @@ def test_blend_adjoint_tiles(g, irr_n, counts, rays):
     (E * to_dev(G)).sum().backward()
     assert rel_err(albedo.grad.cpu().numpy(), g_al_ref).max() <= 1e-3
     assert rel_err(emit.grad.cpu().numpy(), g_em_ref).max() <= 1e-3
+
+
+@pytest.mark.parametrize("rays", [33, 64])
+def test_material_gradients_of_many_objects(g, rays):
+    """Gradients of hits on the same material are summed in a warp before they
+    are added: a scene with every triangle an object and an emitter of its own
+    (more of them in a warp than are summed there) against the same scene as
+    one object and one emitter, whose gradients are the sums.  Every term is
+    positive and each side a sum of at most 2^17 of them in FP32: 1e-4."""
+    import dataclasses
+    sc = synth.room_scene()
+    T = sc.n_tris
+    grads = []
+    for k in (T, 1):
+        ids = (np.arange(T) % k).astype(np.int32)
+        S = g.Scene.from_arrays(dataclasses.replace(
+            sc, tri_object=ids, object_albedo=np.full((k, 3), 0.5), object_flags=np.ones(k, np.int32),
+            tri_emitter=ids, emitter_radiance=np.full((k, 3), 1.5)))
+        V = g.Volume(synth.room_volume(rays_per_probe=rays, gamma=1.0, state_machine=0))
+        albedo = torch.full((k, 3), 0.5, device="cuda", requires_grad=True)
+        emit = torch.full((k, 3), 1.5, device="cuda", requires_grad=True)
+        pos, nrm, cam = synth.room_queries()
+        E = g.IrradianceField.apply(albedo, emit, V, S, synth.room_lights(), to_dev(pos), to_dev(nrm), cam, 0, 2)
+        E.sum().backward()
+        grads.append((albedo.grad.double().sum(0), emit.grad.double().sum(0)))
+    for many, one in zip(*grads):
+        assert bool((one > 0).all()) and float(((many - one).abs() / one).max()) <= 1e-4
