@@ -153,6 +153,7 @@ struct ddgi_volume_s {
     double *rec64 = nullptr, *g64 = nullptr, *g64_prev = nullptr, *gL64 = nullptr, *sw64 = nullptr;
     float* g_irr = nullptr;                // adjoint: texel gradients of two frames
     float* g_prev = nullptr;
+    int32_t* point_scratch = nullptr;      // adjoint: order of the query points (PointOrder)
     uint8_t* pack_w = nullptr;             // tensor-core blend: weight tiles in operand layout
     float* inv_irr_r = nullptr;            // 1 / sum of the rounded weights
     float* inv_dist_r = nullptr;
@@ -498,7 +499,7 @@ void ddgi_volume_destroy(ddgi_volume v) {
     cudaFree(v->shadow_list); cudaFree(v->hit_list); cudaFree(v->class_scratch); cudaFree(v->perm);
     for (void* p : v->snap_irr) cudaFree(p);
     for (void* p : v->snap_dist) cudaFree(p);
-    cudaFree(v->g_irr); cudaFree(v->g_prev);
+    cudaFree(v->g_irr); cudaFree(v->g_prev); cudaFree(v->point_scratch);
     cudaFree(v->pack_w); cudaFree(v->inv_irr_r); cudaFree(v->inv_dist_r);
     cudaFree(v->offsets); cudaFree(v->opt_dirs); cudaFree(v->opt_scratch); cudaFree(v->dyn_boxes);
     for (double* q : v->snap64_irr) cudaFree(q);
@@ -1612,7 +1613,7 @@ ddgi_status ddgi_cascade_autotune(ddgi_cascade c, ddgi_scene s, const ddgi_light
 
 namespace ddgi {
 cudaError_t launch_query_adjoint(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam,
-                                 const float* dE, float* g_irr, cudaStream_t st);
+                                 const float* dE, float* g_irr, int32_t* scratch, cudaStream_t st);
 cudaError_t launch_border_fold(float* g_irr, int P, int n, cudaStream_t st);
 cudaError_t launch_blend_adjoint(const VolView& v_after, const float* w_irr, const float* inv_s, const float* g_irr,
                                  int P, int R, float4* gL, cudaStream_t st);
@@ -1679,6 +1680,21 @@ ddgi_status ddgi_diff_forward(ddgi_volume v, ddgi_scene s, const ddgi_lights* li
     return ddgi_query(v, pos_dev, nrm_dev, n, camera_pos, out_dev, stream);
 }
 
+// Scratch for ordering n query points: allocated once for a volume, of one
+// size, so that a captured pass keeps its address; none (the points are taken
+// as they come) for few points, a capture before the first pass, or no memory.
+static int32_t* point_scratch(ddgi_volume_s* v, int64_t n, cudaStream_t st) {
+    if (n < 16 * v->P || 16 * v->P > kPointsOrdered) return nullptr;
+    if (v->point_scratch) return v->point_scratch;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return nullptr;
+    if (cudaMalloc((void**)&v->point_scratch, point_order_bytes(v->P)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        v->point_scratch = nullptr;
+    }
+    return v->point_scratch;
+}
+
 ddgi_status ddgi_diff_backward(ddgi_volume v, ddgi_scene s, const ddgi_lights* lights, int64_t first_frame,
                                int32_t n_frames, const float* pos_dev, const float* nrm_dev, int64_t n,
                                const float camera_pos[3], const float* dE_dev, float* d_albedo_dev,
@@ -1708,7 +1724,8 @@ ddgi_status ddgi_diff_backward(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
     };
     Lights L = make_lights(lights);
     float3 cam = make_float3(camera_pos[0], camera_pos[1], camera_pos[2]);
-    DDGI_CK(launch_query_adjoint(snap_view(n_frames), pos_dev, nrm_dev, n, cam, dE_dev, v->g_irr, st));
+    DDGI_CK(launch_query_adjoint(snap_view(n_frames), pos_dev, nrm_dev, n, cam, dE_dev, v->g_irr,
+                                 point_scratch(v, n, st), st));
     float* g = v->g_irr;
     float* gp = v->g_prev;
     for (int f = n_frames - 1; f >= 0; --f) {
@@ -1853,7 +1870,7 @@ ddgi_status ddgi_query_backward(ddgi_volume v, const float* pos_dev, const float
     if (n > 0)
         DDGI_CK(launch_query_adjoint(make_view(v), pos_dev, nrm_dev, n,
                                      make_float3(camera_pos[0], camera_pos[1], camera_pos[2]), dE_dev, g_irr_dev,
-                                     st));
+                                     nullptr, st));
     if (fold_borders) DDGI_CK(launch_border_fold(g_irr_dev, (int)v->P, d.irr_n, st));
     return DDGI_OK;
 }

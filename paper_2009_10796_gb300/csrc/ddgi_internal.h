@@ -411,4 +411,30 @@ ddgi_status set_error(ddgi_status s, const std::string& msg);
 // Device view of a registered scene (NULL for a NULL handle).
 const DevScene* scene_device_view(ddgi_scene s);
 
+// Scratch of the query adjoint's point order (k_adjoint.cu): bins by cage and
+// nearest axis of the normal, at most kPointsOrdered points at a time.
+constexpr int kPointBins = 6;            // to a cage
+constexpr int kPointsOrdered = 1 << 20;
+struct PointOrder {
+    int32_t* groups;   // [1] groups of equal bins over all warps; then, cleared with it,
+    int32_t* taken;    // [1] indices given to bins
+    int32_t* bins;     // [kPointBins n_probes] counts, then first indices
+    int32_t* bin;      // [kPointsOrdered] a point's bin,
+    int32_t* rank;     // its place among the bin's,
+    int32_t* order;    // and the points by bin
+};
+inline size_t point_order_bytes(int64_t n_probes) {
+    return sizeof(int32_t) * (2 + (size_t)kPointBins * (size_t)n_probes + 3 * (size_t)kPointsOrdered);
+}
+inline PointOrder point_order(int32_t* scratch, int64_t n_probes) {
+    PointOrder o;
+    o.groups = scratch;
+    o.taken = scratch + 1;
+    o.bins = scratch + 2;
+    o.bin = o.bins + (size_t)kPointBins * (size_t)n_probes;
+    o.rank = o.bin + kPointsOrdered;
+    o.order = o.rank + kPointsOrdered;
+    return o;
+}
+
 }  // namespace ddgi

@@ -210,24 +210,100 @@ __device__ __forceinline__ void query_M_adjoint_warp(const VolView& v, bool vali
     }
 }
 
+__device__ __forceinline__ float3 direction_to(float3 cam, float3 x, float3 n) {
+    const float3 wo = cam - x;
+    const float l = length(wo);
+    return l < 1e-6f ? n : (1.0f / l) * wo;
+}
+
+// ---- order of scattered points ---------------------------------------------
+// A warp of query_M_adjoint_warp wants points of few cages and footprints.
+// Points in random order (a training step's samples of the surfaces) are put
+// into bins by cage and by the axis that their normal is nearest to: a count
+// of each bin, ranges given to the bins in any order, the points' indices in
+// their ranges.  1 M points on the boxes of a room, 2048 probes: 338 us
+// unordered, 178 us ordered, the three passes included.  Points that neighbour
+// each other already (a G-buffer) are found so by the first pass, and the
+// others leave at once.
+__device__ __forceinline__ bool points_scattered(const PointOrder& o, int n) {
+    return *o.groups > kAdjMaxGroups / 2 * ((n + 31) / 32);
+}
+
+__global__ void __launch_bounds__(256) k_point_bins(VolView v, const float* __restrict__ pos,
+                                                    const float* __restrict__ nrm, int n, float3 cam, PointOrder o) {
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    int bin = -1;
+    if (q < n) {
+        const float3 x = f3(pos[3 * q], pos[3 * q + 1], pos[3 * q + 2]);
+        const float3 m = f3(nrm[3 * q], nrm[3 * q + 1], nrm[3 * q + 2]);
+        const Cage k = cage_of(v, local_point(v, x, m, direction_to(cam, x, m)));
+        const float ax = fabsf(m.x), ay = fabsf(m.y), az = fabsf(m.z);
+        const int axis = ax >= ay && ax >= az ? 0 : ay >= az ? 1 : 2;
+        const float along = axis == 0 ? m.x : axis == 1 ? m.y : m.z;
+        const int cell = max(k.base[0], 0) + v.counts.x * (max(k.base[1], 0) + v.counts.y * max(k.base[2], 0));
+        bin = kPointBins * cell + 2 * axis + (along < 0.0f ? 1 : 0);   // cell < probes
+    }
+    const unsigned same = __match_any_sync(0xffffffffu, bin);
+    const int leader = __ffs(same) - 1;
+    int first = 0;
+    if (bin >= 0 && lane == leader) first = atomicAdd(o.bins + bin, __popc(same));
+    first = __shfl_sync(0xffffffffu, first, leader);
+    if (q < n) {
+        o.bin[q] = bin;
+        o.rank[q] = first + __popc(same & ((1u << lane) - 1u));
+    }
+    const int groups = __syncthreads_count(bin >= 0 && lane == leader);
+    if (threadIdx.x == 0) atomicAdd(o.groups, groups);
+}
+
+// Counts -> first indices: a block takes one range for its 256 bins.
+__global__ void __launch_bounds__(256) k_point_ranges(int n_bins, int n, PointOrder o) {
+    pdl_wait();
+    pdl_trigger();
+    if (!points_scattered(o, n)) return;
+    const int b = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const int count = b < n_bins ? o.bins[b] : 0;
+    int end = count;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int below = __shfl_up_sync(0xffffffffu, end, d);
+        if (lane >= d) end += below;
+    }
+    int first = 0;
+    if (lane == 31) first = atomicAdd(o.taken, end);
+    first = __shfl_sync(0xffffffffu, first, 31);
+    if (b < n_bins) o.bins[b] = first + end - count;
+}
+
+__global__ void __launch_bounds__(256) k_point_order(int n, PointOrder o) {
+    pdl_wait();
+    pdl_trigger();
+    if (!points_scattered(o, n)) return;
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < n) o.order[o.bins[o.bin[q]] + o.rank[q]] = q;
+}
+
 template <int FORM>
 __global__ void __launch_bounds__(32 * kAdjWarps) k_query_adjoint(VolView v, const float* __restrict__ pos,
                                                                   const float* __restrict__ nrm, int64_t n, float3 cam,
-                                                                  const float* __restrict__ dE, float* g_irr) {
+                                                                  const float* __restrict__ dE, float* g_irr,
+                                                                  PointOrder o) {
+    pdl_wait();
     __shared__ AdjointScratch sh[kAdjWarps];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const bool ordered = o.order && points_scattered(o, (int)n);
     // warp-uniform loop: 32 consecutive points per warp
     for (int64_t q0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); q0 < n; q0 += stride) {
-        const int64_t q = q0 + (threadIdx.x & 31);
+        int64_t q = q0 + (threadIdx.x & 31);
         float3 x = f3(0.0f, 0.0f, 0.0f), nn = x, wo = x, dM = x;
         bool valid = q < n;
         if (valid) {
+            if (ordered) q = o.order[q];
             x = f3(pos[3 * q], pos[3 * q + 1], pos[3 * q + 2]);
             nn = f3(nrm[3 * q], nrm[3 * q + 1], nrm[3 * q + 2]);
             valid = nn.x != 0.0f || nn.y != 0.0f || nn.z != 0.0f;
-            wo = cam - x;
-            const float l = length(wo);
-            wo = l < 1e-6f ? nn : (1.0f / l) * wo;
+            wo = direction_to(cam, x, nn);
             const float pi = 3.14159265358979323846f;
             dM = f3(pi * dE[3 * q], pi * dE[3 * q + 1], pi * dE[3 * q + 2]);
         }
@@ -455,14 +531,43 @@ static int grid_for(int64_t n, int block) {
     return (int)(b < 1 ? 1 : (b > 65535 ? 65535 : b));
 }
 
-cudaError_t launch_query_adjoint(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam,
-                                 const float* dE, float* g_irr, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
+static cudaError_t query_adjoint(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam,
+                                 const float* dE, float* g_irr, const PointOrder& o, cudaStream_t st) {
     return with_query_form(query_form(v), [&](auto f) {
-        k_query_adjoint<decltype(f)::value><<<grid_for(n, 32 * kAdjWarps), 32 * kAdjWarps, 0, st>>>(v, pos, nrm, n, cam,
-                                                                                                   dE, g_irr);
-        return cudaGetLastError();
+        return launch_pdl(k_query_adjoint<decltype(f)::value>, grid_for(n, 32 * kAdjWarps), 32 * kAdjWarps, 0, st, v, pos,
+                          nrm, n, cam, dE, g_irr, o);
     });
+}
+
+// With scratch (point_order_bytes) points are ordered, kPointsOrdered at a
+// time, where there are at least 16 to a probe.  A training step on 2048
+// probes gains 181 us of 1438 with 1 M points, 14 of 989 with 130,000 and
+// nothing any more with 40,000.  Points in order by cage already lose nothing
+// (1198 us without, 1175 with).
+cudaError_t launch_query_adjoint(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam,
+                                 const float* dE, float* g_irr, int32_t* scratch, cudaStream_t st) {
+    const int n_bins = kPointBins * v.n_probes;
+    while (n > 0) {
+        int64_t m = scratch ? std::min<int64_t>(n, kPointsOrdered) : n;
+        PointOrder o{};
+        if (scratch && m >= 16 * (int64_t)v.n_probes) {
+            o = point_order(scratch, v.n_probes);
+            cudaError_t e = cudaMemsetAsync(o.groups, 0, sizeof(int32_t) * (2 + (size_t)n_bins), st);
+            if (e != cudaSuccess) return e;
+            const int blocks = (int)((m + 255) / 256);
+            k_point_bins<<<blocks, 256, 0, st>>>(v, pos, nrm, (int)m, cam, o);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = launch_pdl(k_point_ranges, (n_bins + 255) / 256, 256, 0, st, n_bins, (int)m, o)) != cudaSuccess) return e;
+            if ((e = launch_pdl(k_point_order, blocks, 256, 0, st, (int)m, o)) != cudaSuccess) return e;
+        }
+        cudaError_t e = query_adjoint(v, pos, nrm, m, cam, dE, g_irr, o, st);
+        if (e != cudaSuccess) return e;
+        pos += 3 * m;
+        nrm += 3 * m;
+        dE += 3 * m;
+        n -= m;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_border_fold(float* g_irr, int P, int n, cudaStream_t st) {

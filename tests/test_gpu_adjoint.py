@@ -265,3 +265,33 @@ def test_material_gradients_of_many_objects(g, rays):
         grads.append((albedo.grad.double().sum(0), emit.grad.double().sum(0)))
     for many, one in zip(*grads):
         assert bool((one > 0).all()) and float(((many - one).abs() / one).max()) <= 1e-4
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 5000, 2 ** 20 + 1500])
+def test_backward_of_points_in_random_order(g, n):
+    """Points are put in order by cage where there are at least 16 to a probe,
+    2^20 at a time.  Emitter gradients of n random points against the sum over
+    parts of 1000, which are taken as they come (1e-4: FP32 sums of 5000
+    positive terms in another order), and against Euler's theorem, as in the
+    full-size test."""
+    S = g.Scene.from_arrays(synth.room_scene())
+    V = g.Volume(synth.room_volume(origin=(1.0, 1.0, 1.0), spacing=(2.5, 2.5, 2.5), counts=(4, 4, 4), gamma=1.0,
+                                   state_machine=0))
+    sc = synth.room_scene()
+    albedo = torch.tensor(sc.object_albedo, dtype=torch.float32, device="cuda")
+    emit = torch.tensor(sc.emitter_radiance, dtype=torch.float32, device="cuda")
+    pos, nrm, cam = synth.room_queries(n=n)
+    pos, nrm = to_dev(pos), to_dev(nrm)
+
+    def grad(a, b):
+        e = emit.clone().requires_grad_(True)
+        E = g.IrradianceField.apply(albedo, e, V, S, synth.Lights(), pos[a:b], nrm[a:b], cam, 0, 2)
+        E.sum().backward()
+        return e.grad.double(), E.detach().double().sum(0)
+
+    got, E = grad(0, n)
+    euler = (emit.double() * got).sum(0)
+    assert bool((E > 0).all()) and float(((euler - E).abs() / E).max()) <= 1e-3
+    if n <= 5000:
+        ref = sum(grad(a, min(a + 1000, n))[0] for a in range(0, n, 1000))
+        assert float(((got - ref).abs() / ref.abs().max(0).values).max()) <= 1e-4
