@@ -107,7 +107,11 @@ enum QueryFormId {
     kQueryE5 = 2,       // RGB9E5 irradiance and FP32 distance, gamma 5, no offsets
     kQueryMoved = 3,    // FP32 atlases, gamma 5, probe offsets
     kQueryGamma1 = 4,   // FP32 atlases, gamma 1, no offsets
-    kQueryGeneral = 5
+    // any gamma, in queries of points alone (point_query_form)
+    kQueryFp32Any = 5,  // FP32 atlases, no offsets
+    kQueryHalfAny = 6,  // FP16 atlases, no offsets
+    kQueryE5Any = 7,    // RGB9E5 irradiance and FP32 distance, no offsets
+    kQueryGeneral = 8
 };
 
 inline int query_form(const VolView& w) {
@@ -130,6 +134,28 @@ inline cudaError_t with_query_form(int form, F&& f) {
         case kQueryMoved: return f(std::integral_constant<int, kQueryMoved>{});
         case kQueryGamma1: return f(std::integral_constant<int, kQueryGamma1>{});
         default: return f(std::integral_constant<int, kQueryGeneral>{});
+    }
+}
+
+// The form of a query of points: where query_form has none for the gamma, one
+// with the gamma's power at run time.  Hit shading and the adjoint stay
+// general there, as their registers are full without it.
+inline int point_query_form(const VolView& w) {
+    const int form = query_form(w);
+    if (form != kQueryGeneral || w.offsets) return form;
+    if (w.irr_format == DDGI_IRR_FP32 && w.dist_format == DDGI_DIST_FP32) return kQueryFp32Any;
+    if (w.irr_format == DDGI_IRR_FP16 && w.dist_format == DDGI_DIST_FP16) return kQueryHalfAny;
+    if (w.irr_format == DDGI_IRR_RGB9E5 && w.dist_format == DDGI_DIST_FP32) return kQueryE5Any;
+    return form;
+}
+
+template <typename F>
+inline cudaError_t with_point_query_form(int form, F&& f) {
+    switch (form) {
+        case kQueryFp32Any: return f(std::integral_constant<int, kQueryFp32Any>{});
+        case kQueryHalfAny: return f(std::integral_constant<int, kQueryHalfAny>{});
+        case kQueryE5Any: return f(std::integral_constant<int, kQueryE5Any>{});
+        default: return with_query_form(form, f);
     }
 }
 

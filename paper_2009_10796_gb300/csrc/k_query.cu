@@ -262,7 +262,7 @@ cudaError_t launch_query(const VolView& v, const float* pos, const float* nrm, i
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + kQueryThreads - 1) / kQueryThreads;
     int grid = (int)(blocks < 1048576 ? blocks : 1048576);
-    return with_query_form(query_form(v), [&](auto f) {
+    return with_point_query_form(point_query_form(v), [&](auto f) {
         constexpr int F = decltype(f)::value;
         return out_host ? launch_pdl(k_query<true, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out)
                         : launch_pdl(k_query<false, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out);
@@ -274,7 +274,7 @@ cudaError_t launch_query_glossy(const VolView& v, const float* pos, const float*
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + 255) / 256;
     int grid = (int)(blocks < 1048576 ? blocks : 1048576);
-    return with_query_form(query_form(v), [&](auto f) {
+    return with_point_query_form(point_query_form(v), [&](auto f) {
         k_query_glossy<decltype(f)::value><<<grid, 256, 0, st>>>(v, pos, nrm, dirs, n, out);
         return cudaGetLastError();
     });

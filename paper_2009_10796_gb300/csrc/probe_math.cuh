@@ -329,17 +329,6 @@ __device__ __forceinline__ float2 sample_dist_at(const VolView& v, int p, const 
                        w00 * a.y + w10 * b.y + w01 * c.y + w11 * d.y);
 }
 
-// FP32-only form of sample_dist_at (the same loads and arithmetic).
-__device__ __forceinline__ float2 sample_dist_fp32(const VolView& v, int p, const Footprint& f) {
-    const int row = v.dist_n + 2;
-    const float2* q = (const float2*)v.dist + (int64_t)p * v.dist_tile + (int64_t)f.y0 * row + f.x0;
-    const float2 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + row), d = __ldg(q + row + 1);
-    float w00 = (1.0f - f.tx) * (1.0f - f.ty), w10 = f.tx * (1.0f - f.ty);
-    float w01 = (1.0f - f.tx) * f.ty, w11 = f.tx * f.ty;
-    return make_float2(w00 * a.x + w10 * b.x + w01 * c.x + w11 * d.x,
-                       w00 * a.y + w10 * b.y + w01 * c.y + w11 * d.y);
-}
-
 __device__ __forceinline__ float3 sample_irr(const VolView& v, int p, float3 dir) {
     return sample_irr_at(v, p, footprint(oct_encode(dir), v.irr_n));
 }
@@ -419,9 +408,11 @@ __device__ __forceinline__ uint64_t gamma_decode_g5_pair(float er, float eg) {
 // What a specialised query form fixes at compile time (query_form).
 template <int FORM>
 struct QueryForm {
-    static constexpr bool kHalf = FORM == kQueryHalf;        // FP16 atlases
-    static constexpr bool kE5 = FORM == kQueryE5;            // RGB9E5 irradiance
-    static constexpr bool kGamma1 = FORM == kQueryGamma1;    // gamma 1 (else 5)
+    static constexpr bool kHalf = FORM == kQueryHalf || FORM == kQueryHalfAny;   // FP16 atlases
+    static constexpr bool kE5 = FORM == kQueryE5 || FORM == kQueryE5Any;         // RGB9E5 irradiance
+    static constexpr bool kGamma1 = FORM == kQueryGamma1;    // gamma 1,
+    static constexpr bool kAnyGamma =                        // or the view's (else 5)
+        FORM == kQueryFp32Any || FORM == kQueryHalfAny || FORM == kQueryE5Any;
     static constexpr bool kMoved = FORM == kQueryMoved;      // probe offsets
 };
 
@@ -605,8 +596,8 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
 // pairs (the blue channel scalar).  Bound by instruction issue for
 // neighbouring points: 1920 x 1080 of them on 16 x 8 x 16 probes, beyond the
 // grid planes on one axis, take 72-83 us by the storage format (general form:
-// 142-182 us).  Points in random order are bound by L2 sectors instead
-// (124-165 us).
+// 142-182 us), with the power of any other gamma 131-149 us (232-277).
+// Points in random order are bound by L2 sectors instead (124-165 us).
 // EDGES: corners of zero trilinear weight are passed over (no lookup, the
 // same sums), which a volume's points on and beyond its grid planes gain
 // from: the glossy lookup of 960 x 540 such points 33.6 -> 22.6 us, a
@@ -638,6 +629,10 @@ __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, 
             acc.x += w * gamma_decode_half_fast(er, 0.5f);
             acc.y += w * gamma_decode_half_fast(eg, 0.5f);
             acc.z += w * gamma_decode_half_fast(eb, 0.5f);
+        } else if constexpr (QueryForm<FORM>::kAnyGamma) {
+            acc.x += w * gamma_decode_half_fast(er, v.half_gamma);
+            acc.y += w * gamma_decode_half_fast(eg, v.half_gamma);
+            acc.z += w * gamma_decode_half_fast(eb, v.half_gamma);
         } else {
             float dr_, dg_;
             f2_unpack(gamma_decode_g5_pair(er, eg), dr_, dg_);

@@ -25,6 +25,7 @@ FORMS = {   # irradiance format, distance format, gamma, offsets
     "fp32": (0, 0, 5.0, False), "half": (1, 1, 5.0, False), "rgb9e5": (2, 0, 5.0, False),
     "moved": (0, 0, 5.0, True), "gamma1": (0, 0, 1.0, False), "half_fp32": (1, 0, 5.0, False),
     "gamma2": (0, 0, 2.0, False), "moved_half": (1, 1, 5.0, True),
+    "half_gamma1": (1, 1, 1.0, False), "half_gamma2.2": (1, 1, 2.2, False), "rgb9e5_gamma2.2": (2, 0, 2.2, False),
 }
 
 
