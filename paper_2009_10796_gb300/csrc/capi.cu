@@ -1645,6 +1645,21 @@ ddgi_status ddgi_scene_set_materials(ddgi_scene s, const float* albedo_dev, cons
     return DDGI_OK;
 }
 
+// Scratch for ordering n query points: allocated once for a volume, of one
+// size, so that a captured pass keeps its address; none (the points are taken
+// as they come) for few points, a capture before the first pass, or no memory.
+static int32_t* point_scratch(ddgi_volume_s* v, int64_t n, cudaStream_t st) {
+    if (n < 16 * v->P || 16 * v->P > kPointsOrdered) return nullptr;
+    if (v->point_scratch) return v->point_scratch;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return nullptr;
+    if (cudaMalloc((void**)&v->point_scratch, point_order_bytes(v->P)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        v->point_scratch = nullptr;
+    }
+    return v->point_scratch;
+}
+
 ddgi_status ddgi_diff_forward(ddgi_volume v, ddgi_scene s, const ddgi_lights* lights, int64_t first_frame,
                               int32_t n_frames, const float* pos_dev, const float* nrm_dev, int64_t n,
                               const float camera_pos[3], float* out_dev, ddgi_stream stream) {
@@ -1677,22 +1692,11 @@ ddgi_status ddgi_diff_forward(ddgi_volume v, ddgi_scene s, const ddgi_lights* li
         DDGI_CK(cudaMemcpyAsync(v->snap_irr[f + 1], v->irr, v->irr_bytes, cudaMemcpyDeviceToDevice, st));
         DDGI_CK(cudaMemcpyAsync(v->snap_dist[f + 1], v->dist, v->dist_bytes, cudaMemcpyDeviceToDevice, st));
     }
-    return ddgi_query(v, pos_dev, nrm_dev, n, camera_pos, out_dev, stream);
-}
-
-// Scratch for ordering n query points: allocated once for a volume, of one
-// size, so that a captured pass keeps its address; none (the points are taken
-// as they come) for few points, a capture before the first pass, or no memory.
-static int32_t* point_scratch(ddgi_volume_s* v, int64_t n, cudaStream_t st) {
-    if (n < 16 * v->P || 16 * v->P > kPointsOrdered) return nullptr;
-    if (v->point_scratch) return v->point_scratch;
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return nullptr;
-    if (cudaMalloc((void**)&v->point_scratch, point_order_bytes(v->P)) != cudaSuccess) {
-        (void)cudaGetLastError();
-        v->point_scratch = nullptr;
-    }
-    return v->point_scratch;
+    int32_t* scratch = pos_dev && nrm_dev && out_dev ? point_scratch(v, n, st) : nullptr;
+    if (!scratch) return ddgi_query(v, pos_dev, nrm_dev, n, camera_pos, out_dev, stream);
+    DDGI_CK(launch_query_ordered(make_view(v), pos_dev, nrm_dev, n,
+                                 make_float3(camera_pos[0], camera_pos[1], camera_pos[2]), out_dev, scratch, st));
+    return DDGI_OK;
 }
 
 ddgi_status ddgi_diff_backward(ddgi_volume v, ddgi_scene s, const ddgi_lights* lights, int64_t first_frame,

@@ -449,6 +449,14 @@ struct PointOrder {
     int32_t* rank;     // its place among the bin's,
     int32_t* order;    // and the points by bin
 };
+// Groups in a warp beyond which the adjoint takes its points one by one; points
+// with half as many on average are scattered.
+constexpr int kAdjMaxGroups = 10;
+cudaError_t order_points(const VolView& v, const float* pos, const float* nrm, int64_t m, float3 cam, int32_t* scratch,
+                         PointOrder& o, cudaStream_t st);
+// launch_query with the points ordered (device output).
+cudaError_t launch_query_ordered(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam, float* out,
+                                 int32_t* scratch, cudaStream_t st);
 inline size_t point_order_bytes(int64_t n_probes) {
     return sizeof(int32_t) * (2 + (size_t)kPointBins * (size_t)n_probes + 3 * (size_t)kPointsOrdered);
 }

@@ -79,7 +79,6 @@ __device__ __forceinline__ void add_run6(float* p, float a0, float a1, float a2,
 // it saves, and each lane adds its own 16 runs in pairs.  1920 x 1080 points
 // of a hall seen from inside: 4126 -> 249 us; the same points shuffled:
 // 1370 -> 785 us.
-constexpr int kAdjMaxGroups = 10;
 template <int FORM>
 __device__ __forceinline__ void query_M_adjoint_warp(const VolView& v, bool valid, float3 x, float3 n, float3 wo,
                                                      float3 dM, float* g_irr, AdjointScratch& sh) {
@@ -225,10 +224,6 @@ __device__ __forceinline__ float3 direction_to(float3 cam, float3 x, float3 n) {
 // unordered, 178 us ordered, the three passes included.  Points that neighbour
 // each other already (a G-buffer) are found so by the first pass, and the
 // others leave at once.
-__device__ __forceinline__ bool points_scattered(const PointOrder& o, int n) {
-    return *o.groups > kAdjMaxGroups / 2 * ((n + 31) / 32);
-}
-
 __global__ void __launch_bounds__(256) k_point_bins(VolView v, const float* __restrict__ pos,
                                                     const float* __restrict__ nrm, int n, float3 cam, PointOrder o) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -539,28 +534,32 @@ static cudaError_t query_adjoint(const VolView& v, const float* pos, const float
     });
 }
 
-// With scratch (point_order_bytes) points are ordered, kPointsOrdered at a
-// time, where there are at least 16 to a probe.  A training step on 2048
-// probes gains 181 us of 1438 with 1 M points, 14 of 989 with 130,000 and
-// nothing any more with 40,000.  Points in order by cage already lose nothing
-// (1198 us without, 1175 with).
+// Orders m points where there is scratch (point_order_bytes) and there are at
+// least 16 of them to a probe; else o stays empty and they are taken as they
+// come.  The adjoint of a training step on 2048 probes gains 181 us of 1438 with
+// 1 M points, 14 of 989 with 130,000 and nothing any more with 40,000.  Points
+// in order by cage already lose nothing (1198 us without, 1175 with).
+cudaError_t order_points(const VolView& v, const float* pos, const float* nrm, int64_t m, float3 cam, int32_t* scratch,
+                         PointOrder& o, cudaStream_t st) {
+    if (!scratch || m < 16 * (int64_t)v.n_probes) return cudaSuccess;
+    const int n_bins = kPointBins * v.n_probes, blocks = (int)((m + 255) / 256);
+    o = point_order(scratch, v.n_probes);
+    cudaError_t e = cudaMemsetAsync(o.groups, 0, sizeof(int32_t) * (2 + (size_t)n_bins), st);
+    if (e != cudaSuccess) return e;
+    k_point_bins<<<blocks, 256, 0, st>>>(v, pos, nrm, (int)m, cam, o);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_pdl(k_point_ranges, (n_bins + 255) / 256, 256, 0, st, n_bins, (int)m, o)) != cudaSuccess) return e;
+    return launch_pdl(k_point_order, blocks, 256, 0, st, (int)m, o);
+}
+
 cudaError_t launch_query_adjoint(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam,
                                  const float* dE, float* g_irr, int32_t* scratch, cudaStream_t st) {
-    const int n_bins = kPointBins * v.n_probes;
     while (n > 0) {
-        int64_t m = scratch ? std::min<int64_t>(n, kPointsOrdered) : n;
+        const int64_t m = scratch ? std::min<int64_t>(n, kPointsOrdered) : n;
         PointOrder o{};
-        if (scratch && m >= 16 * (int64_t)v.n_probes) {
-            o = point_order(scratch, v.n_probes);
-            cudaError_t e = cudaMemsetAsync(o.groups, 0, sizeof(int32_t) * (2 + (size_t)n_bins), st);
-            if (e != cudaSuccess) return e;
-            const int blocks = (int)((m + 255) / 256);
-            k_point_bins<<<blocks, 256, 0, st>>>(v, pos, nrm, (int)m, cam, o);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if ((e = launch_pdl(k_point_ranges, (n_bins + 255) / 256, 256, 0, st, n_bins, (int)m, o)) != cudaSuccess) return e;
-            if ((e = launch_pdl(k_point_order, blocks, 256, 0, st, (int)m, o)) != cudaSuccess) return e;
-        }
-        cudaError_t e = query_adjoint(v, pos, nrm, m, cam, dE, g_irr, o, st);
+        cudaError_t e = order_points(v, pos, nrm, m, cam, scratch, o, st);
+        if (e != cudaSuccess) return e;
+        e = query_adjoint(v, pos, nrm, m, cam, dE, g_irr, o, st);
         if (e != cudaSuccess) return e;
         pos += 3 * m;
         nrm += 3 * m;

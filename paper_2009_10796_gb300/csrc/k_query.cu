@@ -12,15 +12,17 @@ namespace ddgi {
 // Four CTAs per SM (64 registers): 1920 x 1080 points of a hall take 72 us; at
 // five (48 registers, spills) the time was 3 % longer.
 constexpr int kQueryThreads = 256;
-template <bool STAGE_OUT, int FORM>
+// ORDERED: the points are taken in the order of o (launch_query_ordered).
+template <bool STAGE_OUT, int FORM, bool ORDERED = false>
 __global__ void __launch_bounds__(kQueryThreads, 4) k_query(VolView v, const float* __restrict__ pos,
                                                             const float* __restrict__ nrm, int64_t n, float3 cam,
-                                                            float* __restrict__ out) {
+                                                            float* __restrict__ out, PointOrder o) {
     pdl_wait();
     pdl_trigger();
     __shared__ __align__(16) float s_out[3 * kQueryThreads];
     for (int64_t q0 = (int64_t)blockIdx.x * kQueryThreads; q0 < n; q0 += (int64_t)gridDim.x * kQueryThreads) {
-        const int64_t q = q0 + threadIdx.x;
+        int64_t q = q0 + threadIdx.x;
+        if (ORDERED && q < n && points_scattered(o, (int)n)) q = o.order[q];
         float3 E = f3(0.0f, 0.0f, 0.0f);
         if (q < n) {
             float3 x = f3(__ldg(pos + 3 * q), __ldg(pos + 3 * q + 1), __ldg(pos + 3 * q + 2));
@@ -264,9 +266,38 @@ cudaError_t launch_query(const VolView& v, const float* pos, const float* nrm, i
     int grid = (int)(blocks < 1048576 ? blocks : 1048576);
     return with_point_query_form(point_query_form(v), [&](auto f) {
         constexpr int F = decltype(f)::value;
-        return out_host ? launch_pdl(k_query<true, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out)
-                        : launch_pdl(k_query<false, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out);
+        return out_host ? launch_pdl(k_query<true, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out,
+                                     PointOrder{})
+                        : launch_pdl(k_query<false, F>, grid, kQueryThreads, 0, st, v, pos, nrm, n, camera, out,
+                                     PointOrder{});
     });
+}
+
+// Scattered points in order by cage, so that a warp's lookups share sectors,
+// with the scratch of the adjoint's order (the differentiable forward).  1 M
+// points on the boxes of a room, 2048 probes: 159 us as they come, 86 us in
+// order and 33 us for the order.  Its three launches and the ragged bins cost
+// more than they give with 130,000 points (972 us a training step, 977 with the
+// order), so it takes 2^18 points and 128 to a probe.
+cudaError_t launch_query_ordered(const VolView& v, const float* pos, const float* nrm, int64_t n, float3 cam, float* out,
+                                 int32_t* scratch, cudaStream_t st) {
+    for (int64_t a = 0; a < n; a += kPointsOrdered) {
+        const int64_t m = std::min<int64_t>(n - a, kPointsOrdered);
+        const float *x = pos + 3 * a, *y = nrm + 3 * a;
+        PointOrder o{};
+        cudaError_t e = cudaSuccess;
+        if (m >= 1 << 18 && m >= 128 * (int64_t)v.n_probes) e = order_points(v, x, y, m, cam, scratch, o, st);
+        if (e == cudaSuccess && !o.order) {
+            e = launch_query(v, x, y, m, cam, out + 3 * a, st);
+        } else if (e == cudaSuccess) {
+            e = with_point_query_form(point_query_form(v), [&](auto f) {
+                return launch_pdl(k_query<false, decltype(f)::value, true>, (int)((m + kQueryThreads - 1) / kQueryThreads),
+                                  kQueryThreads, 0, st, v, x, y, m, cam, out + 3 * a, o);
+            });
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_query_glossy(const VolView& v, const float* pos, const float* nrm, const float* dirs, int64_t n,

@@ -767,4 +767,9 @@ __device__ __forceinline__ float3 cascade_M(const VolView* vols, int n, float3 x
     return (1.0f / sum) * acc;
 }
 
+// Whether points were put in order (order_points).
+__device__ __forceinline__ bool points_scattered(const PointOrder& o, int n) {
+    return *o.groups > kAdjMaxGroups / 2 * ((n + 31) / 32);
+}
+
 }  // namespace ddgi

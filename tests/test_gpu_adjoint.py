@@ -295,3 +295,22 @@ def test_backward_of_points_in_random_order(g, n):
     if n <= 5000:
         ref = sum(grad(a, min(a + 1000, n))[0] for a in range(0, n, 1000))
         assert float(((got - ref).abs() / ref.abs().max(0).values).max()) <= 1e-4
+
+
+@pytest.mark.parametrize("n", [2 ** 18, 2 ** 18 + 1, 2 ** 20 + 1024, 2 ** 20 + 2 ** 18 + 5])
+def test_forward_of_points_in_random_order(g, n):
+    """The differentiable forward takes points in order by cage; each lands in
+    its own row: against the plain query on the atlas that the forward left
+    (1e-4, the parity tolerance), with background points among them."""
+    sc = synth.room_scene()
+    S = g.Scene.from_arrays(sc)
+    V = g.Volume(synth.room_volume(origin=(1.0, 1.0, 1.0), spacing=(2.5, 2.5, 2.5), counts=(4, 4, 4), gamma=1.0,
+                                   state_machine=0))
+    albedo = torch.tensor(sc.object_albedo, dtype=torch.float32, device="cuda")
+    emit = torch.tensor(sc.emitter_radiance, dtype=torch.float32, device="cuda", requires_grad=True)
+    pos, nrm, cam = synth.room_queries(n=n)
+    nrm[::17] = 0.0
+    pos, nrm = to_dev(pos), to_dev(nrm)
+    E = g.IrradianceField.apply(albedo, emit, V, S, synth.room_lights(), pos, nrm, cam, 0, 1).detach()
+    ref = V.query(pos, nrm, cam)
+    assert bool((E[::17] == 0).all()) and float(((E - ref).abs() / ref.abs().clamp_min(1e-3)).max()) <= 1e-4
