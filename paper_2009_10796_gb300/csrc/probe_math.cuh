@@ -459,11 +459,21 @@ __device__ __forceinline__ uint64_t irr_taps(const VolView& v, int p, const Foot
     return rg;
 }
 
+// A Chebyshev weight is the ratio of a variance, the difference of two moments,
+// to that and the squared distance beyond the mean.  Where both are small the
+// last bits of the moments and of the distance decide it, so their sums are
+// written out as fused operations in one order for each form: FP32 gamma 5
+// queries begin with the second product, all others and the adjoint with the
+// first: the orders in which the plain expressions were compiled before there
+// were forms (in cascades the distance stays the plain expression).  With the
+// other order single points near an occluder move by 0.3 %.
+template <int FORM, bool ADJOINT>
+struct SumOrder {
+    static constexpr bool kFirst = ADJOINT || FORM != kQueryFp32;
+};
+
 // The distance moments of a form's atlas at a footprint as packed (mean, mean
-// square) pairs.  A Chebyshev weight takes the variance, a difference, from
-// these sums, so their order is kept as it was in each direction: the second
-// tap's product first in queries, the first's in the adjoint (ADJOINT).  With
-// the other order points near an occluder moved by up to 0.3 %.
+// square) pairs.
 template <int FORM, bool ADJOINT = false>
 __device__ __forceinline__ float2 dist_taps(const VolView& v, int p, const Footprint& f) {
     if constexpr (FORM == kQueryGeneral) return sample_dist_at(v, p, f);
@@ -488,7 +498,7 @@ __device__ __forceinline__ float2 dist_taps(const VolView& v, int p, const Footp
     }
     const Bilerp w = bilerp_weights(f);
     const uint64_t W00 = f2_pack(w.w00, w.w00), W10 = f2_pack(w.w10, w.w10);
-    uint64_t m = ADJOINT ? f2_fma(W10, b, f2_mul(W00, a)) : f2_fma(W00, a, f2_mul(W10, b));
+    uint64_t m = SumOrder<FORM, ADJOINT>::kFirst ? f2_fma(W10, b, f2_mul(W00, a)) : f2_fma(W00, a, f2_mul(W10, b));
     m = f2_fma(f2_pack(w.w01, w.w01), c, m);
     m = f2_fma(f2_pack(w.w11, w.w11), d, m);
     float2 r;
@@ -567,7 +577,9 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
     const float hb = (1.0f + cw) * 0.5f;
     const float wb = hb * hb + 0.2f;
     const float3 pv = a + q.lb;                                                // biased point - probe
-    const float rr = dot(pv, pv);
+    const float xy = SumOrder<FORM, IEEE>::kFirst ? __fmaf_rn(pv.y, pv.y, __fmul_rn(pv.x, pv.x))
+                                                  : __fmaf_rn(pv.x, pv.x, __fmul_rn(pv.y, pv.y));
+    const float rr = BRANCH ? dot(pv, pv) : __fmaf_rn(pv.z, pv.z, xy);
     float wc = 1.0f;
     if (!BRANCH || rr > 0.0f) {   // without the branch rr = 0 makes a NaN of r, beyond no mean
         const float r = IEEE ? sqrtf(rr) : rr * rsqrtf(rr);
