@@ -1,13 +1,16 @@
 // Probe-ray kernels of the update (Sec. 2.3 and Sec. 6.3):
-//   k_classify     distance-only trace of UNINIT probes -> OFF / NEWLY_VIGILANT / SLEEPING
-//   k_trace_shade  closest hit + shading of every ray of every active probe
+//   k_classify, k_classify_split  distance-only trace of UNINIT probes -> OFF /
+//                     NEWLY_VIGILANT / SLEEPING; k_optimize moves them first
+//   k_trace_primary, k_trace_shadow, k_shade  the update's three passes
+//   k_trace_shade     closest hit + shading of every ray of every active probe
+//                     (the allocation-free update)
 // plus two utility kernels over arbitrary rays (raw closest hit, camera G-buffer).
 //
 // Work layout: rays of one probe are consecutive work items, so a warp
-// traces 32 rays of the same probe (same origin, directions spread by the
-// spherical-Fibonacci pattern).  Kernels are persistent: the grid is sized to
-// the machine and threads stride over the device-side work count, so the host
-// never waits for the active-probe count.
+// traces 32 rays of the same probe (same origin, a compact cone of directions
+// by the ray order).  Kernels are persistent: the grid is sized to the machine
+// and warps take work up to the device-side count, so the host never waits for
+// the active-probe count.
 #include <algorithm>
 
 #include "traverse.cuh"

@@ -1,8 +1,8 @@
 // Ray traversal of the scene's hierarchy in its two forms: the 4-wide
 // nodes that the probe-ray passes walk warp-cooperatively (the while-while
 // scheme of Aila and Laine, HPG 2009, over four child boxes per node), and
-// the binary nodes that the one-ray-per-thread paths (G-buffer, raw ray
-// queries, allocation-free update, adjoint) walk.  Triangles are tested with
+// the binary nodes that the FP64 differentiation walks with one ray a
+// thread.  Triangles are tested with
 // the watertight ray/triangle test of Woop, Benthin and Wald ("Watertight
 // Ray/Triangle Intersection", JCGT 2013).  The edge
 // functions are evaluated with explicitly rounded products and differences
@@ -142,20 +142,11 @@ __device__ __forceinline__ float box_enter(const RayPre& r, float lx, float hx, 
     return tn <= tf * 1.0000005f ? tn : INFINITY;
 }
 
-// Slab test with the near and far planes already chosen by the ray's octant
-// (nx = the box's lo.x when the ray runs toward +x, its hi.x otherwise, and
-// so on): the same entry distance as box_enter, since per axis the near-plane
-// distance is exactly the smaller of the two, without the per-axis min/max.
-__device__ __forceinline__ float box_enter_oct(const RayPre& r, float nx, float fx, float ny, float fy, float nz,
-                                               float fz, float tmax) {
-    float tn = fmax3f((nx - r.o.x) * r.idir.x, (ny - r.o.y) * r.idir.y, fmaxf((nz - r.o.z) * r.idir.z, 0.0f));
-    float tf = fmin3f((fx - r.o.x) * r.idir.x, (fy - r.o.y) * r.idir.y, fminf((fz - r.o.z) * r.idir.z, tmax));
-    return tn <= tf * 1.0000005f ? tn : INFINITY;
-}
-
-// box_enter_oct for the four children of a 4-wide node at once: the slab
-// distances of children (0, 1) and (2, 3) in packed pairs, the same IEEE
-// operations lane by lane, so each k_c equals box_enter_oct's result.
+// The slab test for the four children of a 4-wide node at once, with the near
+// and far planes already chosen by the ray's octant (lo.x is near when the ray
+// runs toward +x, and so on), which saves the per-axis min/max: the distances
+// of children (0, 1) and (2, 3) in packed pairs, box_enter's IEEE operations
+// lane by lane, so each k_c equals its result.
 //
 // FUSED evaluates each plane's distance as p r + c in one multiply-add, r the
 // reciprocal direction and c = -o r moved outward by 1.8e-7 |o r| (SlabRay).
