@@ -43,13 +43,21 @@ def _np(a, dtype):
     return np.ascontiguousarray(np.asarray(a, dtype=dtype))
 
 
+_NUMBERS = frozenset((float, int, np.float32, np.float64))
+
+
 def _xyz(v):
-    """Three floats of a tuple, list, array or tensor of three numbers."""
-    try:
-        x, y, z = v.tolist() if hasattr(v, "tolist") else v
-        return float(x), float(y), float(z)
-    except (TypeError, ValueError):   # other shapes and element types
-        return tuple(float(x) for x in np.asarray(v, dtype=np.float64).reshape(3))
+    """Three floats of whatever numpy makes an array of three numbers of.  Three plain numbers and
+    float arrays, which every call passes, are unpacked directly; anything else goes through numpy,
+    which refuses what is not an array of numbers in host memory (sets, strings, tensors on the
+    device or with a gradient)."""
+    if type(v) is np.ndarray and v.dtype.kind == "f":
+        v = v.tolist()
+    if (type(v) is tuple or type(v) is list) and len(v) == 3:
+        x, y, z = v
+        if type(x) in _NUMBERS and type(y) in _NUMBERS and type(z) in _NUMBERS:
+            return float(x), float(y), float(z)
+    return tuple(float(x) for x in np.asarray(v, dtype=np.float64).reshape(3))
 
 
 def _f3(v):

@@ -140,3 +140,33 @@ def test_vector_arguments_convert_alike():
     for bad in ([1.0, 2.0], None, "abc", np.zeros((2, 3))):
         with pytest.raises((ValueError, TypeError)):
             api._f3(bad)
+
+
+class _DeviceTensor:
+    """As a tensor on the device: has tolist(), is no host array."""
+    def tolist(self):
+        return [0.5, -1.0, 3.0]
+
+    def __array__(self, *args, **kwargs):
+        raise TypeError("can't convert a device tensor to numpy")
+
+
+def test_vector_arguments_refused_as_numpy_refuses_them():
+    """What is no array of three numbers in host memory raises: strings and their like, sets and
+    dicts (no order to take), generators, tensors that carry a gradient or lie on the device."""
+    import numpy as np
+    import torch
+
+    from paper_2009_10796_gb300 import api
+    want = torch.tensor([0.5, -1.0, 3.0])
+    convert = (lambda v: np.asarray(v, dtype=np.float64).reshape(3), api._f3)
+    for make in (lambda: "123", lambda: b"123", lambda: {1.0, 2.0, 3.0}, lambda: {1.0: 0, 2.0: 0, 3.0: 0},
+                 lambda: (x for x in (1.0, 2.0, 3.0)), lambda: want.clone().requires_grad_(True),
+                 lambda: [want[0], want[1], want[2].clone().requires_grad_(True)], lambda: want.bfloat16(),
+                 _DeviceTensor, lambda: [1.0, 2.0, 3.0, 4.0], lambda: [[1.0, 2.0], [3.0, 4.0]]):
+        for f in convert:
+            with pytest.raises((ValueError, TypeError, RuntimeError)):
+                f(make())
+    for good in ((np.float32(0.5), -1, 3), ["0.5", "-1", "3"], [want[0], want[1], want[2]], np.array([[0.5], [-1], [3]]),
+                 np.array([0.5, -1.0, 3.0], np.longdouble), (False, True, 3)):
+        assert list(api._f3(good)) == [float(x) for x in np.asarray(good, dtype=np.float64).reshape(3)]
