@@ -21,11 +21,15 @@ __all__ = ["Scene", "Volume", "Cascade", "IrradianceField", "trace", "lights_str
 
 def _stream(stream):
     """The stream's handle as an integer (None: torch's current stream of the
-    current device, read without building a Stream object)."""
+    current device, read without building a Stream object where this torch has
+    the internal calls for it)."""
     if stream is None:
         if not torch.cuda.is_initialized():
             torch.cuda.init()
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

@@ -170,3 +170,21 @@ def test_vector_arguments_refused_as_numpy_refuses_them():
     for good in ((np.float32(0.5), -1, 3), ["0.5", "-1", "3"], [want[0], want[1], want[2]], np.array([[0.5], [-1], [3]]),
                  np.array([0.5, -1.0, 3.0], np.longdouble), (False, True, 3)):
         assert list(api._f3(good)) == [float(x) for x in np.asarray(good, dtype=np.float64).reshape(3)]
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_current_stream_without_the_internal_calls(monkeypatch, missing):
+    """A torch without the internal calls that read the current stream gives it by its public one."""
+    import types
+
+    import torch
+
+    from paper_2009_10796_gb300 import api
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    monkeypatch.setattr(torch._C, "_cuda_getDevice", lambda: 0, raising=False)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 78, raising=False)
+    assert api._stream(None) == 78
+    monkeypatch.delattr(torch._C, missing)
+    assert api._stream(None) == 77
+    assert api._stream(5) == 5 and api._stream(types.SimpleNamespace(cuda_stream=6)) == 6
