@@ -416,7 +416,7 @@ typedef struct {
  * shade, blend and state advance run over all volumes' probes together; hit
  * shading samples the whole cascade of the previous frame (Sec. 7.3
  * weights).  Per-frame parameters go through device memory, so with
- * use_graph the sequence is captured once (per precision, lights,
+ * use_graph the sequence is captured once (per scene, precision, lights,
  * hysteresis scales and tuning) and replayed.  Blocks the host only while an
  * earlier frame still reads the pinned parameter slot this frame reuses
  * (two slots).  Errors: INVALID_ARG, UNSUPPORTED, CUDA. */

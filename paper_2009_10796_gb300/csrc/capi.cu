@@ -1,6 +1,7 @@
 // C ABI and host runtime: scene registration (BVH build + upload), volume
 // allocation, the per-frame launch sequence, queries, buffer access, timing.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -102,6 +103,7 @@ std::vector<int32_t> ray_order_morton(int R) {
 using namespace ddgi;
 
 struct ddgi_scene_s {
+    const int64_t id = next_id();   // never used again, unlike the handle's address
     DevScene dev{};
     float4* nodes = nullptr;
     float4* nodes4 = nullptr;
@@ -111,6 +113,12 @@ struct ddgi_scene_s {
     float4* emit = nullptr;
     int64_t n_nodes = 0, n_leaves = 0, n_tris = 0;
     int32_t n_objects = 0, n_emitters = 0;
+
+private:
+    static int64_t next_id() {
+        static std::atomic<int64_t> last{0};
+        return ++last;
+    }
 };
 
 struct TimedStage {
@@ -1075,12 +1083,17 @@ struct FrameParams {
     int32_t pad[3];
 };
 
+// What a captured frame holds by value: a change of any of it recaptures.  The
+// scene (its device pointers) goes by its id, since an address can come back
+// after the scene there was destroyed.
 struct GraphKey {
+    int64_t scene = 0;
     int32_t precision = -1, trace_mult = 0, blend_probes = 0;
     float irr_scale = 0.f, vis_scale = 0.f;
     ddgi_lights lights{};
     bool operator==(const GraphKey& o) const { return std::memcmp(this, &o, sizeof(GraphKey)) == 0; }
 };
+static_assert(sizeof(GraphKey) == sizeof(int64_t) + 5 * 4 + sizeof(ddgi_lights), "compared as bytes: no padding");
 
 }  // namespace
 
@@ -1384,6 +1397,7 @@ ddgi_status ddgi_cascade_update(ddgi_cascade c, ddgi_scene s, const ddgi_lights*
 
     if (params->use_graph) {
         GraphKey key;
+        key.scene = s->id;
         key.precision = params->blend_precision;
         key.trace_mult = c->trace_mult;
         key.blend_probes = c->blend_probes;

@@ -98,6 +98,29 @@ def test_cascade_graph_replay_matches_eager(g):
         assert torch.equal(A.buffer(k, 1), B.buffer(k, 1))
 
 
+def test_cascade_graph_follows_the_scene(g):
+    """A replayed frame traces the scene it is given: two scenes that both live in turn, each in both
+    parameter slots, then one created where a destroyed one may have been."""
+    L = synth.room_lights()
+    fine, coarse = _descs()
+    scenes = [g.Scene.from_arrays(synth.room_scene(n_boxes=n)) for n in (12, 3)]
+    A, B = g.Cascade([fine, coarse]), g.Cascade([fine, coarse])
+
+    def frame(f, S):
+        A.update(S, L, f, _camera(0))
+        B.update(S, L, f, _camera(0), use_graph=True)
+        torch.cuda.synchronize()
+        for k in range(2):
+            for a, b in ((A.states(k), B.states(k)), (A.buffer(k, 0), B.buffer(k, 0)), (A.buffer(k, 1), B.buffer(k, 1))):
+                assert torch.equal(a, b), (f, k)
+
+    for f in range(6):
+        frame(f, scenes[(f // 2) % 2])
+    for S in scenes:
+        S.close()
+    frame(6, g.Scene.from_arrays(synth.room_scene(n_boxes=8)))
+
+
 def test_cascade_autotune_and_cache(g, tmp_path):
     sc = synth.room_scene(n_boxes=12)
     L = synth.room_lights()
