@@ -198,8 +198,9 @@ inline cudaError_t once_per_device(DeviceOnce& once, F&& f) {
 }
 
 // Volumes a kernel works on: one view by value (a single volume) or a device
-// table of up to kMaxVolumes views (a cascade).  Probe lists hold entries
-// (volume << 24) | probe, so a single volume's entries are its probe indices.
+// table of up to kMaxVolumes views (a cascade).  A cascade's probe lists hold
+// entries (volume << 24) | probe, and it has below 2^24 probes; a single
+// volume's hold the probe index alone, up to 2^26 (entry_probe).
 constexpr int kMaxVolumes = 8;
 constexpr int kEntryShift = 24;
 constexpr int32_t kEntryMask = (1 << kEntryShift) - 1;
@@ -214,6 +215,12 @@ template <bool MULTI>
 __device__ __forceinline__ const VolView& vol_of(const VolSet& s, int k) {
     if (MULTI) return s.table[k];
     return s.single;
+}
+
+// The probe of a list entry (vol_of takes its volume, entry >> kEntryShift).
+template <bool MULTI>
+__device__ __forceinline__ int entry_probe(int entry) {
+    return MULTI ? entry & kEntryMask : entry;
 }
 
 inline VolSet single_set(const VolView& v) {

@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(256) k_blend_simt(VolSet vs, BlendParams bp, i
             int e = active[g0 + threadIdx.x];
             s_probe[threadIdx.x] = e;
             s_newly[threadIdx.x] =
-                state_newly(vol_of<MULTI>(vs, e >> kEntryShift).states[e & kEntryMask]);
+                state_newly(vol_of<MULTI>(vs, e >> kEntryShift).states[entry_probe<MULTI>(e)]);
         }
         for (int k = threadIdx.x; k < np * R; k += blockDim.x) {
             int pp = k / R, i = k - pp * R;
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(256) k_blend_simt(VolSet vs, BlendParams bp, i
                 ab = fmaf(w, L.z, ab);
             }
             const int e = s_probe[pp];
-            blend_irr_texel(vol_of<MULTI>(vs, e >> kEntryShift), bp, e & kEntryMask, t, ar, ag, ab,
+            blend_irr_texel(vol_of<MULTI>(vs, e >> kEntryShift), bp, entry_probe<MULTI>(e), t, ar, ag, ab,
                             __ldg(inv_s_irr + t), s_newly[pp] != 0, status);
         }
         // distance texels: power-cosine weighted mean distance and mean squared distance
@@ -249,14 +249,14 @@ __global__ void __launch_bounds__(256) k_blend_simt(VolSet vs, BlendParams bp, i
                 m2 = fmaf(w, d * d, m2);
             }
             const int e = s_probe[pp];
-            blend_dist_texel(vol_of<MULTI>(vs, e >> kEntryShift), bp, e & kEntryMask, t, m1, m2,
+            blend_dist_texel(vol_of<MULTI>(vs, e >> kEntryShift), bp, entry_probe<MULTI>(e), t, m1, m2,
                              __ldg(inv_s_dist + t), s_newly[pp] != 0, status);
         }
         __syncthreads();
         if (threadIdx.x < np && s_newly[threadIdx.x]) {
             const int e = s_probe[threadIdx.x];
             {
-                uint8_t* sp = vol_of<MULTI>(vs, e >> kEntryShift).states + (e & kEntryMask);
+                uint8_t* sp = vol_of<MULTI>(vs, e >> kEntryShift).states + entry_probe<MULTI>(e);
                 *sp = state_advanced(*sp);
             }
         }
@@ -407,10 +407,10 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
             int e = active[g0 + threadIdx.x];
             s_probe[threadIdx.x] = e;
             const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
-            s_newly[threadIdx.x] = state_newly(v.states[e & kEntryMask]);
+            s_newly[threadIdx.x] = state_newly(v.states[entry_probe<MULTI>(e)]);
             // the probe's old tiles into L2 while the group is summed (the
             // epilogue then reads them from L2)
-            prefetch_tiles_l2(v, e & kEntryMask);
+            prefetch_tiles_l2(v, entry_probe<MULTI>(e));
         }
         // records -> planes, kRecBatch independent loads in flight per thread.
         // Item k is (ray pair, probe, ray within the pair): two threads read a
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
                 xs[u] = 1 + t - y * nd;
                 ys[u] = 1 + y;
                 const int e = s_probe[pp[u]];
-                old[u] = load_dist<false>(vol_of<MULTI>(vs, e >> kEntryShift), e & kEntryMask, xs[u], ys[u]);
+                old[u] = load_dist<false>(vol_of<MULTI>(vs, e >> kEntryShift), entry_probe<MULTI>(e), xs[u], ys[u]);
                 m1[u] = sum_d[2 * o];
                 m2[u] = sum_d[2 * o + 1];
                 inv[u] = inv_d[t];
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
             for (int u = 0; u < kBD; ++u) {
                 if (o0 + u * (int)blockDim.x >= np * td) break;
                 const int e = s_probe[pp[u]];
-                store_dist_with_borders(vol_of<MULTI>(vs, e >> kEntryShift), e & kEntryMask, xs[u], ys[u],
+                store_dist_with_borders(vol_of<MULTI>(vs, e >> kEntryShift), entry_probe<MULTI>(e), xs[u], ys[u],
                                         blend_dist_value(bp, old[u], m1[u], m2[u], inv[u], s_newly[pp[u]] != 0,
                                                          status));
             }
@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
                 xs[u] = 1 + t - y * ni;
                 ys[u] = 1 + y;
                 const int e = s_probe[pp[u]];
-                old[u] = load_irr<false>(vol_of<MULTI>(vs, e >> kEntryShift), e & kEntryMask, xs[u], ys[u]);
+                old[u] = load_irr<false>(vol_of<MULTI>(vs, e >> kEntryShift), entry_probe<MULTI>(e), xs[u], ys[u]);
                 sum[u] = f3(sum_i[3 * o], sum_i[3 * o + 1], sum_i[3 * o + 2]);
                 inv[u] = inv_i[t];
             }
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
                 if (o0 + u * (int)blockDim.x >= np * ti) break;
                 const int e = s_probe[pp[u]];
                 const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
-                store_irr_with_borders(v, e & kEntryMask, xs[u], ys[u],
+                store_irr_with_borders(v, entry_probe<MULTI>(e), xs[u], ys[u],
                                        blend_irr_value(v, bp, old[u], sum[u].x, sum[u].y, sum[u].z, inv[u],
                                                        s_newly[pp[u]] != 0, status));
             }
@@ -611,7 +611,7 @@ __global__ void __launch_bounds__(kTileMaxThreads, 2) k_blend_tiled(VolSet vs, B
         if (threadIdx.x < np && s_newly[threadIdx.x]) {
             const int e = s_probe[threadIdx.x];
             {
-                uint8_t* sp = vol_of<MULTI>(vs, e >> kEntryShift).states + (e & kEntryMask);
+                uint8_t* sp = vol_of<MULTI>(vs, e >> kEntryShift).states + entry_probe<MULTI>(e);
                 *sp = state_advanced(*sp);
             }
         }

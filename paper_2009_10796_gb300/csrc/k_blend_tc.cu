@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(NT, 1) k_blend_tc(VolSet vs, BlendParams bp, c
         if (tid < PG) {
             const int e = tid < np ? active[g0 + tid] : 0;
             s_probe[tid] = e;
-            s_newly[tid] = tid < np && state_newly(vol_of<MULTI>(vs, e >> kEntryShift).states[e & kEntryMask]);
+            s_newly[tid] = tid < np && state_newly(vol_of<MULTI>(vs, e >> kEntryShift).states[entry_probe<MULTI>(e)]);
         }
         __syncthreads();
         if (control) {
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(NT, 1) k_blend_tc(VolSet vs, BlendParams bp, c
                 const int pp = k / (ui + ud), u = k - pp * (ui + ud);
                 const int e = s_probe[pp];
                 const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
-                const int64_t pb = e & kEntryMask;
+                const int64_t pb = entry_probe<MULTI>(e);
                 const uint8_t* src = u < ui ? (const uint8_t*)v.irr + pb * tile_i + gran * u
                                             : (const uint8_t*)v.dist + pb * tile_d + gran * (u - ui);
                 uint8_t* dst = u < ui ? Ti + pp * tile_i + gran * u : Td + pp * tile_d + gran * (u - ui);
@@ -645,7 +645,7 @@ __global__ void __launch_bounds__(NT, 1) k_blend_tc(VolSet vs, BlendParams bp, c
                 const int pp = k / (ui + ud), u = k - pp * (ui + ud);
                 const int e = s_probe[pp];
                 const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
-                const int64_t pb = e & kEntryMask;
+                const int64_t pb = entry_probe<MULTI>(e);
                 uint8_t* dst = u < ui ? (uint8_t*)v.irr + pb * tile_i + gran * u
                                       : (uint8_t*)v.dist + pb * tile_d + gran * (u - ui);
                 const uint8_t* src = u < ui ? Ti + pp * tile_i + gran * u : Td + pp * tile_d + gran * (u - ui);
@@ -655,7 +655,7 @@ __global__ void __launch_bounds__(NT, 1) k_blend_tc(VolSet vs, BlendParams bp, c
         }
         if (tid < np && s_newly[tid]) {
             const int e = s_probe[tid];
-            uint8_t* sp = vol_of<MULTI>(vs, e >> kEntryShift).states + (e & kEntryMask);
+            uint8_t* sp = vol_of<MULTI>(vs, e >> kEntryShift).states + entry_probe<MULTI>(e);
             *sp = state_advanced(*sp);
         }
         // the next round's weight copies (async proxy) overwrite what these accesses used

@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(256) k_classify(DevScene s, VolSet vs, const f
     for (int q = warp; q < n; q += nwarps) {
         int e = list[q];
         const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
-        int p = e & kEntryMask;
+        int p = entry_probe<MULTI>(e);
         float3 o = probe_pos_phys(v, p);
         int bf = 0;
         float dmin = INFINITY;
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256, kClassCtas) k_classify_split(DevScene s, 
         const int q = (int)(it / nb), b = (int)(it - (unsigned)q * nb);
         const int e = list[q];
         const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
-        const int p = e & kEntryMask;
+        const int p = entry_probe<MULTI>(e);
         const float3 o = probe_pos_phys(v, p);
         const int j = 32 * b + lane;
         const bool valid = j < R;
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(256, trace_ctas(MULTI)) k_trace_primary(
             rec = slot * R + i;
             const int entry = __ldg(active + slot);
             const float4 d4 = __ldg(dirs + i);
-            r = ray_pre_packed(probe_pos_phys(vol_of<MULTI>(vs, entry >> kEntryShift), entry & kEntryMask),
+            r = ray_pre_packed(probe_pos_phys(vol_of<MULTI>(vs, entry >> kEntryShift), entry_probe<MULTI>(entry)),
                                f3(d4.x, d4.y, d4.z), __ldg(dirs + R + 2 * i), __ldg(dirs + R + 2 * i + 1));
         }
         const bool valid = b + lane < total;
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(256, trace_ctas(MULTI)) k_trace_shadow(
         const int slot = (int)fast_div((uint32_t)rec, dR);
         const int i = rec - slot * R;
         const int e = __ldg(active + slot);
-        const float3 o = probe_pos_phys(vol_of<MULTI>(vs, e >> kEntryShift), e & kEntryMask);
+        const float3 o = probe_pos_phys(vol_of<MULTI>(vs, e >> kEntryShift), entry_probe<MULTI>(e));
         const float4 d4 = __ldg(dirs + i);
         const float4 hr = hits[rec];
         float3 ng;
@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(256, 4) k_shade(DevScene s, VolSet vs, Lights 
         float3 ng;
         hit_frame(s, k, ng);
         float t = hr.x;
-        float3 o = probe_pos_phys(v, e & kEntryMask);
+        float3 o = probe_pos_phys(v, entry_probe<MULTI>(e));
         float3 n = (1.0f / length(ng)) * ng;
         float3 x = o + t * d;
         // the sun's cosine term (zero when the shadow ray was blocked) and the

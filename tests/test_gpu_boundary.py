@@ -196,3 +196,25 @@ def test_overlapped_launches_match_ordinary_launches(g, monkeypatch):
     monkeypatch.delenv("DDGI_NO_PDL", raising=False)
     for a, b in zip(overlapped, ordinary):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "tf32"])
+def test_probe_index_above_24_bits(g, precision):
+    """A volume of more than 2^24 probes (up to 2^26 are accepted): the planes past index 2^24
+    get the first frame of a small volume that stands where they are, bit for bit (every
+    atlas is zero before it, so no hit sees another probe)."""
+    nx, ny, nz, tail, s = 66, 64, 4000, 24, 0.25
+    assert nx * ny * (nz - tail) > 1 << 24
+    kw = dict(spacing=(s, s, s), rays_per_probe=8, irr_n=2, dist_n=3, hysteresis_irr=0.9, hysteresis_vis=0.9, seed=77)
+    at = (-3.0, 1.0, 2.0)                                     # exact in FP32, as are all positions
+    S, L = g.Scene.from_arrays(synth.room_scene(n_boxes=12)), synth.room_lights()
+    big = g.Volume(synth.VolumeDesc(origin=(at[0], at[1], at[2] - s * (nz - tail)), counts=(nx, ny, nz), **kw))
+    small = g.Volume(synth.VolumeDesc(origin=at, counts=(nx, ny, tail), **kw))
+    for V in (big, small):
+        V.update(S, L, 3, precision=getattr(g, "BLEND_" + precision.upper()))
+    torch.cuda.synchronize()
+    st = small.states()
+    assert len(torch.unique(st)) > 1 and not (st == 0).any()  # classified, traced and blended
+    n = small.n_probes
+    for a, b in ((big.states(), st), (big.irr_raw(), small.irr_raw()), (big.dist_raw(), small.dist_raw())):
+        assert torch.equal(a.view(big.n_probes, -1)[-n:], b.view(n, -1))
