@@ -1659,19 +1659,22 @@ ddgi_status ddgi_scene_set_materials(ddgi_scene s, const float* albedo_dev, cons
     return DDGI_OK;
 }
 
-// Scratch for ordering n query points: allocated once for a volume, of one
-// size, so that a captured pass keeps its address; none (the points are taken
-// as they come) for few points, a capture before the first pass, or no memory.
-static int32_t* point_scratch(ddgi_volume_s* v, int64_t n, cudaStream_t st) {
-    if (n < 16 * v->P || 16 * v->P > kPointsOrdered) return nullptr;
-    if (v->point_scratch) return v->point_scratch;
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) return nullptr;
+// Scratch for ordering n query points, or none (the points are taken as they
+// come) for few points and on volumes that got none.
+static int32_t* point_scratch(const ddgi_volume_s* v, int64_t n) {
+    return n >= 16 * v->P ? v->point_scratch : nullptr;
+}
+
+// Allocates it with a volume's first snapshots, whatever the number of points,
+// and of one size: a later call with more points allocates nothing (which
+// would break another stream's capture in progress), and a captured pass keeps
+// its address.  Without memory for it the volume goes without.
+static void allocate_point_scratch(ddgi_volume_s* v) {
+    if (v->point_scratch || 16 * v->P > kPointsOrdered) return;
     if (cudaMalloc((void**)&v->point_scratch, point_order_bytes(v->P)) != cudaSuccess) {
         (void)cudaGetLastError();
         v->point_scratch = nullptr;
     }
-    return v->point_scratch;
 }
 
 ddgi_status ddgi_diff_forward(ddgi_volume v, ddgi_scene s, const ddgi_lights* lights, int64_t first_frame,
@@ -1682,6 +1685,7 @@ ddgi_status ddgi_diff_forward(ddgi_volume v, ddgi_scene s, const ddgi_lights* li
     ddgi_status r = diff_check(v, n_frames);
     if (r != DDGI_OK) return r;
     cudaStream_t st = (cudaStream_t)stream;
+    const bool first = v->snap_irr.empty();
     while ((int)v->snap_irr.size() < n_frames + 1) {
         void *a = nullptr, *b = nullptr;
         DDGI_CK(cudaMalloc(&a, v->irr_bytes));
@@ -1689,6 +1693,7 @@ ddgi_status ddgi_diff_forward(ddgi_volume v, ddgi_scene s, const ddgi_lights* li
         v->snap_irr.push_back(a);
         v->snap_dist.push_back(b);
     }
+    if (first) allocate_point_scratch(v);
     DDGI_CK(cudaMemsetAsync(v->irr, 0, v->irr_bytes, st));
     DDGI_CK(cudaMemsetAsync(v->dist, 0, v->dist_bytes, st));
     DDGI_CK(cudaMemsetAsync(v->states, DDGI_STATE_VIGILANT, (size_t)v->P, st));
@@ -1706,7 +1711,7 @@ ddgi_status ddgi_diff_forward(ddgi_volume v, ddgi_scene s, const ddgi_lights* li
         DDGI_CK(cudaMemcpyAsync(v->snap_irr[f + 1], v->irr, v->irr_bytes, cudaMemcpyDeviceToDevice, st));
         DDGI_CK(cudaMemcpyAsync(v->snap_dist[f + 1], v->dist, v->dist_bytes, cudaMemcpyDeviceToDevice, st));
     }
-    int32_t* scratch = pos_dev && nrm_dev && out_dev ? point_scratch(v, n, st) : nullptr;
+    int32_t* scratch = pos_dev && nrm_dev && out_dev ? point_scratch(v, n) : nullptr;
     if (!scratch) return ddgi_query(v, pos_dev, nrm_dev, n, camera_pos, out_dev, stream);
     DDGI_CK(launch_query_ordered(make_view(v), pos_dev, nrm_dev, n,
                                  make_float3(camera_pos[0], camera_pos[1], camera_pos[2]), out_dev, scratch, st));
@@ -1743,7 +1748,7 @@ ddgi_status ddgi_diff_backward(ddgi_volume v, ddgi_scene s, const ddgi_lights* l
     Lights L = make_lights(lights);
     float3 cam = make_float3(camera_pos[0], camera_pos[1], camera_pos[2]);
     DDGI_CK(launch_query_adjoint(snap_view(n_frames), pos_dev, nrm_dev, n, cam, dE_dev, v->g_irr,
-                                 point_scratch(v, n, st), st));
+                                 point_scratch(v, n), st));
     float* g = v->g_irr;
     float* gp = v->g_prev;
     for (int f = n_frames - 1; f >= 0; --f) {

@@ -314,3 +314,38 @@ def test_forward_of_points_in_random_order(g, n):
     E = g.IrradianceField.apply(albedo, emit, V, S, synth.room_lights(), pos, nrm, cam, 0, 1).detach()
     ref = V.query(pos, nrm, cam)
     assert bool((E[::17] == 0).all()) and float(((E - ref).abs() / ref.abs().clamp_min(1e-3)).max()) <= 1e-4
+
+
+def test_more_points_than_before_allocate_nothing(g):
+    """A volume that has run a step on few points runs one on many (which are put in order) while
+    another stream is being captured: no allocation, so the capture survives, and the same result."""
+    sc = synth.room_scene()
+    S, L = g.Scene.from_arrays(sc), synth.room_lights()
+    pos, nrm, cam = synth.room_queries(n=2 ** 18)
+    pos, nrm = to_dev(pos), to_dev(nrm)
+    few = (pos[:64].contiguous(), nrm[:64].contiguous())
+    one = torch.ones_like(pos)
+    counts = dict(n_objects=len(sc.object_albedo), n_emitters=len(sc.emitter_radiance))
+
+    def volume():
+        return g.Volume(synth.room_volume(origin=(1.0, 1.0, 1.0), spacing=(2.5, 2.5, 2.5), counts=(4, 4, 4), gamma=1.0,
+                                          state_machine=0))
+
+    ref, V = volume(), volume()
+    E = ref.diff_forward(S, L, pos, nrm, cam)
+    grads = ref.diff_backward(S, L, pos, nrm, cam, one, **counts)
+    V.diff_forward(S, L, *few, cam)
+    V.diff_backward(S, L, *few, cam, one[:64].contiguous(), **counts)
+    work, x, graph = torch.cuda.Stream(), torch.zeros(8, device="cuda"), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream(), capture_error_mode="global"):
+        x += 1
+        E2 = V.diff_forward(S, L, pos, nrm, cam, stream=work)
+        grads2 = V.diff_backward(S, L, pos, nrm, cam, one, stream=work, **counts)
+        E3, grads3 = E2.clone(), [a.clone() for a in grads2]      # in the capture: run at the replay
+    work.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert bool((x == 1).all()) and torch.equal(E3, E)
+    for a, b in zip(grads3, grads):
+        assert float((a - b).abs().max()) <= 1e-4 * float(b.abs().max())
