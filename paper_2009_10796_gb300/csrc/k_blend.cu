@@ -323,7 +323,7 @@ __device__ __forceinline__ void cp_async_wait_ahead() {
 // the grid is one wave of resident CTAs); blockDim = TiledShape::threads.
 // Up to 8 probes to an SM go to the first n_sm CTAs, one on each, since a CTA
 // streams all of the weights whatever its probes (1079 probes of 8 x 8 and
-// 16 x 16 texels 40.5 -> 38.9 us; at 13.5 probes to an SM two CTAs are faster).
+// 16 x 16 texels 41.0 -> 40.7 us; at 13.5 probes to an SM two CTAs are faster).
 // ROW16: the weight rows start on 16-byte boundaries (R a multiple of 4) and
 // arrive in 16-byte copies, else in 4-byte ones; rays past R weigh zero.  (The
 // row kernel took ray counts off 4 before: a room's frame with 63 rays
@@ -807,14 +807,17 @@ static int smem_optin() {
     return optin;
 }
 
-// Opts both blend kernels of one instantiation into the maximum dynamic
-// shared memory, once per device.
+// Opts the blend kernels of one instantiation into the maximum dynamic
+// shared memory, once per device.  The kernels lie in the module in the order
+// of their first use, and the 16-byte form's time depends on where it lies: the
+// same instructions before the 4-byte form took 59.5 us on the city and 43.0 on
+// 8 x 8 and 16 x 16 texels, in this order 57.5 and 40.8 (alone 57.5 and 41.1).
 template <bool MULTI, int PGS>
 static cudaError_t opt_in_blend() {
     static DeviceOnce tiled, tiled4, rows;
-    cudaError_t e = allow_max_smem(k_blend_tiled<MULTI, PGS, true>, tiled);
-    if (e == cudaSuccess) e = allow_max_smem(k_blend_tiled<MULTI, PGS, false>, tiled4);
+    cudaError_t e = allow_max_smem(k_blend_tiled<MULTI, PGS, false>, tiled4);
     if (e == cudaSuccess) e = allow_max_smem(k_blend_simt<MULTI, PGS>, rows);
+    if (e == cudaSuccess) e = allow_max_smem(k_blend_tiled<MULTI, PGS, true>, tiled);
     return e;
 }
 
@@ -832,7 +835,7 @@ static cudaError_t launch_tiled(const VolSet& vs, const BlendParams& bp, int irr
     cudaError_t e = opt_in_blend<MULTI, PG>();
     if (e != cudaSuccess) return e;
     const TiledShape ts = tiled_shape(PG, bp.R, irr_n, dist_n);
-    auto kernel = bp.R % 4 == 0 ? k_blend_tiled<MULTI, PG, true> : k_blend_tiled<MULTI, PG, false>;
+    auto kernel = bp.R % 4 != 0 ? k_blend_tiled<MULTI, PG, false> : k_blend_tiled<MULTI, PG, true>;
     // one wave of resident CTAs; the kernel splits the active probes evenly
     int occ = 0, dev = 0, sms = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, ts.threads, ts.smem)) != cudaSuccess) return e;
