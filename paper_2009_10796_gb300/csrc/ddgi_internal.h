@@ -97,21 +97,25 @@ inline void set_view_divisors(VolView& w) {
 
 // Forms of the probe query with a specialised device function (the storage
 // format, gamma and offsets fixed at compile time; otherwise the general
-// form's operations in the same order).  The line between them is which
-// combinations are used: FP32 and FP16 atlases and RGB9E5 irradiance with
-// the default gamma, probe offsets (the position optimizer) and gamma 1 (the
-// differentiable path) with FP32 atlases; anything else is general.
+// form's operations).  The line between them is which combinations are used:
+// for hit shading and the adjoint, FP32 and FP16 atlases and RGB9E5 irradiance
+// with the default gamma, probe offsets (the position optimizer) and gamma 1
+// (the differentiable path) with FP32 atlases; for queries of points
+// (point_query_form) those formats with any gamma.  Mixed FP16 and FP32
+// atlases and offsets with other formats take the general form.
 enum QueryFormId {
     kQueryFp32 = 0,     // FP32 atlases, gamma 5, no offsets
     kQueryHalf = 1,     // FP16 atlases, gamma 5, no offsets
     kQueryE5 = 2,       // RGB9E5 irradiance and FP32 distance, gamma 5, no offsets
     kQueryMoved = 3,    // FP32 atlases, gamma 5, probe offsets
     kQueryGamma1 = 4,   // FP32 atlases, gamma 1, no offsets
-    // any gamma, in queries of points alone (point_query_form)
-    kQueryFp32Any = 5,  // FP32 atlases, no offsets
-    kQueryHalfAny = 6,  // FP16 atlases, no offsets
-    kQueryE5Any = 7,    // RGB9E5 irradiance and FP32 distance, no offsets
-    kQueryGeneral = 8
+    // in queries of points alone (point_query_form)
+    kQueryHalfGamma1 = 5,   // FP16 atlases, gamma 1, no offsets
+    kQueryE5Gamma1 = 6,     // RGB9E5 irradiance and FP32 distance, gamma 1, no offsets
+    kQueryFp32Any = 7,      // the three formats with any other gamma, no offsets
+    kQueryHalfAny = 8,
+    kQueryE5Any = 9,
+    kQueryGeneral = 10
 };
 
 inline int query_form(const VolView& w) {
@@ -137,21 +141,23 @@ inline cudaError_t with_query_form(int form, F&& f) {
     }
 }
 
-// The form of a query of points: where query_form has none for the gamma, one
-// with the gamma's power at run time.  Hit shading and the adjoint stay
-// general there, as their registers are full without it.
+// The form of a query of points: where query_form has none for the format
+// and gamma, one of its own.  Hit shading and the adjoint stay general there.
 inline int point_query_form(const VolView& w) {
     const int form = query_form(w);
     if (form != kQueryGeneral || w.offsets) return form;
+    const bool g1 = w.half_gamma == 0.5f;
     if (w.irr_format == DDGI_IRR_FP32 && w.dist_format == DDGI_DIST_FP32) return kQueryFp32Any;
-    if (w.irr_format == DDGI_IRR_FP16 && w.dist_format == DDGI_DIST_FP16) return kQueryHalfAny;
-    if (w.irr_format == DDGI_IRR_RGB9E5 && w.dist_format == DDGI_DIST_FP32) return kQueryE5Any;
+    if (w.irr_format == DDGI_IRR_FP16 && w.dist_format == DDGI_DIST_FP16) return g1 ? kQueryHalfGamma1 : kQueryHalfAny;
+    if (w.irr_format == DDGI_IRR_RGB9E5 && w.dist_format == DDGI_DIST_FP32) return g1 ? kQueryE5Gamma1 : kQueryE5Any;
     return form;
 }
 
 template <typename F>
 inline cudaError_t with_point_query_form(int form, F&& f) {
     switch (form) {
+        case kQueryHalfGamma1: return f(std::integral_constant<int, kQueryHalfGamma1>{});
+        case kQueryE5Gamma1: return f(std::integral_constant<int, kQueryE5Gamma1>{});
         case kQueryFp32Any: return f(std::integral_constant<int, kQueryFp32Any>{});
         case kQueryHalfAny: return f(std::integral_constant<int, kQueryHalfAny>{});
         case kQueryE5Any: return f(std::integral_constant<int, kQueryE5Any>{});

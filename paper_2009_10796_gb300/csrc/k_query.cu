@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(256, 4) k_query_glossy(VolView v, const float*
             float3 r = d - (2.0f * dn) * nn;
             float lr = length(r);
             if (lr > 0.0f) r = (1.0f / lr) * r;
-            M = query_M_look<FORM>(v, x, nn, f3(-d.x, -d.y, -d.z), r);
+            M = query_M_look<FORM, true, corners_per_trip<FORM>(true)>(v, x, nn, f3(-d.x, -d.y, -d.z), r);
         }
         out[3 * q] = M.x;
         out[3 * q + 1] = M.y;

@@ -408,9 +408,12 @@ __device__ __forceinline__ uint64_t gamma_decode_g5_pair(float er, float eg) {
 // What a specialised query form fixes at compile time (query_form).
 template <int FORM>
 struct QueryForm {
-    static constexpr bool kHalf = FORM == kQueryHalf || FORM == kQueryHalfAny;   // FP16 atlases
-    static constexpr bool kE5 = FORM == kQueryE5 || FORM == kQueryE5Any;         // RGB9E5 irradiance
-    static constexpr bool kGamma1 = FORM == kQueryGamma1;    // gamma 1,
+    static constexpr bool kHalf =                            // FP16 atlases
+        FORM == kQueryHalf || FORM == kQueryHalfGamma1 || FORM == kQueryHalfAny;
+    static constexpr bool kE5 =                              // RGB9E5 irradiance
+        FORM == kQueryE5 || FORM == kQueryE5Gamma1 || FORM == kQueryE5Any;
+    static constexpr bool kGamma1 =                          // gamma 1,
+        FORM == kQueryGamma1 || FORM == kQueryHalfGamma1 || FORM == kQueryE5Gamma1;
     static constexpr bool kAnyGamma =                        // or the view's (else 5)
         FORM == kQueryFp32Any || FORM == kQueryHalfAny || FORM == kQueryE5Any;
     static constexpr bool kMoved = FORM == kQueryMoved;      // probe offsets
@@ -517,10 +520,15 @@ struct Cage {
     // Corner c's trilinear factor.  A point on a grid plane or beyond the
     // grid has its fraction clamped to 0 or 1, so that half, three quarters
     // or seven eighths of its cage weigh exactly 0 and need no lookup.
-    __device__ __forceinline__ float trilinear(int c) const { return tx[c & 1] * ty[(c >> 1) & 1] * tz[c >> 2]; }
+    __device__ __forceinline__ float trilinear(int c) const { return side(tx, c & 1) * side(ty, c & 2) * side(tz, c & 4); }
     __device__ __forceinline__ int probe(const VolView& v, int c) const {
-        return (c & 1 ? px[1] : px[0]) + v.counts.x * ((c & 2 ? py[1] : py[0]) + v.counts.y * (c & 4 ? pz[1] : pz[0]));
+        return side(px, c & 1) + v.counts.x * (side(py, c & 2) + v.counts.y * side(pz, c & 4));
     }
+    // x - x_p (high part) to corner c's grid point
+    __device__ __forceinline__ float3 to_grid(int c) const { return f3(side(ax, c & 1), side(ay, c & 2), side(az, c & 4)); }
+    // an element by selection, so that the pairs stay in registers for any c
+    template <typename T>
+    static __device__ __forceinline__ T side(const T (&pair)[2], int upper) { return upper ? pair[1] : pair[0]; }
 };
 
 __device__ __forceinline__ Cage cage_of(const VolView& v, const LocalPoint& q) {
@@ -564,8 +572,7 @@ __device__ __forceinline__ Cage cage_of(const VolView& v, const LocalPoint& q) {
 template <int FORM, bool IEEE = false, bool BRANCH = false>
 __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoint& q, const Cage& k, int c, int p,
                                                float3 n) {
-    const int o0 = c & 1, o1 = (c >> 1) & 1, o2 = c >> 2;
-    float3 a = f3(k.ax[o0], k.ay[o1], k.az[o2]);
+    float3 a = k.to_grid(c);
     if (QueryForm<FORM>::kMoved || (FORM == kQueryGeneral && v.offsets)) {
         const float4 po = __ldg(v.offsets + p);   // the probe's own (moved) position; the cage stays on the grid
         a = f3(a.x - po.x, a.y - po.y, a.z - po.z);
@@ -600,6 +607,20 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
     return wt * wb * fmaxf(wc, 1e-6f);
 }
 
+// Corners that the specialised query takes to a trip of its loop: all eight,
+// but two where the power of any gamma is inlined for three channels of each
+// (1920 x 1080 points inside the grid, FP32 gamma 2.2: 246 us with eight, 216
+// with two, general form 227; in random order 320, 298 and 295; RGB9E5 296, 245
+// and 270), and four for an irradiance query of FP32 atlases at gamma 1 (112 us,
+// with eight 113; in random order 294, 304, general form 288).  The glossy
+// lookup and cascades of that form are no faster so (76 us for points beyond the
+// grid, 74 with eight), and with probe offsets fewer cost neighbouring points
+// 5 % (119 us, 114; general form 136) and give random order 1 % (327, 331; 320).
+template <int FORM>
+__host__ __device__ constexpr int corners_per_trip(bool all) {
+    return QueryForm<FORM>::kAnyGamma ? 2 : FORM == kQueryGamma1 && !all ? 4 : 8;
+}
+
 // The specialised query of query_M_look (FORM < kQueryGeneral): the same
 // operations in the same order, except the decode's zero test
 // (gamma_decode_g5_pair), with the eight cage corners unrolled, the storage
@@ -607,8 +628,8 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
 // channels of the irradiance taps and their decode carried as packed FP32
 // pairs (the blue channel scalar).  Bound by instruction issue for
 // neighbouring points: 1920 x 1080 of them on 16 x 8 x 16 probes, beyond the
-// grid planes on one axis, take 72-83 us by the storage format (general form:
-// 142-182 us), with the power of any other gamma 131-149 us (232-277).
+// grid planes on one axis, take 72-84 us by the storage format (general form:
+// 142-183 us), with the power of any other gamma 128-142 us (234-278).
 // Points in random order are bound by L2 sectors instead (124-165 us).
 // EDGES: corners of zero trilinear weight are passed over (no lookup, the
 // same sums), which a volume's points on and beyond its grid planes gain
@@ -616,27 +637,25 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
 // city frame's hit shading 74 -> 72 us.  Cascades leave it out: a volume of
 // weight 0 at its edges is not read there, and their kernels spill more with
 // the test (2852 -> 2912 us a frame).
-template <int FORM, bool EDGES>
+// CORNERS: corners to a trip of the loop (corners_per_trip).
+template <int FORM, bool EDGES, int CORNERS>
 __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, float3 n, float3 wo, float3 look) {
     const LocalPoint q = local_point(v, x, n, wo);
     const Cage k = cage_of(v, q);
     const Footprint fn = footprint_issue(oct_encode(look), v.irr_n);
     const Bilerp wn = bilerp_weights(fn);
-    int pc[8];
     unsigned act = 0;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        pc[c] = k.probe(v, c);
-        act |= state_active(v.states[pc[c]]) ? 1u << c : 0u;
-    }
+    for (int c = 0; c < 8; ++c) act |= state_active(v.states[k.probe(v, c)]) ? 1u << c : 0u;
     float sumw = 0.0f;
     float3 acc = f3(0.0f, 0.0f, 0.0f);
-#pragma unroll
+#pragma unroll CORNERS
     for (int c = 0; c < 8; ++c) {
         if (!(act & (1u << c)) || (EDGES && k.trilinear(c) == 0.0f)) continue;
-        const float w = corner_weight<FORM, false, !EDGES>(v, q, k, c, pc[c], n);
+        const int p = k.probe(v, c);
+        const float w = corner_weight<FORM, false, !EDGES>(v, q, k, c, p, n);
         float er, eg, eb;
-        f2_unpack(irr_taps<FORM>(v, pc[c], fn, wn, eb), er, eg);
+        f2_unpack(irr_taps<FORM>(v, p, fn, wn, eb), er, eg);
         if constexpr (QueryForm<FORM>::kGamma1) {
             acc.x += w * gamma_decode_half_fast(er, 0.5f);
             acc.y += w * gamma_decode_half_fast(eg, 0.5f);
@@ -672,9 +691,9 @@ __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, 
 // (Sec. 4.4); the bias and the backface weights use n either way.
 // FORM: the view's form (query_form); query_M_look_fast serves all but the
 // general one.
-template <int FORM = kQueryGeneral, bool EDGES = true>
+template <int FORM = kQueryGeneral, bool EDGES = true, int CORNERS = corners_per_trip<FORM>(!EDGES)>
 __device__ __forceinline__ float3 query_M_look(const VolView& v, float3 x, float3 n, float3 wo, float3 look) {
-    if constexpr (FORM != kQueryGeneral) return query_M_look_fast<FORM, EDGES>(v, x, n, wo, look);
+    if constexpr (FORM != kQueryGeneral) return query_M_look_fast<FORM, EDGES, CORNERS>(v, x, n, wo, look);
     const LocalPoint q = local_point(v, x, n, wo);
     float g[3] = {(q.hi.x + q.lb.x) / v.spacing.x, (q.hi.y + q.lb.y) / v.spacing.y,
                   (q.hi.z + q.lb.z) / v.spacing.z};
