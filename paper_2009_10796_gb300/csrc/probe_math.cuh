@@ -227,7 +227,11 @@ __device__ __forceinline__ float3 load_irr(const VolView& v, int p, int x, int y
         float2 a = __half22float2(h0);
         return f3(a.x, a.y, __low2float(h1));
     } else {
-        return rgb9e5_decode(ld<NC>((const uint32_t*)v.irr + t));
+        // (ldexpf: with the power's bits written out as above, the queries that
+        // choose the format here took 160 us for 1920 x 1080 points, 156 so)
+        const uint32_t w = ld<NC>((const uint32_t*)v.irr + t);
+        const float s = ldexpf(1.0f, (int)(w >> 27) - 15 - 9);
+        return f3((float)(w & 511u) * s, (float)((w >> 9) & 511u) * s, (float)((w >> 18) & 511u) * s);
     }
 }
 
