@@ -115,7 +115,8 @@ enum QueryFormId {
     kQueryFp32Any = 7,      // the three formats with any other gamma, no offsets
     kQueryHalfAny = 8,
     kQueryE5Any = 9,
-    kQueryGeneral = 10
+    kQueryGeneral = 10,
+    kQueryFp32First = 11   // kQueryFp32 with the general form's order of sums (SumOrder)
 };
 
 inline int query_form(const VolView& w) {

@@ -679,7 +679,8 @@ cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights
     const int64_t need = ((int64_t)v.n_probes * R + 127) / 128;
     const FastDiv dR = make_fast_div((uint32_t)R);
     return with_query_form(query_form(v), [&](auto f) {
-        return launch_pdl(k_trace_shade<decltype(f)::value>, (int)std::min<int64_t>(grid, need), 128, 0, st, s, v, L, dirs,
+        constexpr int form = decltype(f)::value == kQueryFp32 ? kQueryFp32First : decltype(f)::value;
+        return launch_pdl(k_trace_shade<form>, (int)std::min<int64_t>(grid, need), 128, 0, st, s, v, L, dirs,
                           R, dR, perm, active, count, records);
     });
 }

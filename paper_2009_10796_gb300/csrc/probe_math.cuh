@@ -468,12 +468,16 @@ __device__ __forceinline__ uint64_t irr_taps(const VolView& v, int p, const Foot
 
 // A Chebyshev weight is the ratio of a variance, the difference of two moments,
 // to that and the squared distance beyond the mean.  Where both are small the
-// last bits of the moments and of the distance decide it, so their sums are
-// written out as fused operations in one order for each form: FP32 gamma 5
-// queries begin with the second product, all others and the adjoint with the
-// first: the orders in which the plain expressions were compiled before there
-// were forms (in cascades the distance stays the plain expression).  With the
-// other order single points near an occluder move by 0.3 %.
+// last bits of the moments and of the distance decide it (the other order moves
+// single points near an occluder by 0.3 %), so their sums are written out as
+// fused operations in one order for each form.  They begin with the first product,
+// as the general form's plain expressions are compiled; with the second in FP32
+// gamma 5 queries of a volume's or a cascade's points and hits, as those expressions
+// were compiled for them alone (in cascades the distance stays the plain
+// expression).  The allocation-free update has the first order by a form of its
+// own (kQueryFp32First): the second was 1.04 times as far from 64 bits over 99
+// volumes, 3.5 times in one of them.  For a cascade's query either is as far (3.2e-7
+// to 6.4e-7 rms over six rooms).
 template <int FORM, bool ADJOINT>
 struct SumOrder {
     static constexpr bool kFirst = ADJOINT || FORM != kQueryFp32;
