@@ -129,17 +129,22 @@ inline int query_form(const VolView& w) {
     return kQueryGeneral;
 }
 
-// f(std::integral_constant<int, form>) for a view's form.
-template <typename F>
+// f(std::integral_constant<int, form>) for a view's form.  FORMATS: views of
+// other formats than FP32 occur (not in the differentiable path); OFFSETS: views
+// with probe offsets do (cascades and the allocation-free update have none).
+// What a caller leaves out would take the general form.
+template <bool FORMATS = true, bool OFFSETS = true, typename F>
 inline cudaError_t with_query_form(int form, F&& f) {
-    switch (form) {
-        case kQueryFp32: return f(std::integral_constant<int, kQueryFp32>{});
-        case kQueryHalf: return f(std::integral_constant<int, kQueryHalf>{});
-        case kQueryE5: return f(std::integral_constant<int, kQueryE5>{});
-        case kQueryMoved: return f(std::integral_constant<int, kQueryMoved>{});
-        case kQueryGamma1: return f(std::integral_constant<int, kQueryGamma1>{});
-        default: return f(std::integral_constant<int, kQueryGeneral>{});
+    if (form == kQueryFp32) return f(std::integral_constant<int, kQueryFp32>{});
+    if (form == kQueryGamma1) return f(std::integral_constant<int, kQueryGamma1>{});
+    if constexpr (FORMATS) {
+        if (form == kQueryHalf) return f(std::integral_constant<int, kQueryHalf>{});
+        if (form == kQueryE5) return f(std::integral_constant<int, kQueryE5>{});
     }
+    if constexpr (OFFSETS) {
+        if (form == kQueryMoved) return f(std::integral_constant<int, kQueryMoved>{});
+    }
+    return f(std::integral_constant<int, kQueryGeneral>{});
 }
 
 // The form of a query of points: where query_form has none for the format
@@ -154,16 +159,16 @@ inline int point_query_form(const VolView& w) {
     return form;
 }
 
-template <typename F>
+template <bool FORMATS = true, typename F>
 inline cudaError_t with_point_query_form(int form, F&& f) {
-    switch (form) {
-        case kQueryHalfGamma1: return f(std::integral_constant<int, kQueryHalfGamma1>{});
-        case kQueryE5Gamma1: return f(std::integral_constant<int, kQueryE5Gamma1>{});
-        case kQueryFp32Any: return f(std::integral_constant<int, kQueryFp32Any>{});
-        case kQueryHalfAny: return f(std::integral_constant<int, kQueryHalfAny>{});
-        case kQueryE5Any: return f(std::integral_constant<int, kQueryE5Any>{});
-        default: return with_query_form(form, f);
+    if (form == kQueryFp32Any) return f(std::integral_constant<int, kQueryFp32Any>{});
+    if constexpr (FORMATS) {
+        if (form == kQueryHalfGamma1) return f(std::integral_constant<int, kQueryHalfGamma1>{});
+        if (form == kQueryE5Gamma1) return f(std::integral_constant<int, kQueryE5Gamma1>{});
+        if (form == kQueryHalfAny) return f(std::integral_constant<int, kQueryHalfAny>{});
+        if (form == kQueryE5Any) return f(std::integral_constant<int, kQueryE5Any>{});
     }
+    return with_query_form<FORMATS>(form, f);
 }
 
 // Largest BVH leaf (triangles); the traversal packs a leaf's first triangle

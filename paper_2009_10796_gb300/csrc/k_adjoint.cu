@@ -589,7 +589,7 @@ cudaError_t launch_blend_adjoint(const VolView& v_after, const float* w_irr, con
 cudaError_t launch_shade_adjoint(const DevScene& s, const VolView& v_before, const Lights& L, const float4* dirs,
                                  int P, int R, const int32_t* perm, const float4* gL, float* d_emit,
                                  float* d_albedo, float* g_prev, int with_prev, cudaStream_t st) {
-    return with_query_form(query_form(v_before), [&](auto f) {
+    return with_query_form<false>(query_form(v_before), [&](auto f) {
         k_shade_adjoint<decltype(f)::value><<<grid_for((int64_t)P * R, 32 * kAdjWarps), 32 * kAdjWarps, 0, st>>>(
             s, v_before, L, dirs, P, R, make_fast_div((uint32_t)R), perm, gL, d_emit, d_albedo, g_prev, with_prev);
         return cudaGetLastError();

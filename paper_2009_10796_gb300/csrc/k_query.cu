@@ -234,7 +234,7 @@ cudaError_t launch_query_cascade(const VolSet& vs, const float* pos, const float
     if (n == 0) return cudaSuccess;
     int64_t blocks = (n + 255) / 256;
     int grid = (int)(blocks < 1048576 ? blocks : 1048576);
-    return with_query_form(form, [&](auto f) {
+    return with_query_form<true, false>(form, [&](auto f) {
         k_query_cascade<decltype(f)::value><<<grid, 256, 0, st>>>(vs, pos, nrm, n, camera, out);
         return cudaGetLastError();
     });
@@ -290,7 +290,7 @@ cudaError_t launch_query_ordered(const VolView& v, const float* pos, const float
         if (e == cudaSuccess && !o.order) {
             e = launch_query(v, x, y, m, cam, out + 3 * a, st);
         } else if (e == cudaSuccess) {
-            e = with_point_query_form(point_query_form(v), [&](auto f) {
+            e = with_point_query_form<false>(point_query_form(v), [&](auto f) {
                 return launch_pdl(k_query<false, decltype(f)::value, true>, (int)((m + kQueryThreads - 1) / kQueryThreads),
                                   kQueryThreads, 0, st, v, x, y, m, cam, out + 3 * a, o);
             });

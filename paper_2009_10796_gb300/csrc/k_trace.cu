@@ -17,8 +17,7 @@
 
 namespace ddgi {
 
-template <bool MULTI>
-__global__ void __launch_bounds__(256) k_classify(DevScene s, VolSet vs, const float4* __restrict__ dirs,
+__global__ void __launch_bounds__(256) k_classify(DevScene s, VolView v, const float4* __restrict__ dirs,
                                                   int R, const int32_t* __restrict__ perm,
                                                   const int32_t* __restrict__ list,
                                                   const int32_t* __restrict__ count) {
@@ -32,9 +31,7 @@ __global__ void __launch_bounds__(256) k_classify(DevScene s, VolSet vs, const f
     WwLane<kStackSize4, int2> w;
     w.stack = stack;
     for (int q = warp; q < n; q += nwarps) {
-        int e = list[q];
-        const VolView& v = vol_of<MULTI>(vs, e >> kEntryShift);
-        int p = entry_probe<MULTI>(e);
+        const int p = list[q];
         float3 o = probe_pos_phys(v, p);
         int bf = 0;
         float dmin = INFINITY;
@@ -662,8 +659,8 @@ cudaError_t launch_classify(const DevScene& s, const VolView& v, const float4* d
         return launch_pdl(k_classify_split<false>,
                           bounded_grid(kClassCtas * sm_count(), (int64_t)v.n_probes * ((R + 31) / 32) * 32), 256, 0, st,
                           s, single_set(v), dirs, R, perm, list, count, scratch, next);
-    return launch_pdl(k_classify<false>, bounded_grid(grid, (int64_t)v.n_probes * 32), 256, 0, st, s, single_set(v), dirs,
-                      R, perm, list, count);
+    return launch_pdl(k_classify, bounded_grid(grid, (int64_t)v.n_probes * 32), 256, 0, st, s, v, dirs, R, perm, list,
+                      count);
 }
 
 cudaError_t launch_classify_multi(const DevScene& s, const VolSet& vs, const float4* dirs, int R,
@@ -678,7 +675,7 @@ cudaError_t launch_trace_shade(const DevScene& s, const VolView& v, const Lights
                                float4* records, int grid, cudaStream_t st) {
     const int64_t need = ((int64_t)v.n_probes * R + 127) / 128;
     const FastDiv dR = make_fast_div((uint32_t)R);
-    return with_query_form(query_form(v), [&](auto f) {
+    return with_query_form<true, false>(query_form(v), [&](auto f) {
         constexpr int form = decltype(f)::value == kQueryFp32 ? kQueryFp32First : decltype(f)::value;
         return launch_pdl(k_trace_shade<form>, (int)std::min<int64_t>(grid, need), 128, 0, st, s, v, L, dirs,
                           R, dR, perm, active, count, records);
@@ -707,7 +704,7 @@ static cudaError_t trace_wavefront(const DevScene& s, const VolSet& vs, const Li
                         shadow_count, next_shadow, nullptr)) != cudaSuccess)
         return e;
     if (marks && (e = cudaEventRecord(marks[2], st)) != cudaSuccess) return e;
-    e = with_query_form(form, [&](auto f) {
+    e = with_query_form<true, !MULTI>(form, [&](auto f) {
         return launch_pdl(k_shade<MULTI, decltype(f)::value>, shade_grid, 256, 0, st, s, vs, L, dirs, R, dR, active, hit_list,
                           shadow_count + 1, records);
     });

@@ -57,14 +57,6 @@ __device__ __forceinline__ int wrap(int a, int m) { int r = a % m; return r < 0 
 __device__ __forceinline__ int wrap_add(int a, int s, int m) { int r = a + s; return r >= m ? r - m : r; }
 __device__ __forceinline__ int wrap_sub(int a, int s, int m) { int r = a - s; return r < 0 ? r + m : r; }
 
-// Logical (i, j, k) inside the grid -> physical probe index.
-__device__ __forceinline__ int probe_phys(const VolView& v, int i, int j, int k) {
-    int a = wrap_add(i, v.shift.x, v.counts.x);
-    int b = wrap_add(j, v.shift.y, v.counts.y);
-    int c = wrap_add(k, v.shift.z, v.counts.z);
-    return a + v.counts.x * (b + v.counts.y * c);
-}
-
 __device__ __forceinline__ float3 probe_pos_logical(const VolView& v, int i, int j, int k) {
     return f3(v.origin.x + (float)i * v.spacing.x, v.origin.y + (float)j * v.spacing.y,
               v.origin.z + (float)k * v.spacing.z);
@@ -308,10 +300,6 @@ __device__ __forceinline__ float3 sample_irr_at(const VolView& v, int p, const F
                    load_irr(v, p, f.x0 + 1, f.y0 + 1));
 }
 
-__device__ __forceinline__ float3 sample_irr_at(const VolView& v, int p, const Footprint& f) {
-    return sample_irr_at(v, p, f, bilerp_weights(f));
-}
-
 __device__ __forceinline__ float2 sample_dist_at(const VolView& v, int p, const Footprint& f) {
     const int row = v.dist_n + 2;
     float2 a, b, c, d;
@@ -333,25 +321,9 @@ __device__ __forceinline__ float2 sample_dist_at(const VolView& v, int p, const 
                        w00 * a.y + w10 * b.y + w01 * c.y + w11 * d.y);
 }
 
-__device__ __forceinline__ float3 sample_irr(const VolView& v, int p, float3 dir) {
-    return sample_irr_at(v, p, footprint(oct_encode(dir), v.irr_n));
-}
-
-__device__ __forceinline__ float2 sample_dist(const VolView& v, int p, float3 dir) {
-    return sample_dist_at(v, p, footprint(oct_encode(dir), v.dist_n));
-}
-
-// x^(gamma/2) on the gamma-encoded value; gamma = 5 uses x^2 sqrt(x).
+// x^(gamma/2) on the gamma-encoded value (gamma = 5: x^2 sqrt(x)), sqrt(x) as
+// x * rsqrt(x) (hardware reciprocal square root, about 2 ulp).
 __device__ __forceinline__ float gamma_decode_half(float e, float half_gamma) {
-    e = fmaxf(e, 0.0f);
-    if (half_gamma == 2.5f) return e * e * sqrtf(e);
-    if (half_gamma == 0.5f) return sqrtf(e);
-    return powf(e, half_gamma);
-}
-
-// The same with sqrt(x) as x * rsqrt(x) (hardware reciprocal square root,
-// about 2 ulp), for the query's 8 probes x 3 channels.
-__device__ __forceinline__ float gamma_decode_half_fast(float e, float half_gamma) {
     e = fmaxf(e, 0.0f);
     const float sq = e > 0.0f ? e * rsqrtf(e) : 0.0f;
     if (half_gamma == 2.5f) return e * e * sq;
@@ -399,7 +371,7 @@ __device__ __forceinline__ float3 local_to_probe(const VolView& v, const LocalPo
 
 // x^2.5 of a red / green pair of gamma-encoded values (gamma 5): e^2 times
 // e * rsqrt(e), the squares and products as packed FP32 pairs.  The floor
-// 1e-30 stands in for the zero test of gamma_decode_half_fast: below it both
+// 1e-30 stands in for the zero test of gamma_decode_half: below it both
 // give 0 in FP32 (x^2.5 < 1e-75), above it they are the same operations.
 __device__ __forceinline__ uint64_t gamma_decode_g5_pair(float er, float eg) {
     er = fmaxf(er, 1e-30f);
@@ -665,13 +637,13 @@ __device__ __forceinline__ float3 query_M_look_fast(const VolView& v, float3 x, 
         float er, eg, eb;
         f2_unpack(irr_taps<FORM>(v, p, fn, wn, eb), er, eg);
         if constexpr (QueryForm<FORM>::kGamma1) {
-            acc.x += w * gamma_decode_half_fast(er, 0.5f);
-            acc.y += w * gamma_decode_half_fast(eg, 0.5f);
-            acc.z += w * gamma_decode_half_fast(eb, 0.5f);
+            acc.x += w * gamma_decode_half(er, 0.5f);
+            acc.y += w * gamma_decode_half(eg, 0.5f);
+            acc.z += w * gamma_decode_half(eb, 0.5f);
         } else if constexpr (QueryForm<FORM>::kAnyGamma) {
-            acc.x += w * gamma_decode_half_fast(er, v.half_gamma);
-            acc.y += w * gamma_decode_half_fast(eg, v.half_gamma);
-            acc.z += w * gamma_decode_half_fast(eb, v.half_gamma);
+            acc.x += w * gamma_decode_half(er, v.half_gamma);
+            acc.y += w * gamma_decode_half(eg, v.half_gamma);
+            acc.z += w * gamma_decode_half(eb, v.half_gamma);
         } else {
             float dr_, dg_;
             f2_unpack(gamma_decode_g5_pair(er, eg), dr_, dg_);
@@ -762,9 +734,9 @@ __device__ __forceinline__ float3 query_M_look(const VolView& v, float3 x, float
         }
         float w = wt * wb * fmaxf(wc, 1e-6f);
         float3 e = sample_irr_at(v, p, fn, wn);
-        acc.x += w * gamma_decode_half_fast(e.x, v.half_gamma);
-        acc.y += w * gamma_decode_half_fast(e.y, v.half_gamma);
-        acc.z += w * gamma_decode_half_fast(e.z, v.half_gamma);
+        acc.x += w * gamma_decode_half(e.x, v.half_gamma);
+        acc.y += w * gamma_decode_half(e.y, v.half_gamma);
+        acc.z += w * gamma_decode_half(e.z, v.half_gamma);
         sumw += w;
     }
     if (!(sumw > 0.0f)) return f3(0.0f, 0.0f, 0.0f);
