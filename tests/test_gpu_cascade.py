@@ -141,6 +141,78 @@ def test_cascade_autotune_and_cache(g, tmp_path):
         D.set_tuning(0, 8)
 
 
+def _decoded(C, k):
+    """States and atlases of volume k as the values that are stored, in FP64."""
+    d = C.descs[k]
+    n, m = d.irr_n + 2, d.dist_n + 2
+    raw = C.buffer(k, 0)
+    if d.irr_format == 2:
+        w = raw.view(torch.int32).cpu().numpy().astype(np.int64).reshape(-1, n, n) & 0xFFFFFFFF
+        irr = np.stack([(w >> s) & 511 for s in (0, 9, 18)], -1) * 2.0 ** ((w >> 27) - 24)[..., None]
+    else:
+        irr = raw.view(torch.float16 if d.irr_format else torch.float32).view(-1, n, n, 4)[..., :3].double().cpu().numpy()
+    dist = C.buffer(k, 1).view(torch.float16 if d.dist_format else torch.float32).view(-1, m, m, 2).double().cpu().numpy()
+    return C.states(k).cpu().numpy().copy(), np.ascontiguousarray(irr), np.ascontiguousarray(dist)
+
+
+@pytest.mark.parametrize("irr_format, dist_format, gamma", [(0, 0, 5.0), (1, 1, 5.0), (2, 0, 5.0), (0, 0, 1.0),
+                                                             (1, 0, 5.0), (1, 1, 2.2)])
+def test_cascade_query_forms(g, irr_format, dist_format, gamma):
+    """Hit shading and the query of a cascade by storage format and gamma (each has a form of the
+    probe query; the last two take the general one), against the oracle on the values that are
+    stored: one frame from the GPU's own state, ray by ray, then the query.  A result may be off by the
+    parity tolerance plus twice what the oracle's moves by when the stored values move by four FP32
+    ulps; 0.5 % of the rays may be listed (grazed edges, hit points where the FP32 position
+    does not fix the query)."""
+    sc, L = synth.room_scene(n_boxes=12), synth.room_lights()
+    descs = _descs()
+    for d in descs:
+        d.tracking, d.gamma, d.irr_format, d.dist_format = 0, gamma, irr_format, dist_format
+    S, C, cam = g.Scene.from_arrays(sc), g.Cascade(descs), _camera(0)
+    for f in range(3):
+        C.update(S, L, f, cam)
+    prev = [_decoded(C, k) for k in range(2)]
+    C.update(S, L, 3, cam)
+    torch.cuda.synchronize()
+    h, vols = oracle.SceneHandle(sc), [oracle.make_volume(d) for d in descs]
+    rng = np.random.default_rng(61)
+
+    def moved(state):
+        st, irr, dist = (a.copy() for a in state)
+        for a in (irr, dist):
+            a += 4 * np.abs(np.spacing(a.astype(np.float32))).astype(np.float64) * rng.choice([-1.0, 1.0], size=a.shape)
+        return st, irr, dist
+
+    def frame(states):
+        states = [tuple(a.copy() for a in s) for s in states]
+        return oracle.update_cascade(h, L, vols, 3, *[[s[j] for s in states] for j in range(3)], want_rays=True)
+
+    rays = frame(prev)
+    others = [frame([moved(s) for s in prev]) for _ in range(4)]
+    rec, vol_of, probe_of = (a.cpu().numpy() for a in C.ray_records())
+    flagged = total = 0
+    for k in range(2):
+        ids = probe_of[vol_of == k]
+        _, err = compare_rays(rec[vol_of == k].astype(np.float64), ids, rays[k])
+        sens = np.max([compare_rays(o[k][ids], ids, rays[k])[1] for o in others], axis=0)
+        flagged += int((err > REL + 2.0 * sens).any(-1).sum())
+        total += err.shape[0] * err.shape[1]
+        assert np.median(err) <= 1e-5
+    assert total > 10000 and flagged <= 0.005 * total
+
+    now = [_decoded(C, k) for k in range(2)]
+    pos, nrm, _ = synth.room_queries(n=2048)
+
+    def query(states):
+        return oracle.query_cascade(vols, *[[s[j] for s in states] for j in range(3)], pos, nrm, cam)
+
+    ref = query(now)
+    scale = np.maximum(np.abs(ref), 1e-3 * np.abs(ref).max())        # as rel_err
+    sens = np.max([np.abs(query([moved(s) for s in now]) - ref) / scale for _ in range(4)], axis=0).max(-1)
+    e = rel_err(C.query(to_dev(pos), to_dev(nrm), cam).cpu().numpy(), ref).max(-1)
+    assert np.median(e) <= 1e-5 and (e <= REL + 2.0 * sens).all()
+
+
 def test_terrain_cascades_full_size_frame0_sampled(g):
     """The batched-cascade workload at full size and in the bench's launch
     configuration (four 32^3 tracking volumes at 1 / 2 / 4 / 8 m, 288 rays,

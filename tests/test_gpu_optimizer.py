@@ -79,6 +79,20 @@ def test_optimizer_offsets_states_and_texels(g, case):
     assert e.max() <= REL and e_own.max() <= REL
 
 
+@pytest.mark.parametrize("rays", [7, 31, 33])
+def test_optimizer_ragged_batches(g, rays):
+    """Ray counts that leave a batch of 32 rays partly empty (the only one, or the last of two): the
+    offsets that the oracle's optimizer gives, up to the few probes of the full test."""
+    sc = synth.room_scene()
+    desc = synth.room_volume(optimizer_iters=3, rays_per_probe=rays)
+    off = oracle.optimize(oracle.SceneHandle(sc), desc, 0, np.arange(desc.n_probes), oracle.new_offsets(desc))
+    V = g.Volume(desc)
+    V.update(g.Scene.from_arrays(sc), synth.room_lights(), 0)
+    bad = np.abs(V.offsets().cpu().numpy() - off).max(1) > 1e-4
+    assert np.any(off != 0, axis=1).sum() > 0.05 * len(off)
+    assert bad.sum() <= max(3, int(0.01 * len(off)))
+
+
 def test_optimizer_off_matches_plain_update(g):
     """optimizer_iters = 0 keeps every probe on its grid point."""
     sc = synth.room_scene(n_boxes=6)

@@ -474,3 +474,23 @@ def test_gbuffer_tiles(g, width, height):
     assert (tri >= 0).all()
     assert np.abs(pos.cpu().numpy() - ref).max() <= 1e-4 * 10.0     # FP32 rays against FP64 ones in a 10 m room
     assert np.abs(np.linalg.norm(nrm.cpu().numpy(), axis=1) - 1.0).max() <= 1e-5
+
+
+@pytest.mark.parametrize("width, height", [(1, 1), (7, 5), (33, 9)])
+def test_gbuffer_normals(g, width, height):
+    """Each pixel's normal is that of the triangle its ray hits first, by the order of its vertices; a
+    ray through an edge may take either side's: one of the triangles that the oracle's ray hits when it
+    is turned by 1e-6 (FP32 directions are off by less)."""
+    sc = synth.room_scene(n_boxes=8)
+    S = g.Scene.from_arrays(sc)
+    cam = synth.PinholeCamera(position=np.array([5.0, 5.0, 1.0]), forward=np.array([0.0, 0.0, 1.0]),
+                              up=np.array([0.0, 1.0, 0.0]), vfov_deg=70.0, width=width, height=height)
+    _, nrm = S.raycast_gbuffer(cam.position, cam.forward, cam.up, cam.vfov_deg, width, height)
+    h, dirs, best = oracle.SceneHandle(sc), synth.camera_ray_dirs(cam), np.full(width * height, np.inf)
+    for turn in np.array([[0, 0, 0], [1, 0, 0], [-1, 0, 0], [0, 1, 0], [0, -1, 0]]) * 1e-6:
+        _, tri, _ = oracle.trace(h, np.repeat(cam.position[None], width * height, 0), dirs + turn)
+        v = sc.verts[sc.tris[tri]].astype(np.float64)
+        n = np.cross(v[:, 1] - v[:, 0], v[:, 2] - v[:, 0])
+        n /= np.linalg.norm(n, axis=1, keepdims=True)
+        best = np.minimum(best, np.abs(nrm.cpu().numpy() - n).max(1))
+    assert best.max() <= 1e-5
