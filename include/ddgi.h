@@ -448,8 +448,9 @@ ddgi_status ddgi_cascade_get_window(ddgi_cascade cascade, int32_t vol, double or
 ddgi_status ddgi_cascade_get_ray_records(ddgi_cascade cascade, float* records_dev, int32_t* entries_dev,
                                          int64_t* n_active, ddgi_stream stream);
 
-/* Launch shapes: trace kernels' blocks per SM (1..32) and the SIMT blend's
- * probes per CTA (4, 8 or 16).  ddgi_cascade_autotune times the update under
+/* Launch shapes: trace kernels' blocks per SM (1..32; the ray walks launch no
+ * more than the five that are resident at once, so larger values only widen the
+ * shading pass's grid) and the SIMT blend's probes per CTA (4, 8 or 16).  ddgi_cascade_autotune times the update under
  * each candidate and keeps the fastest, caching the choice in a JSON file at
  * cache_path (keyed by GPU name and workload); *from_cache = 1 when the cache
  * answered.  Timing advances the volumes by the frames it runs. */

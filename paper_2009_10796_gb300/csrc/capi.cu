@@ -1526,7 +1526,9 @@ ddgi_status ddgi_cascade_poll_status(ddgi_cascade c, ddgi_stream stream) {
 }
 
 // Autotuner: times the cascade update under each candidate launch shape
-// (trace blocks per SM x SIMT blend probes per CTA) and keeps the fastest.
+// (trace blocks per SM x SIMT blend probes per CTA) and keeps the fastest.  Above
+// five blocks an SM only the shading's grid grows: the walks' are at most what is
+// resident at once (trace_ctas).
 // Results are cached in a small JSON file keyed by GPU name and workload
 // signature; a cached entry is used without timing.  Timing advances the
 // volumes by the frames it runs (all with params->frame's ray pattern).

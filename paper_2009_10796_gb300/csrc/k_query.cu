@@ -9,8 +9,9 @@ namespace ddgi {
 // (16-byte stores when the run is aligned), so each warp writes whole lines,
 // for page-locked host memory written across the host link; otherwise each
 // thread stores its own three floats (device memory).
-// Four CTAs per SM (64 registers): 1920 x 1080 points of a hall take 72 us; at
-// five (48 registers, spills) the time was 3 % longer.
+// Four CTAs per SM (64 registers, of which the FP32 forms spill 8 to 28 bytes):
+// 1920 x 1080 points of a hall take 73 us, as many inside the grid 109; at five
+// (48 registers, larger spills) the time was 3 % longer.
 constexpr int kQueryThreads = 256;
 // ORDERED: the points are taken in the order of o (launch_query_ordered).
 template <bool STAGE_OUT, int FORM, bool ORDERED = false>

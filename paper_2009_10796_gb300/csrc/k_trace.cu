@@ -476,7 +476,11 @@ __device__ __forceinline__ Hit closest_hit_warp(const DevScene& s, const RayPre&
     return w.h;
 }
 
-// Closest hits of arbitrary rays, a warp for 32 consecutive ones.
+// Closest hits of arbitrary rays, a warp for 32 consecutive ones.  Rays that
+// share nothing gain as well against one ray a thread over the binary hierarchy:
+// 1 M of them with random origins and directions over 196,610 city triangles
+// 471 -> 291 us, bounced from what a camera sees 312 -> 151 us, 1000 of them
+// 53 -> 23 us.
 __global__ void __launch_bounds__(256, 4) k_trace_rays(DevScene s, const float* __restrict__ orig,
                                                                 const float* __restrict__ dir, int64_t n,
                                                                 float* __restrict__ t_out,
@@ -506,9 +510,9 @@ __global__ void __launch_bounds__(256, 4) k_trace_rays(DevScene s, const float* 
 
 // Camera G-buffer, a warp for a tile of 8 x 4 pixels, whose rays stay together
 // further down the hierarchy than a row of 32.  Bound by the walk's
-// instruction issue, as the probe rays are: 1920 x 1080 over 196,610 city
-// triangles take 139 us, 199 us with one ray a thread over the binary
-// hierarchy.
+// instruction issue, as the probe rays are (81 % of the cycles, 31.7 of 32 lanes):
+// 1920 x 1080 over 196,610 city triangles take 139 us, 199 us with one ray a
+// thread over the binary hierarchy.
 __global__ void __launch_bounds__(256, 4) k_gbuffer(DevScene s, float3 cpos, float3 fwd, float3 right,
                                                              float3 up, float tan_half, float aspect, int w, int h,
                                                              float* __restrict__ out_pos,

@@ -548,7 +548,12 @@ __device__ __forceinline__ Cage cage_of(const VolView& v, const LocalPoint& q) {
 // frame against 2580); a single volume's are slower (city frame with FP16
 // atlases 504 us against 498).  IEEE: the distance and the lookup's
 // coordinates by rounded square root and division (the adjoint, where one
-// point's weight can be a whole texel's gradient).
+// point's weight can be a whole texel's gradient).  The backface cosine, the
+// Chebyshev ratio and the adjoint's decode (decode_slope) use the hardware's
+// reciprocals there too, about 2 ulp each: rounded as well they were no closer to 64
+// bits (texel gradients of 1280 x 720 points 3.0e-5 rms, 2.7e-5 as it is, the
+// same over fifteen drawn cases) and took 267 us for 1920 x 1080 points
+// instead of 234.
 template <int FORM, bool IEEE = false, bool BRANCH = false>
 __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoint& q, const Cage& k, int c, int p,
                                                float3 n) {
