@@ -130,3 +130,10 @@ def test_query_forms_where_the_variance_cancels(g, form):
     e = (np.abs(E - ref) / np.maximum(np.abs(ref), 1e-30)).max(-1)
     assert (spread > REL).sum() > 10                                 # the weights do depend on the last bits
     assert (e <= REL + 2.0 * spread).all()
+
+
+@pytest.mark.parametrize("n", [1, 257])
+def test_rgb9e5_gamma1_matches_oracle(g, monkeypatch, n):
+    """The one form of point queries that the table above has no row for."""
+    monkeypatch.setitem(FORMS, "rgb9e5_gamma1", (2, 0, 1.0, False))
+    test_query_forms_match_oracle(g, "rgb9e5_gamma1", n)
