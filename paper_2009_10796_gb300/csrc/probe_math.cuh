@@ -601,12 +601,13 @@ __device__ __forceinline__ float corner_weight(const VolView& v, const LocalPoin
 // lookup and cascades of that form are no faster so (76 us for points beyond the
 // grid, 74 with eight), and with probe offsets fewer cost neighbouring points
 // 5 % (119 us, 114; general form 136) and give random order 1 % (327, 331; 320).
+// all: a glossy lookup or a cascade.
 template <int FORM>
 __host__ __device__ constexpr int corners_per_trip(bool all) {
     return QueryForm<FORM>::kAnyGamma ? 2 : FORM == kQueryGamma1 && !all ? 4 : 8;
 }
 
-// The specialised query of query_M_look (FORM < kQueryGeneral): the same
+// The specialised query of query_M_look (any FORM but kQueryGeneral): the same
 // operations in the same order, except the decode's zero test
 // (gamma_decode_g5_pair), with the eight cage corners unrolled, the storage
 // format, gamma and offsets fixed at compile time, and the red and green
